@@ -32,13 +32,23 @@ struct Geo {
 };
 
 struct PcgState;
+struct FxW;
+struct FxR;
 
 // Device tables and workspaces of one precision.
 template <typename T>
 struct Tables {
   typedef typename std::conditional<sizeof(T) == 4, float2, double2>::type C;
   C* tw = nullptr;            // exp(-2 pi i k / Lmax)
-  T* sig = nullptr;           // kernel symbol / prod L
+  T* sig = nullptr;           // FP32: kernel symbol / prod L
+  // FP64 passes: the constants of the fixed-point transforms (fix_core.cuh)
+  FxW* ftw = nullptr;         // exp(-2 pi i k / Lmax)
+  FxR* fsig = nullptr;        // kernel symbol / prod L / 2^sig_exp
+  int sig_exp = 0;
+  FxW* fchirp[3] = {nullptr, nullptr, nullptr};
+  FxW* fbhat[3] = {nullptr, nullptr, nullptr};   // / 2^bexp
+  int bexp[3] = {0, 0, 0};
+  // FP32 DST tables
   C* chirp[3] = {nullptr, nullptr, nullptr};
   C* bhat[3] = {nullptr, nullptr, nullptr};
   C* S = nullptr;             // operator spectrum workspace
@@ -138,8 +148,10 @@ cudaError_t launch_axmy(long long N, cudaStream_t s, const double* u, double c, 
                         double* y);
 // order-independent 64-bit hash of the bits of N doubles, added into *h (zero it first)
 cudaError_t launch_hash(long long N, cudaStream_t s, const double* u, unsigned long long* h);
+// sig32 and, as fixed-point constants over 2^*sig_exp, fsig (waits for the
+// stream to choose the exponent).
 cudaError_t build_symbol(const Geo& g, double c, double Z, double a, double expo, cudaStream_t s,
-                         double* sig64, float* sig32, const double2* tw64);
+                         FxR* fsig, int* sig_exp, float* sig32, const double2* tw64);
 size_t partial_capacity(const Geo& g);
 
 // --- launch accounting (plan.cu) ----------------------------------------------

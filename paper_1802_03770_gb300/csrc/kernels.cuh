@@ -25,6 +25,7 @@
 #pragma once
 
 #include "fft_core.cuh"
+#include "fix_core.cuh"
 
 #ifndef FL_ROW_MIN_CTAS
 #define FL_ROW_MIN_CTAS 7
@@ -72,7 +73,7 @@ struct PcgState {
 };
 
 enum { PRE_NONE = 0, PRE_PUPDATE = 1, PRE_ACCUM = 2 };
-enum { COLS_FWD = 0, COLS_CONV = 1, COLS_INV = 2, COLS_FULL = 3 };
+enum { COLS_FWD = 0, COLS_CONV = 1, COLS_INV = 2 };
 enum { DPRE_NONE = 0, DPRE_UPDATE = 1 };
 // What the last CTA of a pass does with the pass's partial sums:
 // FIN_PQ: pq = sum, alpha = rz / pq; FIN_STEP: the CG scalar step.
@@ -276,6 +277,7 @@ struct RowsFwdArgs {
   int rows, n, H, lg, lgmax;
   int rows_per_plane, plane_stride;  // spectrum row = (r / rpp) * ps + r % rpp
   int pre;
+  const FxW* ftw;          // FP64: twiddles as fixed-point constants
 };
 
 template <typename T, int THREADS, int VPT, int LGLO, int LGHI>
@@ -388,9 +390,14 @@ __device__ __forceinline__ void body_rows_fwd_fixed(const RowsFwdArgs<T>& a, int
   }
 }
 
+// FP64: fixed-point lines (fix_passes.cuh)
+template <int THREADS, int VPT, int LGLO, int LGHI>
+__device__ __forceinline__ void fx_body_rows_fwd(const RowsFwdArgs<double>& a, int bx);
+
 template <typename T, int THREADS, int VPT, int LGLO = 4, int LGHI = clog2(THREADS * VPT)>
 __device__ __forceinline__ void body_rows_fwd(const RowsFwdArgs<T>& a, int bx, int by) {
-  body_rows_fwd_fixed<T, THREADS, VPT, LGLO, LGHI, (LGLO > kFixedLgMin ? LGLO : kFixedLgMin)>(a, bx, by);
+  if constexpr (sizeof(T) == 8) fx_body_rows_fwd<THREADS, VPT, LGLO, LGHI>(a, bx);
+  else body_rows_fwd_fixed<T, THREADS, VPT, LGLO, LGHI, (LGLO > kFixedLgMin ? LGLO : kFixedLgMin)>(a, bx, by);
 }
 
 template <typename T, int THREADS, int VPT, int LGLO = 4>
@@ -419,6 +426,11 @@ struct ColsArgs {
   long long sig_line, sig_outer;
   int Lo;                  // length of the outer axis in the spectrum (3D: L_1), 0 if unused
   int ltx;                 // log2 of the columns per CTA
+  // FP64: twiddles and symbol as fixed-point constants, the symbol divided
+  // by 2^sig_exp
+  const FxW* ftw;
+  const FxR* fsig;
+  int sig_exp;
 };
 
 // The tile is kept in its natural layout, buf[r * TX + c] (row r of the line,
@@ -533,9 +545,14 @@ __device__ __forceinline__ void body_cols_fixed(const ColsArgs<T>& a, int bx, in
   }
 }
 
+// FP64: fixed-point lines (fix_passes.cuh)
+template <int THREADS, int VPT, int LGLO, int LGHI>
+__device__ __forceinline__ void fx_body_cols(const ColsArgs<double>& a, int bx, int by);
+
 template <typename T, int THREADS, int VPT, int LGLO = 4, int LGHI = clog2(THREADS * VPT)>
 __device__ __forceinline__ void body_cols(const ColsArgs<T>& a, int bx, int by) {
-  body_cols_fixed<T, THREADS, VPT, LGLO, LGHI, (LGLO > kFixedLgMin ? LGLO : kFixedLgMin)>(a, bx, by);
+  if constexpr (sizeof(T) == 8) fx_body_cols<THREADS, VPT, LGLO, LGHI>(a, bx, by);
+  else body_cols_fixed<T, THREADS, VPT, LGLO, LGHI, (LGLO > kFixedLgMin ? LGLO : kFixedLgMin)>(a, bx, by);
 }
 
 template <typename T, int THREADS, int VPT, int LGLO = 4>
@@ -571,6 +588,7 @@ struct RowsInvArgs {
   int nparts;              // CTAs of the pass (partials to sum)
   PcgState* fst;
   T* outm;                 // nullable: M x itself (restricted to Omega)
+  const FxW* ftw;          // FP64: twiddles as fixed-point constants
 };
 
 template <typename T, int THREADS, int VPT, int LGLO, int LGHI>
@@ -690,9 +708,14 @@ __device__ __forceinline__ void body_rows_inv_fixed(const RowsInvArgs<T>& a, int
   }
 }
 
+// FP64: fixed-point lines (fix_passes.cuh)
+template <int THREADS, int VPT, int LGLO, int LGHI>
+__device__ __forceinline__ void fx_body_rows_inv(const RowsInvArgs<double>& a, int bx);
+
 template <typename T, int THREADS, int VPT, int LGLO = 4, int LGHI = clog2(THREADS * VPT)>
 __device__ __forceinline__ void body_rows_inv(const RowsInvArgs<T>& a, int bx, int by) {
-  body_rows_inv_fixed<T, THREADS, VPT, LGLO, LGHI, (LGLO > kFixedLgMin ? LGLO : kFixedLgMin)>(a, bx, by);
+  if constexpr (sizeof(T) == 8) fx_body_rows_inv<THREADS, VPT, LGLO, LGHI>(a, bx);
+  else body_rows_inv_fixed<T, THREADS, VPT, LGLO, LGHI, (LGLO > kFixedLgMin ? LGLO : kFixedLgMin)>(a, bx, by);
 }
 
 template <typename T, int THREADS, int VPT, int LGLO = 4>
@@ -752,6 +775,12 @@ struct DstRowsArgs {
   // mask, out = mask_out ? (B^{-1} in + add) : 0 (the second half of the
   // capacitance solve on an occluded domain)
   const T* add;
+  // FP64: twiddles, chirp and chirp kernel as fixed-point constants, the
+  // chirp kernel divided by 2^bexp
+  const FxW* ftw;
+  const FxW* fchirp;
+  const FxW* fbhat;
+  int bexp;
 };
 
 template <typename T, int THREADS, int VPT, int LGLO, int LGHI>
@@ -884,9 +913,14 @@ __device__ __forceinline__ void body_dst_rows_fixed(const DstRowsArgs<T>& a, int
   }
 }
 
+// FP64: fixed-point lines (fix_passes.cuh)
+template <int THREADS, int VPT, int LGLO, int LGHI>
+__device__ __forceinline__ void fx_body_dst_rows(const DstRowsArgs<double>& a, int bx);
+
 template <typename T, int THREADS, int VPT, int LGLO = 4, int LGHI = clog2(THREADS * VPT)>
 __device__ __forceinline__ void body_dst_rows(const DstRowsArgs<T>& a, int bx, int by) {
-  body_dst_rows_fixed<T, THREADS, VPT, LGLO, LGHI, (LGLO > kFixedLgMin ? LGLO : kFixedLgMin)>(a, bx, by);
+  if constexpr (sizeof(T) == 8) fx_body_dst_rows<THREADS, VPT, LGLO, LGHI>(a, bx);
+  else body_dst_rows_fixed<T, THREADS, VPT, LGLO, LGHI, (LGLO > kFixedLgMin ? LGLO : kFixedLgMin)>(a, bx, by);
 }
 
 template <typename T, int THREADS, int VPT, int LGLO = 4>
@@ -911,6 +945,10 @@ struct DstColsArgs {
   int n, ncols, lg, lgmax;
   long long ostride, lstride;
   int ltx;
+  const FxW* ftw;          // FP64: as in DstRowsArgs
+  const FxW* fchirp;
+  const FxW* fbhat;
+  int bexp;
 };
 
 template <typename T, int THREADS, int VPT, int LGLO, int LGHI>
@@ -976,9 +1014,14 @@ __device__ __forceinline__ void body_dst_cols_fixed(const DstColsArgs<T>& a, int
   }
 }
 
+// FP64: fixed-point lines (fix_passes.cuh)
+template <int THREADS, int VPT, int LGLO, int LGHI>
+__device__ __forceinline__ void fx_body_dst_cols(const DstColsArgs<double>& a, int bx, int by);
+
 template <typename T, int THREADS, int VPT, int LGLO = 4, int LGHI = clog2(THREADS * VPT)>
 __device__ __forceinline__ void body_dst_cols(const DstColsArgs<T>& a, int bx, int by) {
-  body_dst_cols_fixed<T, THREADS, VPT, LGLO, LGHI, (LGLO > kFixedLgMin ? LGLO : kFixedLgMin)>(a, bx, by);
+  if constexpr (sizeof(T) == 8) fx_body_dst_cols<THREADS, VPT, LGLO, LGHI>(a, bx, by);
+  else body_dst_cols_fixed<T, THREADS, VPT, LGLO, LGHI, (LGLO > kFixedLgMin ? LGLO : kFixedLgMin)>(a, bx, by);
 }
 
 template <typename T, int THREADS, int VPT, int LGLO = 4>
@@ -989,6 +1032,8 @@ __global__ void __launch_bounds__(THREADS, min_ctas(THREADS, LGLO)) k_dst_cols(D
 }
 
 }  // namespace fl
+
+#include "fix_passes.cuh"
 
 namespace fl {
 

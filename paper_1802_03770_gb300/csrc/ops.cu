@@ -267,10 +267,35 @@ __global__ void __launch_bounds__(THREADS) k_rows_c2c(double2* buf, int rows, in
   }
 }
 
+// In-place complex FFTs along a slow axis (full length in and out), TX
+// columns per CTA: line element r of column kx at outer index o is
+// buf[o * ostride + r * lstride + kx].
+template <int THREADS, int VPT, int LGLO = 4>
+__global__ void __launch_bounds__(THREADS) k_cols_c2c(double2* buf, int H, int lg, int lgmax, long long ostride,
+                                                     long long lstride, int ltx, const double2* tw) {
+  constexpr int LGC = clog2(THREADS * VPT);
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const SBuf<double2> sb{reinterpret_cast<double2*>(smem_raw)};
+  const int L = 1 << lg, TX = 1 << ltx;
+  const int kx0 = blockIdx.x << ltx;
+  const int ncol = min(TX, H - kx0);
+  double2* base = buf + (size_t)blockIdx.y * ostride + kx0;
+  for (int e = threadIdx.x; e < TX * L; e += THREADS) {
+    const int r = e >> ltx, c = e & (TX - 1);
+    sb[e] = c < ncol ? base[(size_t)r * lstride + c] : make_double2(0.0, 0.0);
+  }
+  __syncthreads();
+  fft_smem<VPT, true, LGC, LGLO>(sb, lg, 0, ltx, TX, tw, lgmax, false);
+  for (int e = threadIdx.x; e < TX * L; e += THREADS) {
+    const int r = e >> ltx, c = e & (TX - 1);
+    if (c < ncol) base[(size_t)r * lstride + c] = sb[e];
+  }
+}
+
 __global__ void k_extract_symbol(const double2* buf, int d, int L0, int L1, int L2, double inv,
-                                 double* sig64, float* sig32, long long total) {
-  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i >= total) return;
+                                 double* sig64, float* sig32, unsigned* amax, long long total) {
+  const long long at = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const long long i = at < total ? at : total - 1;
   const int Ls[3] = {L0, L1, L2};
   long long rem = i, src = 0, mul = 1;
   for (int ax = d - 1; ax >= 0; --ax) {
@@ -283,6 +308,17 @@ __global__ void k_extract_symbol(const double2* buf, int d, int L0, int L1, int 
   const double v = buf[src].x * inv;
   sig64[i] = v;
   sig32[i] = (float)v;
+  // upper words of |v| order like the values
+  const unsigned top = __reduce_max_sync(0xffffffffu, (unsigned)__double2hiint(v) & 0x7fffffffu);
+  if ((threadIdx.x & 31) == 0) atomicMax(amax, top);
+}
+
+// sig = fixed-point constants of sig / 2^expo, in place (8 bytes each)
+__global__ void k_fix_symbol(double* sig, int expo, long long total) {
+  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (i >= total) return;
+  const FxR w = fx_real(__double2ll_rn(ldexp(sig[i], kFxFrac - expo)));
+  reinterpret_cast<FxR*>(sig)[i] = w;
 }
 
 // ---------------------------------------------------------------------------
@@ -339,6 +375,8 @@ cudaError_t configure_kernels_f64() {
   FL_SET(k_cols<double, 512, 16, 13>);
   FL_SET(k_dst_cols<double, 512, 16, 13>);
   FL_SET(k_rows_c2c<2 * Cfg<double>::RT, Cfg<double>::RV>);
+  FL_SET(k_cols_c2c<Cfg<double>::CT, Cfg<double>::CV>);
+  FL_SET(k_cols_c2c<2 * Cfg<double>::CT, Cfg<double>::CV, 13>);
 #undef FL_SET
   return e;
 }
@@ -408,13 +446,14 @@ ApplyChain<T> build_apply(const Geo& g, const Tables<T>& tb, const ApplyIO<T>& i
     a.u = io.u; a.p = io.p; a.acc = io.acc; a.x32 = io.x32; a.mask = io.mask;
     a.S = tb.S; a.tw = tb.tw; a.st = io.st;
     a.rows = (int)rows; a.n = g.n[d - 1]; a.H = g.H; a.lg = g.lg[d - 1]; a.lgmax = g.lgmax;
-    a.rows_per_plane = rpp; a.plane_stride = pstride; a.pre = io.pre;
+    a.rows_per_plane = rpp; a.plane_stride = pstride; a.pre = io.pre; a.ftw = tb.ftw;
   }
   ch.ncols = 0;
   auto cols = [&](int axis, int mode, int rows_in, int rows_out, long long lstride,
                   long long ostride, int nouter, long long sig_line, long long sig_outer, int Lo) {
     ColsArgs<T>& a = ch.cols[ch.ncols];
     a.S = tb.S; a.tw = tb.tw; a.sig = tb.sig; a.st = io.st;
+    a.ftw = tb.ftw; a.fsig = tb.fsig; a.sig_exp = tb.sig_exp;
     a.H = g.H; a.lg = g.lg[axis]; a.lgmax = g.lgmax;
     a.rows_in = rows_in; a.rows_out = rows_out; a.lstride = lstride; a.ostride = ostride;
     a.nouter = nouter; a.mode = mode; a.sig_line = sig_line; a.sig_outer = sig_outer; a.Lo = Lo;
@@ -444,7 +483,7 @@ ApplyChain<T> build_apply(const Geo& g, const Tables<T>& tb, const ApplyIO<T>& i
     a.rows_per_plane = rpp; a.plane_stride = pstride; a.dot_self = io.dot_self;
     a.fin = (io.partials && io.st) ? io.fin : FIN_NONE;
     a.nparts = ch.row_blocks; a.fst = io.st;
-    a.outm = io.outm;
+    a.outm = io.outm; a.ftw = tb.ftw;
   }
   return ch;
 }
@@ -460,8 +499,8 @@ cudaError_t launch_apply(const Geo& g, const Tables<T>& tb, cudaStream_t s, cons
             } else {
               FL_ROWS_LAUNCH(k_rows_fwd, T, Lx, ch.row_blocks, ch.row_smem, s, ch.fwd);
             });
-  static const char* const kn[2][4] = {{"cols_fwd<f64>", "cols_conv<f64>", "cols_inv<f64>", "cols_full<f64>"},
-                                       {"cols_fwd<f32>", "cols_conv<f32>", "cols_inv<f32>", "cols_full<f32>"}};
+  static const char* const kn[2][3] = {{"cols_fwd<f64>", "cols_conv<f64>", "cols_inv<f64>"},
+                                       {"cols_fwd<f32>", "cols_conv<f32>", "cols_inv<f32>"}};
   for (int j = 0; j < ch.ncols; ++j)
     FL_KERNEL(kn[sizeof(T) == 4][ch.cols[j].mode], s,
               FL_COLS_LAUNCH(k_cols, T, 1 << ch.cols[j].lg, ch.cols_grid[j], ch.cols_smem[j], s,
@@ -491,6 +530,7 @@ PrecChain<T> build_precond(const Geo& g, const Tables<T>& tb, const PrecIO<T>& i
   {
     DstRowsArgs<T>& a = ch.first;
     a.in = io.in; a.out = tb.t; a.tw = tb.tw; a.chirp = tb.chirp[d - 1]; a.bhat = tb.bhat[d - 1];
+    a.ftw = tb.ftw; a.fchirp = tb.fchirp[d - 1]; a.fbhat = tb.fbhat[d - 1]; a.bexp = tb.bexp[d - 1];
     a.st = io.st; a.x = io.x; a.r = io.r; a.p = io.p; a.q = io.q;
     a.rr_part = io.rr_part;
     a.dotw = nullptr; a.dot_part = nullptr; a.post = 1.0;
@@ -502,6 +542,7 @@ PrecChain<T> build_precond(const Geo& g, const Tables<T>& tb, const PrecIO<T>& i
   auto cols = [&](int axis, long long lstride, long long ostride, int nouter) {
     DstColsArgs<T>& a = ch.cols[ch.ncols];
     a.v = tb.t; a.tw = tb.tw; a.chirp = tb.chirp[axis]; a.bhat = tb.bhat[axis]; a.st = io.st;
+    a.ftw = tb.ftw; a.fchirp = tb.fchirp[axis]; a.fbhat = tb.fbhat[axis]; a.bexp = tb.bexp[axis];
     a.post = 1.0;
     a.n = g.n[axis]; a.ncols = nx; a.lg = g.lg[axis]; a.lgmax = g.lgmax;
     a.ostride = ostride; a.lstride = lstride;
@@ -534,6 +575,7 @@ PrecChain<T> build_precond(const Geo& g, const Tables<T>& tb, const PrecIO<T>& i
   {
     DstRowsArgs<T>& a = ch.last;
     a.in = tb.t; a.out = io.out; a.tw = tb.tw; a.chirp = tb.chirp[d - 1]; a.bhat = tb.bhat[d - 1];
+    a.ftw = tb.ftw; a.fchirp = tb.fchirp[d - 1]; a.fbhat = tb.fbhat[d - 1]; a.bexp = tb.bexp[d - 1];
     a.st = io.st; a.x = nullptr; a.r = nullptr; a.p = nullptr; a.q = nullptr;
     a.rr_part = nullptr;
     a.dotw = io.dotw; a.dot_part = io.dot_part; a.post = post;
@@ -687,7 +729,7 @@ cudaError_t launch_sum(cudaStream_t s, const double* part, int count, double* ou
 
 #if FL_OPS_PART == 2
 cudaError_t build_symbol(const Geo& g, double c, double Z, double a, double expo, cudaStream_t s,
-                         double* sig64, float* sig32, const double2* tw64) {
+                         FxR* fsig, int* sig_exp, float* sig32, const double2* tw64) {
   typedef Cfg<double> K;
   const int d = g.d;
   long long total = 1, half = 1;
@@ -722,25 +764,46 @@ cudaError_t build_symbol(const Geo& g, double c, double Z, double a, double expo
   }
   // slower axes: strided lines, full length in and out
   for (int axis = d - 2; axis >= 0; --axis) {
-    ColsArgs<double> ca;
-    ca.S = buf; ca.tw = tw64; ca.sig = nullptr; ca.st = nullptr;
-    ca.H = Ls[d - 1]; ca.lg = g.lg[axis]; ca.lgmax = g.lgmax;
-    ca.rows_in = Ls[axis]; ca.rows_out = Ls[axis]; ca.mode = COLS_FULL;
-    ca.sig_line = 0; ca.sig_outer = 0; ca.Lo = 0;
-    if (d == 2) { ca.lstride = Ls[1]; ca.ostride = 0; ca.nouter = 1; }
-    else if (axis == 1) { ca.lstride = Ls[2]; ca.ostride = (long long)Ls[1] * Ls[2]; ca.nouter = Ls[0]; }
-    else { ca.lstride = (long long)Ls[1] * Ls[2]; ca.ostride = Ls[2]; ca.nouter = Ls[1]; }
-    const int tx = col_tx<double>(Ls[axis]);
-    ca.ltx = ilog2i(tx);
-    dim3 grid((ca.H + tx - 1) / tx, ca.nouter);
-    FL_KERNEL("cols_symbol", s,
-              FL_COLS_LAUNCH(k_cols, double, Ls[axis], grid, tile_bytes<double>(tx, Ls[axis]), s, ca));
+    long long lstride, ostride = 0;
+    int nouter = 1;
+    if (d == 2) { lstride = Ls[1]; }
+    else if (axis == 1) { lstride = Ls[2]; ostride = (long long)Ls[1] * Ls[2]; nouter = Ls[0]; }
+    else { lstride = (long long)Ls[1] * Ls[2]; ostride = Ls[2]; nouter = Ls[1]; }
+    const int L = Ls[axis], tx = col_tx<double>(L);
+    const dim3 grid((Ls[d - 1] + tx - 1) / tx, nouter);
+    if (L <= K::CT * K::CV)
+      FL_KERNEL("cols_c2c", s,
+                k_cols_c2c<K::CT, K::CV><<<grid, K::CT, tile_bytes<double>(tx, L), s>>>(
+                    buf, Ls[d - 1], g.lg[axis], g.lgmax, ostride, lstride, ilog2i(tx), tw64));
+    else
+      FL_KERNEL("cols_c2c", s,
+                k_cols_c2c<2 * K::CT, K::CV, clog2(2 * K::CT * K::CV)><<<grid, 2 * K::CT, tile_bytes<double>(tx, L), s>>>(
+                    buf, Ls[d - 1], g.lg[axis], g.lgmax, ostride, lstride, ilog2i(tx), tw64));
   }
   double inv = 1.0;
   for (int i = 0; i < d; ++i) inv /= (double)g.L[i];
-  FL_KERNEL("extract_symbol", s,
-            k_extract_symbol<<<(unsigned)((half + bt - 1) / bt), bt, 0, s>>>(buf, d, Ls[0], Ls[1], Ls[2], inv,
-                                                                  sig64, sig32, half));
+  double* sig64 = reinterpret_cast<double*>(fsig);
+  unsigned* amax = nullptr;
+  e = cudaMallocAsync(&amax, sizeof(unsigned), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(amax, 0, sizeof(unsigned), s);
+  if (e == cudaSuccess)
+    FL_KERNEL("extract_symbol", s,
+              k_extract_symbol<<<(unsigned)((half + bt - 1) / bt), bt, 0, s>>>(buf, d, Ls[0], Ls[1], Ls[2], inv,
+                                                                    sig64, sig32, amax, half));
+  unsigned top = 0;
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&top, amax, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e == cudaSuccess) {
+    // |sig| <= 2^sig_exp
+    *sig_exp = (int)(top >> 20) - 1022;
+    FL_KERNEL("fix_symbol", s,
+              k_fix_symbol<<<(unsigned)((half + bt - 1) / bt), bt, 0, s>>>(sig64, *sig_exp, half));
+  }
+  if (amax) cudaFreeAsync(amax, s);
+  if (e != cudaSuccess) {
+    cudaFreeAsync(buf, s);
+    return e;
+  }
   e = cudaGetLastError();
   cudaError_t e2 = cudaFreeAsync(buf, s);
   return e != cudaSuccess ? e : e2;

@@ -218,6 +218,20 @@ int ilog2(int v) {
   return l;
 }
 
+// a complex constant of modulus <= 1 for the fixed-point FP64 passes
+FxW fix_const(long double re, long double im) {
+  const long double one = (long double)(1ll << kFxFrac);
+  const FxR x = fx_real(llrintl(re * one)), y = fx_real(llrintl(im * one));
+  return FxW{x.h, x.l, y.h, y.l};
+}
+
+template <typename X>
+fl_status upload_table(fl_plan* p, X** dst, const std::vector<X>& v) {
+  FL_CUDA(dalloc(p, dst, v.size() * sizeof(X)));
+  FL_CUDA(cudaMemcpy(*dst, v.data(), v.size() * sizeof(X), cudaMemcpyHostToDevice));
+  return FL_OK;
+}
+
 // twiddles exp(-2 pi i k / Lmax), chirps and chirp-kernel spectra for the
 // DST-I of each axis (see kernels.cuh), in long double.
 fl_status build_tables(fl_plan* p) {
@@ -226,11 +240,16 @@ fl_status build_tables(fl_plan* p) {
   const long double pi = 3.141592653589793238462643383279502884L;
   std::vector<double2> tw64(Lmax);
   std::vector<float2> tw32(Lmax);
+  std::vector<FxW> twx(Lmax);
   for (int k = 0; k < Lmax; ++k) {
     const long double ang = -2.0L * pi * (long double)k / (long double)Lmax;
-    tw64[k] = make_double2((double)cosl(ang), (double)sinl(ang));
-    tw32[k] = make_float2((float)cosl(ang), (float)sinl(ang));
+    const long double cs = cosl(ang), sn = sinl(ang);
+    tw64[k] = make_double2((double)cs, (double)sn);
+    tw32[k] = make_float2((float)cs, (float)sn);
+    twx[k] = fix_const(cs, sn);
   }
+  fl_status us = upload_table(p, &p->t64.ftw, twx);
+  if (us != FL_OK) return us;
   FL_CUDA(dalloc(p, &p->t64.tw, Lmax * sizeof(double2)));
   FL_CUDA(dalloc(p, &p->t32.tw, Lmax * sizeof(float2)));
   FL_CUDA(cudaMemcpy(p->t64.tw, tw64.data(), Lmax * sizeof(double2), cudaMemcpyHostToDevice));
@@ -244,31 +263,32 @@ fl_status build_tables(fl_plan* p) {
       const long double ang = pi * (long double)m2 / (2.0L * (long double)N1);
       return std::complex<long double>(cosl(ang), sinl(ang));
     };
-    std::vector<double2> c64(n);
+    std::vector<FxW> cx(n);
     std::vector<float2> c32(n);
     for (int j = 0; j < n; ++j) {
       const auto c = chirp(j + 1);
-      c64[j] = make_double2((double)c.real(), (double)c.imag());
+      cx[j] = fix_const(c.real(), c.imag());
       c32[j] = make_float2((float)c.real(), (float)c.imag());
     }
     std::vector<std::complex<long double>> b(L, 0.0L);
     for (int m = -(n - 1); m <= n - 1; ++m) b[(m + L) % L] = std::conj(chirp(m));
     host_fft(b);
-    std::vector<double2> b64(L);
+    std::vector<FxW> bx(L);
     std::vector<float2> b32(L);
+    long double top = 0.0L;
+    for (int k = 0; k < L; ++k) top = std::max(top, fabsl(b[k].real()) + fabsl(b[k].imag()));
+    const int bexp = std::ilogb(top / (long double)L) + 1;   // moduli below 2^bexp
     for (int k = 0; k < L; ++k) {
       const auto v = b[k] / (long double)L;
-      b64[k] = make_double2((double)v.real(), (double)v.imag());
+      bx[k] = fix_const(ldexpl(v.real(), -bexp), ldexpl(v.imag(), -bexp));
       b32[k] = make_float2((float)v.real(), (float)v.imag());
     }
-    FL_CUDA(dalloc(p, &p->t64.chirp[ax], n * sizeof(double2)));
-    FL_CUDA(dalloc(p, &p->t32.chirp[ax], n * sizeof(float2)));
-    FL_CUDA(dalloc(p, &p->t64.bhat[ax], L * sizeof(double2)));
-    FL_CUDA(dalloc(p, &p->t32.bhat[ax], L * sizeof(float2)));
-    FL_CUDA(cudaMemcpy(p->t64.chirp[ax], c64.data(), n * sizeof(double2), cudaMemcpyHostToDevice));
-    FL_CUDA(cudaMemcpy(p->t32.chirp[ax], c32.data(), n * sizeof(float2), cudaMemcpyHostToDevice));
-    FL_CUDA(cudaMemcpy(p->t64.bhat[ax], b64.data(), L * sizeof(double2), cudaMemcpyHostToDevice));
-    FL_CUDA(cudaMemcpy(p->t32.bhat[ax], b32.data(), L * sizeof(float2), cudaMemcpyHostToDevice));
+    p->t64.bexp[ax] = bexp;
+    us = upload_table(p, &p->t64.fchirp[ax], cx);
+    if (us == FL_OK) us = upload_table(p, &p->t64.fbhat[ax], bx);
+    if (us == FL_OK) us = upload_table(p, &p->t32.chirp[ax], c32);
+    if (us == FL_OK) us = upload_table(p, &p->t32.bhat[ax], b32);
+    if (us != FL_OK) return us;
     // eigenvalues of C h^d L along this axis: c (-a) 4 sin^2(pi k / (2 (n+1)))
     std::vector<double> mu(n);
     for (int k = 0; k < n; ++k) {
@@ -1097,9 +1117,10 @@ fl_status fl_plan_create(int d, const int64_t* n, double h, double alpha, const 
   if (st != FL_OK) { free_plan(p); return st; }
   long long half = 1;
   for (int i = 0; i < g.d; ++i) half *= g.L[i] / 2 + 1;
-  FL_TRY(dalloc(p, &p->t64.sig, half * sizeof(double)));
+  FL_TRY(dalloc(p, &p->t64.fsig, half * sizeof(FxR)));
   FL_TRY(dalloc(p, &p->t32.sig, half * sizeof(float)));
-  FL_TRY(build_symbol(g, p->c, p->Z, p->a, d + alpha, p->stream, p->t64.sig, p->t32.sig, p->t64.tw));
+  FL_TRY(build_symbol(g, p->c, p->Z, p->a, d + alpha, p->stream, p->t64.fsig,
+                      &p->t64.sig_exp, p->t32.sig, p->t64.tw));
   FL_TRY(cudaStreamSynchronize(p->stream));
   FL_TRY(dalloc(p, &p->t64.S, g.spec * sizeof(double2)));
   FL_TRY(dalloc(p, &p->t32.S, g.spec * sizeof(float2)));
