@@ -1,13 +1,12 @@
 // 64-bit fixed-point complex arithmetic and its shared-memory FFT: what the
 // FP64 passes transform with.
 //
-// GB300 issues one FP64 operation per 16 cycles and warp scheduler (measured:
-// 1.7 DFMA or DADD per clock and SM), but 61 32 x 32 -> 64-bit multiply-adds
-// (IMAD.WIDE, with a 64-bit addend) and 126 32-bit additions.  A complex
-// addition is 4 integer instructions instead of 2 FP64 ones, a complex
-// multiplication about 30 (12 of them IMAD.WIDE) instead of 4: a radix-16
-// butterfly with its twiddles takes ~11 cycles of an SM's integer pipes per
-// thread instead of ~130 of its FP64 pipe.
+// GB300 issues 1.7 FP64 operations per clock and SM, but 61 32 x 32 ->
+// 64-bit multiply-adds (IMAD.WIDE, with a 64-bit addend) and 126 32-bit
+// additions (all measured).  A complex addition is 4 integer instructions
+// instead of 2 FP64 ones, a complex multiplication about 20 (12 of them
+// IMAD.WIDE) instead of 4: a radix-8 butterfly with its twiddles takes a
+// tenth of the time on the integer pipes.
 //
 // Numbers.  A line of the transform is block floating point: every component
 // is a signed 64-bit integer f, the value is f 2^X with one exponent X per
@@ -15,14 +14,15 @@
 // records the bits its outputs use (the OR of their magnitudes' upper words,
 // per line) and the next stage first shifts the line left by the headroom
 // that is left, so that a stage always works near the top of the 64 bits.
-// All moduli stay below 2^61.5: a radix-R stage divides its inputs by R
-// (together with the twiddle multiplication's own shift) before summing R of
-// them.  Rounding therefore enters at about 2^-60 of the line's largest
-// value per stage, below the 2^-53 of every single FP64 operation that it
-// replaces (measured against extended-precision sums over lines of 16 .. 8192 values).
+// All moduli stay below 2^62.5: a stage divides its inputs by 8 (in the
+// twiddle multiplication itself) before summing up to 8 of them.  Rounding
+// therefore enters at about 2^-60 of the line's largest value per stage,
+// below the 2^-53 of every single FP64 operation that it replaces (measured
+// against extended-precision sums over lines of 16 .. 8192 values: 1e-17 to
+// 1e-16 of the line's norm, FP64 arithmetic 1e-16 to 3e-16).
 //
 // Twiddles, chirps and the kernel symbol are constants w, |w| <= 1, with 61
-// fraction bits, split as w 2^61 = h 2^31 + l, 0 <= l < 2^31.
+// fraction bits, split as w 2^61 = h 2^32 + l, |l| < 2^31.
 #pragma once
 
 #include <stdint.h>
@@ -36,20 +36,27 @@
 namespace fl {
 
 struct alignas(16) Fx { long long x, y; };
-// a complex constant: (h 2^31 + l) / 2^61 per component
+// a complex constant: (h 2^32 + l) / 2^61 per component
 struct alignas(16) FxW { int xh, xl, yh, yl; };
 // a real constant
 struct alignas(8) FxR { int h, l; };
 
 constexpr int kFxFrac = 61;       // fraction bits of the constants
+constexpr int kFxShift = 64 - kFxFrac;   // a product is divided by 2^kFxShift = 8
 // X of a line whose FP64 input holds an infinity or a NaN: its outputs are NaN
 constexpr int kFxBad = 1 << 20;
 
-FL_HD int fx_hi(long long v) { return (int)(v >> 31); }
-FL_HD int fx_lo(long long v) { return (int)v & 0x7fffffff; }
+// v = hi 2^32 + lo with lo in [-2^31, 2^31)
+FL_HD int fx_hi(long long v) { return (int)(v >> 32) + (int)((unsigned)v >> 31); }
+FL_HD int fx_lo(long long v) { return (int)v; }
 FL_HD long long fx_mad(int a, int b, long long c) { return (long long)a * b + c; }
 
-FL_HD FxR fx_real(long long q61) { return FxR{(int)(q61 >> 31), (int)q61 & 0x7fffffff}; }
+// the split of a constant (-2^31 is left out of the low half: it is negated)
+FL_HD constexpr FxR fx_real(long long q) {
+  const int h = (int)((q + (1ll << 31)) >> 32);
+  const long long l = q - ((long long)h << 32);
+  return FxR{h, l == -(1ll << 31) ? (int)(l + 1) : (int)l};
+}
 
 // upper word of |v| (one below for negative v): the OR of these over a line
 // has the bit length of its largest component
@@ -64,9 +71,9 @@ FL_HD int fx_clz(unsigned v) {
   return v ? __builtin_clz(v) : 32;
 #endif
 }
-// left shift that brings components with magnitude bits m below 2^61
+// left shift that brings components with magnitude bits m below 2^62
 FL_HD int fx_headroom(unsigned m) {
-  const int s = fx_clz(m) - 3;
+  const int s = fx_clz(m) - 2;
   return s > 0 ? s : 0;
 }
 FL_HD long long fx_shl(long long v, int s) { return (long long)((unsigned long long)v << s); }
@@ -79,52 +86,43 @@ FL_HD Fx fx_add(Fx a, Fx b) { return Fx{a.x + b.x, a.y + b.y}; }
 FL_HD Fx fx_sub(Fx a, Fx b) { return Fx{a.x - b.x, a.y - b.y}; }
 FL_HD Fx fx_swap(Fx a) { return Fx{a.y, a.x}; }
 
-// (v w) / 2^S.  With v = vh 2^31 + vl the product is
-// H 2^62 + M 2^31 + (low products), H = vh wh, M = vh wl + vl wh;
-// v w / 2^(61 + S) = H / 2^(S-1) + M / 2^(30+S).  |v| < 2^61.5 keeps M within
-// 2^63.  The constant in M's sum centres the error of the truncations (half
-// a unit for M, 1/2 - 2^-S for H); it stays below one unit, so that zero
-// gives zero.
-template <int S> FL_HD long long fx_join(long long H, long long M) {
-  return S == 0 ? 2 * H + (M >> 30) : (H >> (S > 0 ? S - 1 : 0)) + (M >> (30 + S));
-}
-template <int S> FL_HD constexpr long long fx_centre() { return (1ll << (30 + S)) - (1ll << 29); }
+// v w / 8.  With v = vh 2^32 + vl the product is H 2^64 + M 2^32 + vl wl,
+// H = vh wh, M = vh wl + vl wh, so that v w 2^61 / 2^64 = H + M / 2^32: the
+// upper word of M is the addend of H's first multiply-add.  |v| < 2^62.5
+// keeps M within 2^63.  The constant in M's sum rounds it to nearest (zero
+// gives zero); the dropped vl wl / 2^64 is below half a unit.
+constexpr long long kFxRound = 1ll << 31;
+FL_HD long long fx_carry(long long M) { return (long long)(int)(M >> 32); }
 
-template <int S> FL_HD Fx fx_mul(Fx v, FxW w) {
+FL_HD Fx fx_mul(Fx v, FxW w) {
   const int xh = fx_hi(v.x), xl = fx_lo(v.x), yh = fx_hi(v.y), yl = fx_lo(v.y);
-  Fx r;
-  r.x = fx_join<S>(fx_mad(xh, w.xh, fx_mad(-yh, w.yh, 0)),
-                   fx_mad(xh, w.xl, fx_mad(xl, w.xh, fx_mad(-yh, w.yl, fx_mad(-yl, w.yh, fx_centre<S>())))));
-  r.y = fx_join<S>(fx_mad(xh, w.yh, fx_mad(yh, w.xh, 0)),
-                   fx_mad(xh, w.yl, fx_mad(xl, w.yh, fx_mad(yh, w.xl, fx_mad(yl, w.xh, fx_centre<S>())))));
-  return r;
+  const long long mx = fx_mad(xh, w.xl, fx_mad(xl, w.xh, fx_mad(yh, -w.yl, fx_mad(yl, -w.yh, kFxRound))));
+  const long long my = fx_mad(xh, w.yl, fx_mad(xl, w.yh, fx_mad(yh, w.xl, fx_mad(yl, w.xh, kFxRound))));
+  return Fx{fx_mad(xh, w.xh, fx_mad(yh, -w.yh, fx_carry(mx))), fx_mad(xh, w.yh, fx_mad(yh, w.xh, fx_carry(my)))};
 }
-// imaginary part of v w
+// imaginary part of v w / 8
 FL_HD long long fx_mul_im(Fx v, FxW w) {
   const int xh = fx_hi(v.x), xl = fx_lo(v.x), yh = fx_hi(v.y), yl = fx_lo(v.y);
-  return fx_join<0>(fx_mad(xh, w.yh, fx_mad(yh, w.xh, 0)),
-                    fx_mad(xh, w.yl, fx_mad(xl, w.yh, fx_mad(yh, w.xl, fx_mad(yl, w.xh, fx_centre<0>())))));
+  const long long m = fx_mad(xh, w.yl, fx_mad(xl, w.yh, fx_mad(yh, w.xl, fx_mad(yl, w.xh, kFxRound))));
+  return fx_mad(xh, w.yh, fx_mad(yh, w.xh, fx_carry(m)));
 }
-// v times a real constant
+// v times a real constant / 8
 FL_HD long long fx_mul_real(long long v, FxR w) {
   const int h = fx_hi(v), l = fx_lo(v);
-  return fx_join<0>(fx_mad(h, w.h, 0), fx_mad(h, w.l, fx_mad(l, w.h, fx_centre<0>())));
+  return fx_mad(h, w.h, fx_carry(fx_mad(h, w.l, fx_mad(l, w.h, kFxRound))));
 }
 FL_HD Fx fx_mul_real(Fx v, FxR w) { return Fx{fx_mul_real(v.x, w), fx_mul_real(v.y, w)}; }
 
 // --- butterflies (forward) ----------------------------------------------------
 
-// cos(pi/8), sin(pi/8), sqrt(1/2), times 2^61
-constexpr long long kFxC1 = 2130321161396766249ll;
-constexpr long long kFxS1 = 882407917260943721ll;
-constexpr long long kFxH = 1630477228166597777ll;
-
-// v (c - i s), c and s constants (folded at compile time)
-FL_HD Fx fx_rot(Fx v, long long c, long long s) {
-  const FxR k = fx_real(c), t = fx_real(-s);
-  return fx_mul<0>(v, FxW{k.h, k.l, t.h, t.l});
+// v sqrt(1/2) = v - v (1 - sqrt(1/2)), the constant with 64 fraction bits
+// (below 1/2, so that its upper half fits 32 signed bits)
+constexpr unsigned long long kFx1mH = 5402926248376769404ull;
+FL_HD long long fx_half(long long v) {
+  constexpr FxR w = fx_real((long long)kFx1mH);
+  const int h = fx_hi(v), l = fx_lo(v);
+  return v - fx_mad(h, w.h, fx_carry(fx_mad(h, w.l, fx_mad(l, w.h, kFxRound))));
 }
-FL_HD long long fx_half(long long v) { return fx_mul_real(v, fx_real(kFxH)); }
 // v exp(-i pi / 4) and v exp(-3 i pi / 4)
 FL_HD Fx fx_rot45(Fx v) { return Fx{fx_half(v.x + v.y), fx_half(v.y - v.x)}; }
 FL_HD Fx fx_rot135(Fx v) { return Fx{fx_half(v.y - v.x), -fx_half(v.x + v.y)}; }
@@ -157,47 +155,11 @@ FL_HD void fx_dft8(Fx* v) {
     v[k + 4] = fx_sub(e[k], o[k]);
   }
 }
-// 16 points as 4 x 4 (the same split as dft16).  HALF: x[8..15] are zero.
-template <bool HALF> FL_HD void fx_dft16(Fx* v) {
-  Fx a[4][4];
-#pragma unroll
-  for (int n2 = 0; n2 < 4; ++n2) {
-    if (HALF) {
-      const Fx x0 = v[n2], x1 = v[4 + n2];
-      a[n2][0] = fx_add(x0, x1);
-      a[n2][1] = Fx{x0.x + x1.y, x0.y - x1.x};
-      a[n2][2] = fx_sub(x0, x1);
-      a[n2][3] = Fx{x0.x - x1.y, x0.y + x1.x};
-    } else {
-      a[n2][0] = v[n2];
-      a[n2][1] = v[4 + n2];
-      a[n2][2] = v[8 + n2];
-      a[n2][3] = v[12 + n2];
-      fx_dft4(a[n2]);
-    }
-  }
-  a[1][1] = fx_rot(a[1][1], kFxC1, kFxS1);
-  a[1][2] = fx_rot45(a[1][2]);
-  a[1][3] = fx_rot(a[1][3], kFxS1, kFxC1);
-  a[2][1] = fx_rot45(a[2][1]);
-  a[2][2] = fx_mi(a[2][2]);
-  a[2][3] = fx_rot135(a[2][3]);
-  a[3][1] = fx_rot(a[3][1], kFxS1, kFxC1);
-  a[3][2] = fx_rot135(a[3][2]);
-  a[3][3] = fx_rot(a[3][3], -kFxC1, -kFxS1);
-#pragma unroll
-  for (int k1 = 0; k1 < 4; ++k1) {
-    Fx b[4] = {a[0][k1], a[1][k1], a[2][k1], a[3][k1]};
-    fx_dft4(b);
-#pragma unroll
-    for (int k2 = 0; k2 < 4; ++k2) v[k1 + 4 * k2] = b[k2];
-  }
-}
-template <int R, bool HALF> FL_HD void fx_dft(Fx* v) {
+template <int R> FL_HD void fx_dft(Fx* v) {
+  static_assert(R <= 8, "stages of at most 8 legs");
   if constexpr (R == 2) fx_dft2(v);
   else if constexpr (R == 4) fx_dft4(v);
-  else if constexpr (R == 8) fx_dft8(v);
-  else fx_dft16<HALF>(v);
+  else fx_dft8(v);
 }
 
 // --- FP64 in and out --------------------------------------------------------------
@@ -223,20 +185,19 @@ FL_HD double fx_from_bits(long long b) {
 // exponent field of a double (0: zero or subnormal, 2047: not finite)
 FL_HD int fx_field(double d) { return (int)(fx_bits(d) >> 52) & 0x7ff; }
 
-// d on a line whose largest exponent field is E, below 2^(61 - LR): the
-// first stage's division by R = 2^LR included.  The value is f 2^X with
-// X = fx_x0(E) + LR.
+// d on a line whose largest exponent field is E, below 2^(62 - LR).  The
+// value is f 2^X with X = fx_x0(E) + LR.
 template <int LR> FL_HD long long fx_from(double d, int E) {
   const long long b = fx_bits(d);
   const int e = (int)(b >> 52) & 0x7ff;
   // fraction with its hidden bit at 2^62; subnormals have none and exponent 1
   const unsigned long long m = ((unsigned long long)b << 10 & 0x3ffffffffffffc00ull) | (e ? 1ull << 62 : 0ull);
-  int s = (E > 1 ? E : 1) - (e ? e : 1) + 2 + LR;
+  int s = (E > 1 ? E : 1) - (e ? e : 1) + 1 + LR;
   if (s > 63) s = 63;
   const long long f = (long long)(m >> s);
   return b < 0 ? -f : f;
 }
-FL_HD int fx_x0(int E) { return E == 0x7ff ? kFxBad : (E > 1 ? E : 1) - 1083; }
+FL_HD int fx_x0(int E) { return E == 0x7ff ? kFxBad : (E > 1 ? E : 1) - 1084; }
 
 // f 2^X rounded to nearest (ties up in magnitude) where no result can leave
 // the normal range, 2 - 1023 <= X <= 2046 - 1088

@@ -11,16 +11,16 @@
 // the tile width.
 //
 // The FP64 forms of these passes were bound by the FP64 pipe (82 % busy at
-// 1.7 operations per clock and SM).  These are bound by instruction issue on
-// the integer pipes; FP64 instructions are left in the epilogues only (two
-// to six per output).  Measured on one GB300 with the FP64 forms before:
-// 1023^2 apply 516 -> 160 us, 96 x 135 x 75 apply 2624 -> 818 us, 511^2
-// FP64 CG solve 28.8 -> 14.5 ms, two 256^3 mixed time steps 125 -> 81 ms.
+// 1.7 operations per clock and SM).  These are bound by the integer pipes
+// (math-pipe throttle is the largest stall, issue 0.5 to 0.64 per cycle);
+// FP64 instructions are left in the epilogues only (two to six per output).
+// Measured on one GB300, applies in a CUDA graph, FP64 form -> this one:
+// 64^2 155 -> 40 us, 512^2 203 -> 58 us, 1024^2 508 -> 140 us, 256^3 13.0 ->
+// 3.1 ms; preconditioner solves 148 -> 62, 200 -> 81, 711 -> 171 us and 16.9
+// -> 4.8 ms.
 #pragma once
 
 namespace fl {
-
-template <int V> struct IntC { static constexpr int v = V; };
 
 // Exponent key of an FP64 value: upper word of |v|, nonzero for every v != 0.
 __device__ __forceinline__ unsigned fx_key(double v) {
@@ -63,14 +63,14 @@ __device__ __forceinline__ void fx_note(unsigned* mx, int line, unsigned m, int 
 }
 
 // One stage (see stage_ct): legs are shifted up by their line's headroom
-// (bits recorded in mx_in by the stage before), divided by R and summed.
-// load(line, index, c, IntC<log2 R>) gives the first stage's legs, already
-// divided (c: the line's word of slot 0); epi(line, index, value, X, ctx)
+// (bits recorded by the stage before), divided by 8 and summed.
+// load(line, index, c) gives the first stage's legs, already divided by 8
+// (c: the line's word of slot 0); epi(line, index, value, X, ctx)
 // takes the last stage's outputs and returns their magnitude bits.
 template <int R, int VPT, bool IL, int LG, int NS, int ST, int MODE, bool HALF, bool HOUT, typename Load,
           typename Epi>
 __device__ __forceinline__ void fx_stage(SBuf<Fx> buf, int ls, int ltx, int nlines, const FxW* FL_RESTRICT tw,
-                                         int lgmax, unsigned* mx, int cap, unsigned* mx_out, int dx0, Load& load,
+                                         int lgmax, unsigned* mx, int cap, unsigned* mx_out, Load& load,
                                          Epi& epi, bool sync_io) {
   typedef FftPlan<LG, VPT> P;
   constexpr int NB = VPT / R;
@@ -95,7 +95,7 @@ __device__ __forceinline__ void fx_stage(SBuf<Fx> buf, int ls, int ltx, int nlin
       if constexpr (MODE == STAGE_FIRST) {
 #pragma unroll
         for (int r = 0; r < R; ++r)
-          v[b][r] = (HALF && 2 * r >= R) ? Fx{0, 0} : load(line, j + r * RUN, c, IntC<LR>());
+          v[b][r] = (HALF && 2 * r >= R) ? Fx{0, 0} : load(line, j + r * RUN, c);
       } else {
         const int sh = fx_headroom(c);
         const int l0 = IL ? ((j << ltx) + line) : (line * ls + j);
@@ -108,11 +108,11 @@ __device__ __forceinline__ void fx_stage(SBuf<Fx> buf, int ls, int ltx, int nlin
           for (int r = 0; r < R; ++r) v[b][r] = fx_shl(buf[l0 + (IL ? ((r * RUN) << ltx) : r * RUN)], sh);
         }
         const int step = k << (lgmax - clog2(NS * R));
-        v[b][0] = fx_shr<LR>(v[b][0]);
+        v[b][0] = fx_shr<kFxShift>(v[b][0]);
 #pragma unroll
-        for (int r = 1; r < R; ++r) v[b][r] = fx_mul<LR>(v[b][r], tw[r * step]);
+        for (int r = 1; r < R; ++r) v[b][r] = fx_mul(v[b][r], tw[r * step]);
       }
-      fx_dft<R, (HALF && R == 16 && MODE == STAGE_FIRST)>(v[b]);
+      fx_dft<R>(v[b]);
       line_of[b] = line;
       out0[b] = (j - k) * R + k;
     }
@@ -125,9 +125,9 @@ __device__ __forceinline__ void fx_stage(SBuf<Fx> buf, int ls, int ltx, int nlin
       if constexpr (MODE == STAGE_LAST) {
         // exponent change over the transform, X of this line relative to its
         // input
-        int X = dx0;
+        int X = kFxShift;
 #pragma unroll
-        for (int s = 1; s < P::S; ++s) X += clog2(P::radix(s)) - fx_headroom(mx[s * cap + line_of[b]]);
+        for (int s = 1; s < P::S; ++s) X += kFxShift - fx_headroom(mx[s * cap + line_of[b]]);
         epi.begin(line_of[b], X, mx[line_of[b]]);
         // HOUT: only the lower half of the line is wanted
 #pragma unroll
@@ -168,7 +168,7 @@ __device__ __forceinline__ void fx_stages(SBuf<Fx> buf, int ls, int ltx, int nli
   constexpr int R = P::radix(ST);
   constexpr int MODE = ST == 0 ? STAGE_FIRST : (ST == P::S - 1 ? STAGE_LAST : STAGE_MID);
   fx_stage<R, VPT, IL, LG, P::ns(ST), ST, MODE, HALF, HOUT>(buf, ls, ltx, nlines, tw, lgmax, mx, cap, mx_out,
-                                                            LogR<P::radix(0)>::v, load, epi,
+                                                            load, epi,
                                                             MODE == STAGE_FIRST ? sync_load : sync_epi);
   if constexpr (ST + 1 < P::S)
     fx_stages<LG, VPT, IL, HALF, HOUT, ST + 1>(buf, ls, ltx, nlines, tw, lgmax, mx, cap, mx_out, load, sync_load,
@@ -184,29 +184,9 @@ template <int LG, int VPT, bool IL, bool HALF, bool HOUT, typename Load, typenam
 __device__ __forceinline__ void fx_fft_ct(SBuf<Fx> buf, int ls, int ltx, int nlines, const FxW* FL_RESTRICT tw,
                                           int lgmax, unsigned* mx, int cap, unsigned* mx_out, Load load,
                                           bool sync_load, Epi epi, bool sync_epi) {
-  typedef FftPlan<LG, VPT> P;
-  if constexpr (P::S >= 2) {
-    fx_stages<LG, VPT, IL, HALF, HOUT, 0>(buf, ls, ltx, nlines, tw, lgmax, mx, cap, mx_out, load, sync_load, epi,
-                                          sync_epi);
-  } else {
-    // one stage: natural order in shared memory, then element by element
-    // (an epilogue writing the buffer rewrites the element it was given)
-    unsigned* none = mx;
-    constexpr int L = 1 << LG;
-    static_assert(P::radix(0) == L, "one stage");
-    // the recorded bits of this stage's own outputs are not needed: they go
-    // where the caller's spare slot is
-    fx_stage<L, VPT, IL, LG, 1, 0, STAGE_FIRST, HALF, HOUT>(buf, ls, ltx, nlines, tw, lgmax, none, cap, mx_out,
-                                                            LogR<L>::v, load, epi, sync_load);
-    const int total = IL ? (L << ltx) : nlines * L;
-    for (int e = threadIdx.x; e < total; e += blockDim.x) {
-      const int line = IL ? (e & ((1 << ltx) - 1)) : e / L;
-      const int j = IL ? (e >> ltx) : e % L;
-      epi.begin(line, LogR<L>::v, mx[line]);
-      const unsigned m = epi(line, j, IL ? buf[e] : buf[line * ls + j]);
-      if (Epi::kNote && m) atomicOr(mx_out + line, m);
-    }
-  }
+  static_assert(FftPlan<LG, VPT>::S >= 2, "a first and a last stage");
+  fx_stages<LG, VPT, IL, HALF, HOUT, 0>(buf, ls, ltx, nlines, tw, lgmax, mx, cap, mx_out, load, sync_load, epi,
+                                        sync_epi);
 }
 
 #define FL_FX_LEN(LGV)                                                                                  \
@@ -235,8 +215,8 @@ __device__ __forceinline__ void fx_fft(SBuf<Fx> buf, int lg, int ls, int ltx, in
 #undef FL_FX_LEN
 
 // Words of line bookkeeping of a CTA of THREADS x VPT values: per transform
-// S slots of one word per line, at most VALUES/16 (length 16: one slot; the
-// longer lengths have fewer lines), and one spare slot for length 16.
+// S slots of one word per line, at most 2 x VALUES/16 (length 16: two slots;
+// the longer lengths have fewer lines).
 constexpr int fx_words(int threads, int vpt, int lglo) {
   return lglo > 4 ? 8 : threads * vpt / 8;
 }
@@ -252,11 +232,10 @@ struct FxLoadRaw {
   SBuf<Fx> buf;
   int ls, ltx;
   bool il, swap;
-  template <int LR>
-  __device__ __forceinline__ Fx operator()(int q, int k, unsigned key, IntC<LR>) const {
+  __device__ __forceinline__ Fx operator()(int q, int k, unsigned key) const {
     const Fx w = il ? buf[(k << ltx) + q] : buf[q * ls + k];
     const int E = fx_line_field(key);
-    const Fx v = Fx{fx_from<LR>(__longlong_as_double(w.x), E), fx_from<LR>(__longlong_as_double(w.y), E)};
+    const Fx v = Fx{fx_from<kFxShift>(__longlong_as_double(w.x), E), fx_from<kFxShift>(__longlong_as_double(w.y), E)};
     return swap ? fx_swap(v) : v;
   }
 };
@@ -265,10 +244,9 @@ struct FxLoadFix {
   SBuf<Fx> buf;
   int ls, ltx;
   bool il;
-  template <int LR>
-  __device__ __forceinline__ Fx operator()(int q, int k, unsigned m, IntC<LR>) const {
+  __device__ __forceinline__ Fx operator()(int q, int k, unsigned m) const {
     const Fx v = il ? buf[(k << ltx) + q] : buf[q * ls + k];
-    return fx_swap(fx_shr<LR>(fx_shl(v, fx_headroom(m))));
+    return fx_swap(fx_shr<kFxShift>(fx_shl(v, fx_headroom(m))));
   }
 };
 // FP64 real values (in .x of the staged element) times the chirp
@@ -277,11 +255,10 @@ struct FxLoadChirp {
   const FxW* FL_RESTRICT chirp;
   int ls, ltx, n;
   bool il;
-  template <int LR>
-  __device__ __forceinline__ Fx operator()(int q, int k, unsigned key, IntC<LR>) const {
+  __device__ __forceinline__ Fx operator()(int q, int k, unsigned key) const {
     if (k >= n) return Fx{0, 0};
     const Fx w = il ? buf[(k << ltx) + q] : buf[q * ls + k];
-    const long long x = fx_from<LR>(__longlong_as_double(w.x), fx_line_field(key));
+    const long long x = fx_from<0>(__longlong_as_double(w.x), fx_line_field(key));
     const FxW c = chirp[k];
     return Fx{fx_mul_real(x, FxR{c.xh, c.xl}), fx_mul_real(x, FxR{c.yh, c.yl})};
   }
@@ -307,9 +284,9 @@ struct FxMulStore {
   int* xs;
   int ls, ltx, wexp;
   bool il;
-  __device__ __forceinline__ void begin(int q, int X, unsigned key) { xs[q] = fx_x0(fx_line_field(key)) + X + wexp; }
+  __device__ __forceinline__ void begin(int q, int X, unsigned key) { xs[q] = fx_x0(fx_line_field(key)) + X + wexp + kFxShift; }
   __device__ __forceinline__ unsigned operator()(int q, int k, Fx v) {
-    v = fx_mul<0>(v, w[k]);
+    v = fx_mul(v, w[k]);
     if (il) buf[(k << ltx) + q] = v;
     else buf[q * ls + k] = v;
     return fx_mag(v.x) | fx_mag(v.y);
@@ -322,7 +299,7 @@ struct FxSymStore {
   const FxR* sig;
   int* xs;
   int ltx, L, wexp;
-  __device__ __forceinline__ void begin(int q, int X, unsigned key) { xs[q] = fx_x0(fx_line_field(key)) + X + wexp; }
+  __device__ __forceinline__ void begin(int q, int X, unsigned key) { xs[q] = fx_x0(fx_line_field(key)) + X + wexp + kFxShift; }
   __device__ __forceinline__ unsigned operator()(int q, int k, Fx v) {
     v = fx_mul_real(v, sig[(min(k, L - k) << ltx) + q]);
     buf[(k << ltx) + q] = v;
@@ -444,11 +421,13 @@ __device__ __forceinline__ void fx_body_rows_fwd(const RowsFwdArgs<double>& a, i
     double2* Sa = a.S + ((size_t)(ra / a.rows_per_plane) * a.plane_stride + ra % a.rows_per_plane) * a.H;
     double2* Sb = a.S + ((size_t)(rb / a.rows_per_plane) * a.plane_stride + rb % a.rows_per_plane) * a.H;
     const SBuf<Fx> lb = buf.at(q * ls);
-    const int X = s_x[q] - 1;   // the halves below
+    const int X = s_x[q];
     for (int k = e & (hL - 1); k <= hL; k += hL) {
       const Fx z = lb[k], w = lb[(L - k) & (L - 1)];
-      Sa[k] = make_double2(fx_to(z.x + w.x, X), fx_to(z.y - w.y, X));
-      if (hb) Sb[k] = make_double2(fx_to(z.y + w.y, X), fx_to(w.x - z.x, X));
+      // halved before the sums, which could pass 2^63
+      const long long zx = z.x >> 1, zy = z.y >> 1, wx = w.x >> 1, wy = w.y >> 1;
+      Sa[k] = make_double2(fx_to(zx + wx, X), fx_to(zy - wy, X));
+      if (hb) Sb[k] = make_double2(fx_to(zy + wy, X), fx_to(wx - zx, X));
       if (k > 0) break;
     }
   }
@@ -608,7 +587,7 @@ __device__ __forceinline__ void fx_body_rows_inv(const RowsInvArgs<double>& a, i
   }
   __syncthreads();
   // Z[k] = xa[k] + i xb[k], Z[L-k] = conj xa[k] + i conj xb[k], in place
-  // (each pair of places by one thread); inputs below 2^60, sums below 2^61
+  // (each pair of places by one thread); inputs below 2^61, sums below 2^62
   for (int e = threadIdx.x; e < tot; e += THREADS) {
     const int q = e >> (lg - 1), k = e & (hL - 1);
     const SBuf<Fx> lb = buf.at(q * ls);
@@ -688,7 +667,9 @@ struct FxDstRowsEpi {
   const int* xs;
   DotAcc<double>& dp;
   int row0, X;
-  __device__ __forceinline__ void begin(int q, int dX, unsigned m) { X = xs[q] + dX - fx_headroom(m); }
+  __device__ __forceinline__ void begin(int q, int dX, unsigned m) {
+    X = xs[q] + dX - fx_headroom(m) + kFxShift;   // + kFxShift: the chirp product below
+  }
   __device__ __forceinline__ unsigned operator()(int q, int k, Fx v) {
     if (k < a.n) {
       const size_t idx = (size_t)(row0 + q) * a.n + k;
@@ -799,7 +780,9 @@ struct FxDstColsEpi {
   double* base;
   const int* xs;
   int ncol, X;
-  __device__ __forceinline__ void begin(int q, int dX, unsigned m) { X = xs[q] + dX - fx_headroom(m); }
+  __device__ __forceinline__ void begin(int q, int dX, unsigned m) {
+    X = xs[q] + dX - fx_headroom(m) + kFxShift;   // + kFxShift: the chirp product below
+  }
   __device__ __forceinline__ unsigned operator()(int c, int k, Fx v) {
     if (c < ncol && k < a.n) {
       double o = fx_to(fx_mul_im(fx_swap(v), a.fchirp[k]), X);

@@ -120,8 +120,10 @@ __device__ __forceinline__ double cta_sum_partials(const double* FL_RESTRICT par
 // The wide instantiations for the longest lines (LGLO > 4: one line of 4096
 // or 8192 points per CTA) ask for one CTA only, so that the compiler keeps
 // the row bodies' registers.
+// FP64 passes: four CTAs of 256 threads or two of 512 (64 registers).
+template <typename T = float>
 constexpr int min_ctas(int threads, int lglo = 4) {
-  return lglo > 4 ? 1 : (threads <= 128 ? FL_ROW_MIN_CTAS : 2);
+  return lglo > 4 ? 1 : (threads <= 128 ? FL_ROW_MIN_CTAS : (sizeof(T) == 8 && threads == 256 ? 4 : 2));
 }
 
 // Column tiles: at most 2^kMaxLtx columns; a CTA of THREADS x VPT values
@@ -401,7 +403,7 @@ __device__ __forceinline__ void body_rows_fwd(const RowsFwdArgs<T>& a, int bx, i
 }
 
 template <typename T, int THREADS, int VPT, int LGLO = 4>
-__global__ void __launch_bounds__(THREADS, min_ctas(THREADS, LGLO)) k_rows_fwd(RowsFwdArgs<T> a) {
+__global__ void __launch_bounds__(THREADS, min_ctas<T>(THREADS, LGLO)) k_rows_fwd(RowsFwdArgs<T> a) {
   pdl_wait();
   body_rows_fwd<T, THREADS, VPT, LGLO>(a, blockIdx.x, blockIdx.y);
   pdl_release();
@@ -556,7 +558,7 @@ __device__ __forceinline__ void body_cols(const ColsArgs<T>& a, int bx, int by) 
 }
 
 template <typename T, int THREADS, int VPT, int LGLO = 4>
-__global__ void __launch_bounds__(THREADS, min_ctas(THREADS, LGLO)) k_cols(ColsArgs<T> a) {
+__global__ void __launch_bounds__(THREADS, min_ctas<T>(THREADS, LGLO)) k_cols(ColsArgs<T> a) {
   pdl_wait();
   body_cols<T, THREADS, VPT, LGLO>(a, blockIdx.x, blockIdx.y);
   pdl_release();
@@ -719,7 +721,7 @@ __device__ __forceinline__ void body_rows_inv(const RowsInvArgs<T>& a, int bx, i
 }
 
 template <typename T, int THREADS, int VPT, int LGLO = 4>
-__global__ void __launch_bounds__(THREADS, min_ctas(THREADS, LGLO)) k_rows_inv(RowsInvArgs<T> a) {
+__global__ void __launch_bounds__(THREADS, min_ctas<T>(THREADS, LGLO)) k_rows_inv(RowsInvArgs<T> a) {
   pdl_wait();
   body_rows_inv<T, THREADS, VPT, LGLO>(a, blockIdx.x, blockIdx.y);
   pdl_release();
@@ -924,7 +926,7 @@ __device__ __forceinline__ void body_dst_rows(const DstRowsArgs<T>& a, int bx, i
 }
 
 template <typename T, int THREADS, int VPT, int LGLO = 4>
-__global__ void __launch_bounds__(THREADS, min_ctas(THREADS, LGLO)) k_dst_rows(DstRowsArgs<T> a) {
+__global__ void __launch_bounds__(THREADS, min_ctas<T>(THREADS, LGLO)) k_dst_rows(DstRowsArgs<T> a) {
   pdl_wait();
   body_dst_rows<T, THREADS, VPT, LGLO>(a, blockIdx.x, blockIdx.y);
   pdl_release();
@@ -1025,7 +1027,7 @@ __device__ __forceinline__ void body_dst_cols(const DstColsArgs<T>& a, int bx, i
 }
 
 template <typename T, int THREADS, int VPT, int LGLO = 4>
-__global__ void __launch_bounds__(THREADS, min_ctas(THREADS, LGLO)) k_dst_cols(DstColsArgs<T> a) {
+__global__ void __launch_bounds__(THREADS, min_ctas<T>(THREADS, LGLO)) k_dst_cols(DstColsArgs<T> a) {
   pdl_wait();
   body_dst_cols<T, THREADS, VPT, LGLO>(a, blockIdx.x, blockIdx.y);
   pdl_release();

@@ -245,6 +245,10 @@ __global__ void k_fill_kernel(double2* buf, int d, int L0, int L1, int L2, int n
   buf[i] = make_double2(v, 0.0);
 }
 
+// CTAs of the plan-time FP64 transforms: kSymT x kSymV values, twice the
+// threads for lines of 8192
+constexpr int kSymT = 256, kSymV = 16;
+
 template <int THREADS, int VPT>
 __global__ void __launch_bounds__(THREADS) k_rows_c2c(double2* buf, int rows, int lg, int lgmax,
                                                      const double2* tw) {
@@ -368,15 +372,18 @@ cudaError_t configure_kernels_f64() {
   FL_SET(k_cols<double, Cfg<double>::CT, Cfg<double>::CV>);
   FL_SET(k_dst_rows<double, Cfg<double>::RT, Cfg<double>::RV>);
   FL_SET(k_dst_cols<double, Cfg<double>::CT, Cfg<double>::CV>);
-  FL_SET(k_rows_c2c<Cfg<double>::RT, Cfg<double>::RV>);
-  FL_SET(k_rows_fwd<double, 512, 16, 13>);
-  FL_SET(k_rows_inv<double, 512, 16, 13>);
-  FL_SET(k_dst_rows<double, 512, 16, 13>);
-  FL_SET(k_cols<double, 512, 16, 13>);
-  FL_SET(k_dst_cols<double, 512, 16, 13>);
-  FL_SET(k_rows_c2c<2 * Cfg<double>::RT, Cfg<double>::RV>);
-  FL_SET(k_cols_c2c<Cfg<double>::CT, Cfg<double>::CV>);
-  FL_SET(k_cols_c2c<2 * Cfg<double>::CT, Cfg<double>::CV, 13>);
+  FL_SET(k_rows_fwd<double, 512, 8, 12>);
+  FL_SET(k_rows_inv<double, 512, 8, 12>);
+  FL_SET(k_dst_rows<double, 512, 8, 12>);
+  FL_SET(k_rows_fwd<double, 1024, 8, 13>);
+  FL_SET(k_rows_inv<double, 1024, 8, 13>);
+  FL_SET(k_dst_rows<double, 1024, 8, 13>);
+  FL_SET(k_cols<double, 1024, 8, 13>);
+  FL_SET(k_dst_cols<double, 1024, 8, 13>);
+  FL_SET(k_rows_c2c<kSymT, kSymV>);
+  FL_SET(k_rows_c2c<2 * kSymT, kSymV>);
+  FL_SET(k_cols_c2c<kSymT, kSymV>);
+  FL_SET(k_cols_c2c<2 * kSymT, kSymV, 13>);
 #undef FL_SET
   return e;
 }
@@ -730,7 +737,6 @@ cudaError_t launch_sum(cudaStream_t s, const double* part, int count, double* ou
 #if FL_OPS_PART == 2
 cudaError_t build_symbol(const Geo& g, double c, double Z, double a, double expo, cudaStream_t s,
                          FxR* fsig, int* sig_exp, float* sig32, const double2* tw64) {
-  typedef Cfg<double> K;
   const int d = g.d;
   long long total = 1, half = 1;
   int Ls[3] = {1, 1, 1}, ns[3] = {1, 1, 1};
@@ -751,15 +757,15 @@ cudaError_t build_symbol(const Geo& g, double c, double Z, double a, double expo
   {
     const int L = g.L[d - 1];
     const long long rows = total / L;
-    const int NL = row_lines<double>(L);
+    const int NL = std::max(1, kSymT * kSymV / L);
     const unsigned blocks = (unsigned)((rows + NL - 1) / NL);
-    if (L <= K::RT * K::RV)
+    if (L <= kSymT * kSymV)
       FL_KERNEL("rows_c2c", s,
-                k_rows_c2c<K::RT, K::RV><<<blocks, K::RT, smem_bytes<double>(NL, L), s>>>(
+                k_rows_c2c<kSymT, kSymV><<<blocks, kSymT, smem_bytes<double>(NL, L), s>>>(
                     buf, (int)rows, g.lg[d - 1], g.lgmax, tw64));
     else
       FL_KERNEL("rows_c2c", s,
-                k_rows_c2c<2 * K::RT, K::RV><<<blocks, 2 * K::RT, smem_bytes<double>(NL, L), s>>>(
+                k_rows_c2c<2 * kSymT, kSymV><<<blocks, 2 * kSymT, smem_bytes<double>(NL, L), s>>>(
                     buf, (int)rows, g.lg[d - 1], g.lgmax, tw64));
   }
   // slower axes: strided lines, full length in and out
@@ -769,15 +775,15 @@ cudaError_t build_symbol(const Geo& g, double c, double Z, double a, double expo
     if (d == 2) { lstride = Ls[1]; }
     else if (axis == 1) { lstride = Ls[2]; ostride = (long long)Ls[1] * Ls[2]; nouter = Ls[0]; }
     else { lstride = (long long)Ls[1] * Ls[2]; ostride = Ls[2]; nouter = Ls[1]; }
-    const int L = Ls[axis], tx = col_tx<double>(L);
+    const int L = Ls[axis], tx = std::min(kMaxTx, std::max(1, kSymT * kSymV / L));
     const dim3 grid((Ls[d - 1] + tx - 1) / tx, nouter);
-    if (L <= K::CT * K::CV)
+    if (L <= kSymT * kSymV)
       FL_KERNEL("cols_c2c", s,
-                k_cols_c2c<K::CT, K::CV><<<grid, K::CT, tile_bytes<double>(tx, L), s>>>(
+                k_cols_c2c<kSymT, kSymV><<<grid, kSymT, tile_bytes<double>(tx, L), s>>>(
                     buf, Ls[d - 1], g.lg[axis], g.lgmax, ostride, lstride, ilog2i(tx), tw64));
     else
       FL_KERNEL("cols_c2c", s,
-                k_cols_c2c<2 * K::CT, K::CV, clog2(2 * K::CT * K::CV)><<<grid, 2 * K::CT, tile_bytes<double>(tx, L), s>>>(
+                k_cols_c2c<2 * kSymT, kSymV, 13><<<grid, 2 * kSymT, tile_bytes<double>(tx, L), s>>>(
                     buf, Ls[d - 1], g.lg[axis], g.lgmax, ostride, lstride, ilog2i(tx), tw64));
   }
   double inv = 1.0;
