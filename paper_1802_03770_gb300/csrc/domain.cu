@@ -19,17 +19,19 @@
 // B z~ = r~ with z~ = 0 at every neighbour outside Omega: B_Omega z = r.
 //
 // C is formed once per (shift, scale) from |Gamma| FP64 box solves of unit
-// vectors, factorised as L D L^T (right-looking, one launch per pivot), and
-// each application solves with the factor in one CTA (FP64, for either
-// precision of the box solves).
+// vectors and factorised as L D L^T (right-looking, one launch per pivot);
+// the same eliminations applied to the identity give W = L^{-1}.  Each
+// application is then s = -W^T D^{-1} W E^T w: two triangular matrix-vector
+// products over the whole GPU (FP64, for either precision of the box
+// solves), bound by the FP64 rate and the launches.  The blocked
+// substitutions they replace ran in one CTA, one dependent block of 32
+// unknowns after another: 86 us for |Gamma| = 255 between events, now 12 + 7.
 #include "chain.cuh"
 #include "domain.h"
 
 namespace fl {
 
 namespace {
-
-constexpr int kDomThreads = 1024;
 
 // e = unit vector at Gamma point `cur` (and the previous one cleared).
 __global__ void k_dom_unit(double* e, const int* __restrict__ idx, int prev, int cur) {
@@ -46,92 +48,82 @@ __global__ void k_dom_gather(const double* __restrict__ z, const int* __restrict
   if (b < m) C[(size_t)b * m + col] = z[idx[b]];
 }
 
-// C = (C + C^T) / 2 (the box solves are symmetric up to rounding).
+// Lower triangle: (C + C^T) / 2 (the box solves are symmetric up to
+// rounding).  Strict upper triangle: zeros, where W^T is built.
 __global__ void k_dom_symmetrize(double* C, int m) {
   const int i = blockIdx.y * blockDim.y + threadIdx.y;
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < m && j < i) {
-    const double v = 0.5 * (C[(size_t)i * m + j] + C[(size_t)j * m + i]);
-    C[(size_t)i * m + j] = v;
-    C[(size_t)j * m + i] = v;
+    C[(size_t)i * m + j] = 0.5 * (C[(size_t)i * m + j] + C[(size_t)j * m + i]);
+    C[(size_t)j * m + i] = 0.0;
   }
 }
 
-// Pivot k of the right-looking L D L^T factorisation (lower triangle):
-// A_ij -= A_ik A_jk / A_kk for k < j <= i.
+// Pivot k of the right-looking L D L^T factorisation, rows i > k, with the
+// factors l_i = A_ik / A_kk (one division per row and CTA: FP64 divisions
+// are tens of operations).  z = 0: A_ij -= l_i A_jk, k < j <= i (lower
+// triangle); z = 1: W_ij -= l_i W_kj, j <= k (W_ij at [j][i], W_kk = 1).
+constexpr int kDomTile = 16;
 __global__ void k_dom_ldl_step(double* C, int m, int k) {
-  const int i = k + 1 + blockIdx.y * blockDim.y + threadIdx.y;
-  const int j = k + 1 + blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < m && j <= i) {
-    const double piv = C[(size_t)k * m + k];
-    C[(size_t)i * m + j] -= C[(size_t)i * m + k] * C[(size_t)j * m + k] / piv;
+  __shared__ double l[kDomTile];
+  const bool inv = blockIdx.z == 1;
+  // the index that runs along threadIdx.x is the contiguous one: j of A, i of W
+  const int i0 = k + 1 + (inv ? blockIdx.x : blockIdx.y) * kDomTile;
+  if (threadIdx.y == 0 && i0 + threadIdx.x < m)
+    l[threadIdx.x] = C[(size_t)(i0 + threadIdx.x) * m + k] / C[(size_t)k * m + k];
+  __syncthreads();
+  if (!inv) {
+    const int i = i0 + threadIdx.y, j = k + 1 + blockIdx.x * kDomTile + threadIdx.x;
+    if (i < m && j <= i) C[(size_t)i * m + j] -= l[threadIdx.y] * C[(size_t)j * m + k];
+  } else {
+    const int i = i0 + threadIdx.x, j = blockIdx.y * kDomTile + threadIdx.y;
+    if (i < m && j <= k) C[(size_t)j * m + i] -= l[threadIdx.x] * (j < k ? C[(size_t)j * m + k] : 1.0);
   }
 }
 
-// After the last pivot: L'_ik = A_ik / A_kk below the diagonal (unit lower
-// factor), D_k = A_kk on it.
-__global__ void k_dom_ldl_scale(double* C, int m) {
-  const int i = blockIdx.y * blockDim.y + threadIdx.y;
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < m && k < i) C[(size_t)i * m + k] /= C[(size_t)k * m + k];
-}
-
-// s = -C^{-1} w_Gamma with C = L' D L'^T, scattered to us at Gamma (us is
-// zero elsewhere and stays so).  One CTA; the triangular solves run in
-// blocks of 32 unknowns: warp 0 solves the block (shuffles), then every
-// thread updates the unknowns after (forward) or before (backward) it.
+// t = -D^{-1} W w_Gamma: 32 rows per CTA (threadIdx.x), their columns split
+// over threadIdx.y.
 template <typename T>
-__global__ void __launch_bounds__(kDomThreads) k_dom_solve(const T* __restrict__ w,
-                                                           const int* __restrict__ idx,
-                                                           const double* __restrict__ LD, int m,
-                                                           T* __restrict__ us, const PcgState* st) {
-  extern __shared__ double b[];   // m values
+__global__ void __launch_bounds__(1024) k_dom_fwd(const T* __restrict__ w, const int* __restrict__ idx,
+                                                  const double* __restrict__ LD, int m,
+                                                  double* __restrict__ t, const PcgState* st) {
+  __shared__ double part[32][33];
+  pdl_wait();
   if (st && st->done) return;
-  const int tid = threadIdx.x, lane = tid & 31;
-  for (int a = tid; a < m; a += kDomThreads) b[a] = -(double)w[idx[a]];
-  __syncthreads();
-  // forward: L' y = b
-  for (int kb = 0; kb < m; kb += 32) {
-    const int nb = min(32, m - kb);
-    if (tid < 32) {
-      double v = lane < nb ? b[kb + lane] : 0.0;
-      for (int t = 0; t < nb; ++t) {
-        const double y = __shfl_sync(0xffffffffu, v, t);
-        if (lane > t && lane < nb) v -= LD[(size_t)(kb + lane) * m + kb + t] * y;
-      }
-      if (lane < nb) b[kb + lane] = v;
-    }
-    __syncthreads();
-    for (int i = kb + nb + tid; i < m; i += kDomThreads) {
-      const double* row = LD + (size_t)i * m + kb;
-      double acc = 0.0;
-      for (int t = 0; t < nb; ++t) acc += row[t] * b[kb + t];
-      b[i] -= acc;
-    }
-    __syncthreads();
+  const int i = blockIdx.x * 32 + threadIdx.x;
+  double acc = 0.0;
+  if (i < m) {
+#pragma unroll 4
+    for (int j = threadIdx.y; j < i; j += 32) acc += LD[(size_t)j * m + i] * (double)w[idx[j]];
   }
-  for (int a = tid; a < m; a += kDomThreads) b[a] /= LD[(size_t)a * m + a];
+  part[threadIdx.y][threadIdx.x] = acc;
   __syncthreads();
-  // backward: L'^T x = y
-  for (int kb = ((m - 1) / 32) * 32; kb >= 0; kb -= 32) {
-    const int nb = min(32, m - kb);
-    if (tid < 32) {
-      double v = lane < nb ? b[kb + lane] : 0.0;
-      for (int t = nb - 1; t >= 0; --t) {
-        const double x = __shfl_sync(0xffffffffu, v, t);
-        if (lane < t) v -= LD[(size_t)(kb + t) * m + kb + lane] * x;
-      }
-      if (lane < nb) b[kb + lane] = v;
-    }
-    __syncthreads();
-    for (int i = tid; i < kb; i += kDomThreads) {
-      double acc = 0.0;
-      for (int t = 0; t < nb; ++t) acc += LD[(size_t)(kb + t) * m + i] * b[kb + t];
-      b[i] -= acc;
-    }
-    __syncthreads();
+  // one warp per row
+  double v = part[threadIdx.x][threadIdx.y];
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  const int row = blockIdx.x * 32 + threadIdx.y;
+  if (threadIdx.x == 0 && row < m) t[row] = -(v + (double)w[idx[row]]) / LD[(size_t)row * m + row];
+  pdl_release();
+}
+
+// us = W^T t at Gamma (us is zero elsewhere and stays so): one warp per row.
+constexpr int kDomBwdWarps = 8;
+template <typename T>
+__global__ void __launch_bounds__(32 * kDomBwdWarps) k_dom_bwd(const double* __restrict__ t,
+                                                              const int* __restrict__ idx,
+                                                              const double* __restrict__ LD, int m,
+                                                              T* __restrict__ us, const PcgState* st) {
+  pdl_wait();
+  if (st && st->done) return;
+  const int j = blockIdx.x * kDomBwdWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (j < m) {
+    double acc = 0.0;
+#pragma unroll 4
+    for (int i = j + 1 + lane; i < m; i += 32) acc += LD[(size_t)j * m + i] * t[i];
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) us[idx[j]] = (T)(t[j] + acc);
   }
-  for (int a = tid; a < m; a += kDomThreads) us[idx[a]] = (T)b[a];
+  pdl_release();
 }
 
 }  // namespace
@@ -150,34 +142,27 @@ cudaError_t dom_build_capacitance(const Geo& g, const Tables<double>& tb, const 
     }
   }
   if (err != cudaSuccess) return err;
-  const dim3 blk(16, 16);
-  const dim3 grid((dd.m + 15) / 16, (dd.m + 15) / 16);
-  FL_KERNEL("dom_symmetrize", s, k_dom_symmetrize<<<grid, blk, 0, s>>>(dd.LD, dd.m));
+  const dim3 blk(kDomTile, kDomTile);
+  const int tiles = (dd.m + kDomTile - 1) / kDomTile;
+  FL_KERNEL("dom_symmetrize", s, k_dom_symmetrize<<<dim3(tiles, tiles), blk, 0, s>>>(dd.LD, dd.m));
   for (int k = 0; k + 1 < dd.m; ++k) {
-    const int r = dd.m - k - 1;
-    const dim3 gk((r + 15) / 16, (r + 15) / 16);
-    FL_KERNEL("dom_ldl_step", s, k_dom_ldl_step<<<gk, blk, 0, s>>>(dd.LD, dd.m, k));
+    const int below = (dd.m - k - 1 + kDomTile - 1) / kDomTile, left = (k + kDomTile) / kDomTile;
+    FL_KERNEL("dom_ldl_step", s,
+              k_dom_ldl_step<<<dim3(below, below > left ? below : left, 2), blk, 0, s>>>(dd.LD, dd.m, k));
   }
-  FL_KERNEL("dom_ldl_scale", s, k_dom_ldl_scale<<<grid, blk, 0, s>>>(dd.LD, dd.m));
   return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t dom_interface_solve(const DomainData& dd, const T* w, T* us, const PcgState* st,
                                 cudaStream_t s) {
-  FL_KERNEL(sizeof(T) == 4 ? "dom_solve<f32>" : "dom_solve<f64>", s,
-            k_dom_solve<T><<<1, kDomThreads, dd.m * sizeof(double), s>>>(w, dd.idx, dd.LD, dd.m, us, st));
-  return cudaGetLastError();
-}
-
-cudaError_t configure_domain_kernels() {
-  cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void*>(&k_dom_solve<float>),
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       kMaxGamma * (int)sizeof(double));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(reinterpret_cast<const void*>(&k_dom_solve<double>),
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxGamma * (int)sizeof(double));
-  return e;
+  FL_KERNEL(sizeof(T) == 4 ? "dom_fwd<f32>" : "dom_fwd<f64>", s,
+            pdl_launch(k_dom_fwd<T>, (dd.m + 31) / 32, dim3(32, 32), 0, s, w, (const int*)dd.idx,
+                       (const double*)dd.LD, dd.m, dd.t, st));
+  FL_KERNEL(sizeof(T) == 4 ? "dom_bwd<f32>" : "dom_bwd<f64>", s,
+            pdl_launch(k_dom_bwd<T>, (dd.m + kDomBwdWarps - 1) / kDomBwdWarps, 32 * kDomBwdWarps, 0, s,
+                       (const double*)dd.t, (const int*)dd.idx, (const double*)dd.LD, dd.m, us, st));
+  return launch_status();
 }
 
 template cudaError_t dom_interface_solve<float>(const DomainData&, const float*, float*, const PcgState*,

@@ -16,10 +16,13 @@ constexpr int kMaxGamma = 2048;
 struct DomainData {
   int m = 0;              // |Gamma|
   int* idx = nullptr;     // linear indices of Gamma in the box (m)
-  double* LD = nullptr;   // m x m: L' strictly below the diagonal, D on it
+  // m x m: D on the diagonal, W = L^{-1} transposed strictly above it (W_ij at
+  // [j][i]), the unscaled L below
+  double* LD = nullptr;
+  double* t = nullptr;    // m: D^{-1} W w between the two products
 };
 
-// Fills dd.LD with the L D L^T factor of C = E^T B^{-1} E for
+// Fills dd.LD with the inverted L D L^T factor of C = E^T B^{-1} E for
 // B = shift I + scale C h^d L_box, from m FP64 box solves of unit vectors
 // (e and z: N-double scratch; tb's tridiagonal table must hold shift,
 // scale).
@@ -31,7 +34,5 @@ cudaError_t dom_build_capacitance(const Geo& g, const Tables<double>& tb, const 
 template <typename T>
 cudaError_t dom_interface_solve(const DomainData& dd, const T* w, T* us, const PcgState* st,
                                 cudaStream_t s);
-
-cudaError_t configure_domain_kernels();
 
 }  // namespace fl

@@ -1104,6 +1104,7 @@ fl_status fl_plan_create(int d, const int64_t* n, double h, double alpha, const 
       FL_TRY(dalloc(p, &p->dom.idx, gam.size() * sizeof(int)));
       FL_TRY(cudaMemcpy(p->dom.idx, gam.data(), gam.size() * sizeof(int), cudaMemcpyHostToDevice));
       FL_TRY(dalloc(p, &p->dom.LD, (size_t)p->dom.m * p->dom.m * sizeof(double)));
+      FL_TRY(dalloc(p, &p->dom.t, (size_t)p->dom.m * sizeof(double)));
     }
     FL_TRY(dalloc(p, &p->dw32, g.N * sizeof(float)));
     FL_TRY(dalloc(p, &p->dus32, g.N * sizeof(float)));
@@ -1111,7 +1112,6 @@ fl_status fl_plan_create(int d, const int64_t* n, double h, double alpha, const 
     FL_TRY(dalloc(p, &p->dus64, g.N * sizeof(double)));
     FL_TRY(cudaMemset(p->dus32, 0, g.N * sizeof(float)));
     FL_TRY(cudaMemset(p->dus64, 0, g.N * sizeof(double)));
-    FL_TRY(configure_domain_kernels());
   }
   st = build_tables(p);
   if (st != FL_OK) { free_plan(p); return st; }
