@@ -47,7 +47,7 @@ FL_BATCHED_KERNEL(dst_cols, DstColsArgs)
 #undef FL_BATCHED_KERNEL
 
 template <typename T>
-__global__ void __launch_bounds__(kTriCols * kTriSeg)
+__global__ void __launch_bounds__(kTriCols<T> * kTriSeg)
     kb_tri_cols(const TriArgs<T>* __restrict__ args, const int* __restrict__ off, int nprob) {
   pdl_wait();
   const int i = batch_problem(off, nprob);
@@ -212,7 +212,7 @@ cudaError_t launch_batched(const BatchPass& bp, cudaStream_t s) {
       break;
     case BK_TRI_COLS:
       FL_KERNEL(sizeof(T) == 4 ? "b_tri_cols<f32>" : "b_tri_cols<f64>", s,
-                pdl_launch(kb_tri_cols<T>, bp.blocks, kTriCols * kTriSeg, 0, s,
+                pdl_launch(kb_tri_cols<T>, bp.blocks, kTriCols<T> * kTriSeg, 0, s,
                            (const TriArgs<T>*)bp.args, bp.off, bp.nprob));
       break;
     case BK_CG_START:

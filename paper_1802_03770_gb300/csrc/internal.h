@@ -104,7 +104,7 @@ struct PrecIO {
   const T* add = nullptr;         // nullable: out = mask ? (B^{-1} in + add) : 0
   int row_threads = 0;            // threads of a row-pass CTA; 0: the default shape
   int col_threads = 0;            // threads of a strided-pass CTA; 0: the default shape
-  int tri_cols = 0;               // columns per tridiagonal-pass CTA; 0: kTriCols
+  int tri_cols = 0;               // columns per tridiagonal-pass CTA; 0: the precision's kTriCols
 };
 
 // --- ops.cu: launchers (return the first CUDA error) --------------------------

@@ -1058,25 +1058,34 @@ namespace fl {
 // Each column runs as kTriSeg segments of m <= kTriM rows, one thread each;
 // the segment carries (factor R = r^m) are a linear-recurrence scan across
 // the 32 lanes of one warp per column.
-constexpr int kTriCols = 8;    // columns per CTA: 32-byte row pieces in FP32
+//
+// FP64 is bound by the FP64 pipe (1.7 operations per clock and SM): eight
+// operations per value, one exp2 per segment, and four columns per CTA, so
+// that a 2D plan of 512 columns has 128 CTAs (eight columns and twelve
+// operations with two exp2 per thread: 36.9 us at 511^2, now 15.8 us, both
+// between events).
+// FP32 is bound by the latency of its one load and store phase.
+template <typename T> constexpr int kTriCols = sizeof(T) == 8 ? 4 : 8;   // columns per CTA: 32-byte row pieces
 constexpr int kTriSeg = 32;    // segments per column (one warp lane each)
 constexpr int kTriM = 32;      // max rows per segment: n <= 1024
-constexpr int kTriTab = 4;     // table entries per column
+template <typename T> constexpr int kTriTab = sizeof(T) == 8 ? 5 : 4;   // table entries per column
 
 // Per-column constants, data-independent (FP64, once per shift and scale):
-// tab[4c] = r (rounded to T; every other entry is formed from this r),
-// tab[4c+1] = r^m, tab[4c+2] = log2(r), tab[4c+3] = K, with
-// gamma / (1 - r^2) = K w_0 (w_0 = r^{-1} x_0).
+// tab[0] = r (rounded to T; every other entry is formed from this r),
+// tab[1] = r^m, tab[2] = log2(r), tab[3] = K, with
+// gamma / (1 - r^2) = K w_0 (w_0 = r^{-1} x_0), and in FP64 tab[4] = r^e,
+// e = 2n + 2 - m S for the S = ceil(n/m) segments that hold rows.
 template <typename T>
 __global__ void k_tri_table(T* tab, const T* mu_col, const T* mu_outer, int ncols, int n_inner,
                             double shift, double scale, double cA, int n, int m, int diag) {
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= ncols) return;
   const double mu = (double)mu_col[c % n_inner] + (mu_outer ? (double)mu_outer[c / n_inner] : 0.0);
+  T* o = tab + kTriTab<T> * c;
   if (diag) {
     // no stencil along axis 0 (a 1D problem): z = t / (shift + scale mu)
-    tab[kTriTab * c + 0] = (T)(1.0 / (shift + scale * mu));
-    tab[kTriTab * c + 1] = tab[kTriTab * c + 2] = tab[kTriTab * c + 3] = (T)0;
+    o[0] = (T)(1.0 / (shift + scale * mu));
+    for (int i = 1; i < kTriTab<T>; ++i) o[i] = (T)0;
     return;
   }
   const double e = (shift + scale * mu) / (scale * cA);
@@ -1085,10 +1094,11 @@ __global__ void k_tri_table(T* tab, const T* mu_col, const T* mu_outer, int ncol
   const double lr = log1p(-(1.0 - r));
   const double omr2 = (1.0 - r) * (1.0 + r);
   const double v0 = (r - exp((2.0 * n + 1.0) * lr)) / omr2;
-  tab[kTriTab * c + 0] = rt;
-  tab[kTriTab * c + 1] = (T)exp((double)m * lr);
-  tab[kTriTab * c + 2] = (T)(lr * 1.4426950408889634073599246810018921);
-  tab[kTriTab * c + 3] = (T)(r * r / ((1.0 + r * v0) * omr2));
+  o[0] = rt;
+  o[1] = (T)exp((double)m * lr);
+  o[2] = (T)(lr * 1.4426950408889634073599246810018921);
+  o[3] = (T)(r * r / ((1.0 + r * v0) * omr2));
+  if constexpr (sizeof(T) == 8) o[4] = (T)exp((2.0 * n + 2.0 - (double)m * ((n + m - 1) / m)) * lr);
 }
 
 template <typename T>
@@ -1121,16 +1131,17 @@ __device__ __forceinline__ T lane_scan(T b, T R, bool up) {
   return b;
 }
 
-// TC columns per CTA of TC * kTriSeg threads (warp w scans column w).
-template <typename T, int TC = kTriCols>
-__device__ __forceinline__ void body_tri_cols(const TriArgs<T>& a, int bx) {
+// TC columns per CTA of TC * kTriSeg threads (warp w scans column w), up to M
+// rows per segment.  FP32.
+template <typename T, int TC, int M>
+__device__ __forceinline__ void body_tri_cols_f32(const TriArgs<T>& a, int bx) {
   __shared__ T s_e[kTriSeg][TC + 1];   // segment end values (forward, backward)
   __shared__ T s_c[kTriSeg][TC + 1];   // carries into each segment
   __shared__ T s_w0[TC];
   if (a.st && a.st->done) return;
   if (a.diag) {
     const int dc = bx * TC + (int)threadIdx.x;
-    if ((int)threadIdx.x < TC && dc < a.ncols) a.v[dc] *= a.tab[kTriTab * dc];
+    if ((int)threadIdx.x < TC && dc < a.ncols) a.v[dc] *= a.tab[kTriTab<T> * dc];
     return;
   }
   const int c = threadIdx.x % TC, s = threadIdx.x / TC;
@@ -1139,26 +1150,26 @@ __device__ __forceinline__ void body_tri_cols(const TriArgs<T>& a, int bx) {
   const int n = a.n, m = a.m, i0 = s * m;
   T* FL_RESTRICT vc = a.v + col;
   const size_t ld = (size_t)a.ncols;
-  T y[kTriM];
+  T y[M];
 #pragma unroll
-  for (int j = 0; j < kTriM; ++j)
+  for (int j = 0; j < M; ++j)
     y[j] = (act && j < m && i0 + j < n) ? vc[(size_t)(i0 + j) * ld] : (T)0;
   T r = (T)0, R = (T)0, l2r = (T)0, K = (T)0;
   if (act) {
-    r = a.tab[kTriTab * col];
-    R = a.tab[kTriTab * col + 1];
-    l2r = a.tab[kTriTab * col + 2];
-    K = a.tab[kTriTab * col + 3];
+    r = a.tab[kTriTab<T> * col];
+    R = a.tab[kTriTab<T> * col + 1];
+    l2r = a.tab[kTriTab<T> * col + 2];
+    K = a.tab[kTriTab<T> * col + 3];
   }
   // scan lanes: warp w scans column w, lane = segment
   const int wc = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int wcol = bx * TC + wc;
-  const T wR = wcol < a.ncols ? a.tab[kTriTab * wcol + 1] : (T)0;
+  const T wR = wcol < a.ncols ? a.tab[kTriTab<T> * wcol + 1] : (T)0;
   // forward recurrence within the segment
   {
     T acc = (T)0;
 #pragma unroll
-    for (int j = 0; j < kTriM; ++j)
+    for (int j = 0; j < M; ++j)
       if (j < m) {
         acc = y[j] + r * acc;
         y[j] = acc;
@@ -1176,7 +1187,7 @@ __device__ __forceinline__ void body_tri_cols(const TriArgs<T>& a, int bx) {
     const T cin = s_c[s][c];
     T pw = r;
 #pragma unroll
-    for (int j = 0; j < kTriM; ++j)
+    for (int j = 0; j < M; ++j)
       if (j < m) {
         y[j] = (i0 + j < n) ? y[j] + pw * cin : (T)0;
         pw *= r;
@@ -1186,7 +1197,7 @@ __device__ __forceinline__ void body_tri_cols(const TriArgs<T>& a, int bx) {
   {
     T acc = (T)0;
 #pragma unroll
-    for (int j = kTriM - 1; j >= 0; --j)
+    for (int j = M - 1; j >= 0; --j)
       if (j < m) {
         acc = y[j] + r * acc;
         y[j] = acc;
@@ -1208,7 +1219,7 @@ __device__ __forceinline__ void body_tri_cols(const TriArgs<T>& a, int bx) {
   {
     T p = tri_exp2(l2r * (T)(i0 + 1));
 #pragma unroll
-    for (int j = 0; j < kTriM; ++j)
+    for (int j = 0; j < M; ++j)
       if (j < m) {
         y[j] = r * y[j] - g * p;
         p *= r;
@@ -1219,7 +1230,7 @@ __device__ __forceinline__ void body_tri_cols(const TriArgs<T>& a, int bx) {
     T pw = r * r;
     T qv = tri_exp2(l2r * (T)(2 * n + 2 - i0 - m));
 #pragma unroll
-    for (int j = kTriM - 1; j >= 0; --j)
+    for (int j = M - 1; j >= 0; --j)
       if (j < m) {
         y[j] = (y[j] + pw * cin + g * qv) * inv_sc;
         pw *= r;
@@ -1227,14 +1238,141 @@ __device__ __forceinline__ void body_tri_cols(const TriArgs<T>& a, int bx) {
       }
   }
 #pragma unroll
-  for (int j = 0; j < kTriM; ++j)
+  for (int j = 0; j < M; ++j)
     if (j < m && i0 + j < n) vc[(size_t)(i0 + j) * ld] = y[j];
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kTriCols * kTriSeg) k_tri_cols(TriArgs<T> a) {
+// FP64: one exp2 per segment, eight operations per value.
+template <typename T, int TC, int M>
+__device__ __forceinline__ void body_tri_cols_f64(const TriArgs<T>& a, int bx) {
+  __shared__ T s_e[kTriSeg][TC + 1];   // segment end values (forward, backward)
+  __shared__ T s_c[kTriSeg][TC + 1];   // carries into each segment
+  __shared__ T s_p[kTriSeg][TC + 1];   // r^(m s)
+  __shared__ T s_w0[TC];
+  if (a.st && a.st->done) return;
+  if (a.diag) {
+    const int dc = bx * TC + (int)threadIdx.x;
+    if ((int)threadIdx.x < TC && dc < a.ncols) a.v[dc] *= a.tab[kTriTab<T> * dc];
+    return;
+  }
+  const int c = threadIdx.x % TC, s = threadIdx.x / TC;
+  const int col = bx * TC + c;
+  const bool act = col < a.ncols;
+  const int n = a.n, m = a.m, i0 = s * m;
+  T* FL_RESTRICT vc = a.v + col;
+  const size_t ld = (size_t)a.ncols;
+  T y[M];
+#pragma unroll
+  for (int j = 0; j < M; ++j)
+    y[j] = (act && j < m && i0 + j < n) ? vc[(size_t)(i0 + j) * ld] : (T)0;
+  T r = (T)0, K = (T)0, qe = (T)0;
+  if (act) {
+    r = a.tab[kTriTab<T> * col];
+    K = a.tab[kTriTab<T> * col + 3];
+    qe = a.tab[kTriTab<T> * col + 4];
+  }
+  // scan lanes: warp w scans column w, lane = segment
+  const int wc = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int wcol = bx * TC + wc;
+  const T wR = wcol < a.ncols ? a.tab[kTriTab<T> * wcol + 1] : (T)0;
+  // (log2 r is -infinity where r rounds to nothing beside 1)
+  s_p[lane][wc] = lane == 0 ? (T)1 : (wcol < a.ncols ? tri_exp2(a.tab[kTriTab<T> * wcol + 2] * (T)(lane * m)) : (T)0);
+  // forward recurrence within the segment
+  {
+    T acc = (T)0;
+#pragma unroll
+    for (int j = 0; j < M; ++j)
+      if (j < m) {
+        acc = y[j] + r * acc;
+        y[j] = acc;
+      }
+    s_e[s][c] = acc;
+  }
+  __syncthreads();
+  {
+    const T b = lane_scan(s_e[lane][wc], wR, true);
+    const T ex = __shfl_up_sync(0xffffffffu, b, 1);
+    s_c[lane][wc] = lane > 0 ? ex : (T)0;
+  }
+  __syncthreads();
+  {
+    T t = r * s_c[s][c];
+#pragma unroll
+    for (int j = 0; j < M; ++j)
+      if (j < m) {
+        y[j] = (i0 + j < n) ? y[j] + t : (T)0;
+        t *= r;
+      }
+  }
+  // backward recurrence within the segment
+  {
+    T acc = (T)0;
+#pragma unroll
+    for (int j = M - 1; j >= 0; --j)
+      if (j < m) {
+        acc = y[j] + r * acc;
+        y[j] = acc;
+      }
+    s_e[s][c] = acc;
+  }
+  __syncthreads();
+  {
+    const T b = lane_scan(s_e[lane][wc], wR, false);
+    const T ex = __shfl_down_sync(0xffffffffu, b, 1);
+    s_c[lane][wc] = lane < 31 ? ex : (T)0;
+    if (lane == 0) s_w0[wc] = b;   // w_0 of the column
+  }
+  __syncthreads();
+  if (!act || i0 >= n) return;
+  const T inv_sc = (T)a.inv_sc;
+  const T g = K * s_w0[c];
+  // z_i = (r w_i - g (r^{i+1} - r^{2n+1-i})) / (scale cA), w_i = w_local + r^{m-j} cin:
+  // one term falling like r^j and one like r^{m-1-j}
+  {
+    const T ri = r * inv_sc;
+    T t = -g * (r * s_p[s][c]) * inv_sc;
+#pragma unroll
+    for (int j = 0; j < M; ++j)
+      if (j < m) {
+        y[j] = ri * y[j] + t;
+        t *= r;
+      }
+  }
+  {
+    const int last = (n + m - 1) / m - 1;
+    T t = (r * r * s_c[s][c] + g * (qe * s_p[last - s][c])) * inv_sc;
+#pragma unroll
+    for (int j = M - 1; j >= 0; --j)
+      if (j < m) {
+        y[j] += t;
+        t *= r;
+      }
+  }
+#pragma unroll
+  for (int j = 0; j < M; ++j)
+    if (j < m && i0 + j < n) vc[(size_t)(i0 + j) * ld] = y[j];
+}
+
+// The body for m <= M rows per segment: with M = 32 throughout, a 3D plan of
+// 256^3 (m = 8) spent most of its instructions on rows that are not there
+// and held one CTA per SM (149 us, now 47 us).
+template <typename T, int TC, int M>
+__device__ __forceinline__ void body_tri_cols_m(const TriArgs<T>& a, int bx) {
+  if constexpr (sizeof(T) == 8) body_tri_cols_f64<T, TC, M>(a, bx);
+  else body_tri_cols_f32<T, TC, M>(a, bx);
+}
+
+template <typename T, int TC = kTriCols<T>>
+__device__ __forceinline__ void body_tri_cols(const TriArgs<T>& a, int bx) {
+  if (a.m <= 8) body_tri_cols_m<T, TC, 8>(a, bx);
+  else if (a.m <= 16) body_tri_cols_m<T, TC, 16>(a, bx);
+  else body_tri_cols_m<T, TC, kTriM>(a, bx);
+}
+
+template <typename T, int M>
+__global__ void __launch_bounds__(kTriCols<T> * kTriSeg) k_tri_cols(TriArgs<T> a) {
   pdl_wait();
-  body_tri_cols<T>(a, blockIdx.x);
+  body_tri_cols_m<T, kTriCols<T>, M>(a, blockIdx.x);
   pdl_release();
 }
 

@@ -568,7 +568,7 @@ PrecChain<T> build_precond(const Geo& g, const Tables<T>& tb, const PrecIO<T>& i
     a.n = g.n[0];
     a.ncols = (int)(g.N / g.n[0]);
     a.m = (g.n[0] + kTriSeg - 1) / kTriSeg;
-    const int tc = io.tri_cols > 0 ? io.tri_cols : kTriCols;
+    const int tc = io.tri_cols > 0 ? io.tri_cols : kTriCols<T>;
     ch.tri_blocks = (a.ncols + tc - 1) / tc;
   }
   if (d == 2) {
@@ -630,7 +630,8 @@ cudaError_t launch_precond(const Geo& g, const Tables<T>& tb, cudaStream_t s, co
   for (int j = 0; j <= ch.ncols; ++j) {
     if (j == ch.tri_after)
       FL_KERNEL((sizeof(T) == 4 ? "tri_cols" "<f32>" : "tri_cols" "<f64>"), s,
-                pdl_launch(k_tri_cols<T>, ch.tri_blocks, kTriCols * kTriSeg, 0, s, ch.tri));
+                const auto tri = ch.tri.m <= 8 ? k_tri_cols<T, 8> : ch.tri.m <= 16 ? k_tri_cols<T, 16> : k_tri_cols<T, kTriM>;
+                pdl_launch(tri, ch.tri_blocks, kTriCols<T> * kTriSeg, 0, s, ch.tri));
     if (j < ch.ncols)
       FL_KERNEL((sizeof(T) == 4 ? "dst_cols" "<f32>" : "dst_cols" "<f64>"), s,
                 FL_COLS_LAUNCH(k_dst_cols, T, 1 << ch.cols[j].lg, ch.cols_grid[j], ch.cols_smem[j], s,

@@ -1126,8 +1126,8 @@ fl_status fl_plan_create(int d, const int64_t* n, double h, double alpha, const 
   FL_TRY(dalloc(p, &p->t32.S, g.spec * sizeof(float2)));
   FL_TRY(dalloc(p, &p->t64.t, g.N * sizeof(double)));
   FL_TRY(dalloc(p, &p->t32.t, g.N * sizeof(float)));
-  FL_TRY(dalloc(p, &p->t64.tri_tab, (size_t)kTriTab * (g.N / g.n[0]) * sizeof(double)));
-  FL_TRY(dalloc(p, &p->t32.tri_tab, (size_t)kTriTab * (g.N / g.n[0]) * sizeof(float)));
+  FL_TRY(dalloc(p, &p->t64.tri_tab, (size_t)kTriTab<double> * (g.N / g.n[0]) * sizeof(double)));
+  FL_TRY(dalloc(p, &p->t32.tri_tab, (size_t)kTriTab<float> * (g.N / g.n[0]) * sizeof(float)));
   st = alloc_vecs(p, p->v32);
   if (st == FL_OK) st = alloc_vecs(p, p->v64);
   if (st != FL_OK) { free_plan(p); return st; }
