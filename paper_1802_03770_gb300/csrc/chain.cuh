@@ -249,9 +249,19 @@ void launch_rows_fwd_w8(const RowsFwdArgs<float>& a, int grid, size_t smem, cuda
 void launch_rows_inv_w8(const RowsInvArgs<float>& a, int grid, size_t smem, cudaStream_t s);
 void launch_dst_rows_w8(const DstRowsArgs<float>& a, int grid, size_t smem, cudaStream_t s);
 cudaError_t configure_rows_w8();
-// whether a plan's FP32 row passes on lines of L points take the 256 x 8 shape
-template <typename T> inline bool rows_w8(const Tables<T>& tb, int L) {
-  return sizeof(T) == 4 && tb.rshape == 1 && L >= 256 && L <= 2048;
+// Whether a plan's FP32 row pass of `ctas` CTAs on lines of L points takes
+// the 256 x 8 shape: where the plan asks for it, and by default where the
+// pass is a fraction of a wave, bound by one CTA's chain, which that shape
+// halves.  Larger grids are bound by instructions and keep 128 x 16.  Measured
+// in CUDA graphs, 128 x 16 -> 256 x 8: preconditioner 200^2 (50 CTAs) 23.8 ->
+// 14.6 us, 511^2 (256) 25.8 -> 21.9, 1000 x 500 (500) 27.7 -> 29.6, 600^2 (600)
+// 23.6 -> 26.8; apply 255^2 (32) 21.9 -> 19.5, 600^2 (300) 32.1 -> 29.7, 1024^2
+// (512) 35.8 -> 36.5; lines of 256 gain less (100^2 21.8 -> 21.1) and lose
+// from 250 CTAs on (40 x 100 x 100 59.0 -> 60.2).
+template <typename T> inline bool rows_w8(const Tables<T>& tb, int L, int ctas) {
+  if (sizeof(T) != 4 || L < 256 || L > 2048) return false;
+  if (tb.rshape == 1) return true;
+  return ctas <= (L >= 512 ? 304 : 152);
 }
 
 template <typename T>

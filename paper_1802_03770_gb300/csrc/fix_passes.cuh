@@ -344,7 +344,7 @@ __device__ __forceinline__ void fx_body_rows_fwd(const RowsFwdArgs<double>& a, i
   const int NL = (VPT * THREADS) >> lg;
   const int pair0 = bx * NL;
   const int npairs = (a.rows + 1) / 2;
-  const int nl = min(NL, npairs - pair0);
+  const int nl = NL == 1 ? 1 : min(NL, npairs - pair0);
   fx_zero<W>(s_mx);
   __syncthreads();
   const double beta = (a.pre == PRE_PUPDATE) ? a.st->beta : 0.0;
@@ -414,12 +414,12 @@ __device__ __forceinline__ void fx_body_rows_fwd(const RowsFwdArgs<double>& a, i
                                               FxStore{buf, ls, s_x}, true);
   __syncthreads();
   // k = 0 also writes k = L/2
+  const SpecRows spec(2 * pair0, a.rows_per_plane, a.plane_stride, a.H);
   for (int e = threadIdx.x; e < tot; e += THREADS) {
     const int q = e >> (lg - 1);
-    const int ra = 2 * (pair0 + q), rb = ra + 1;
-    const bool hb = rb < a.rows;
-    double2* Sa = a.S + ((size_t)(ra / a.rows_per_plane) * a.plane_stride + ra % a.rows_per_plane) * a.H;
-    double2* Sb = a.S + ((size_t)(rb / a.rows_per_plane) * a.plane_stride + rb % a.rows_per_plane) * a.H;
+    const bool hb = 2 * (pair0 + q) + 1 < a.rows;
+    double2* Sa = a.S + spec(2 * q);
+    double2* Sb = a.S + spec(2 * q + 1);
     const SBuf<Fx> lb = buf.at(q * ls);
     const int X = s_x[q];
     for (int k = e & (hL - 1); k <= hL; k += hL) {
@@ -535,13 +535,11 @@ __device__ __forceinline__ void fx_body_rows_inv(const RowsInvArgs<double>& a, i
   const int NL = (VPT * THREADS) >> lg;
   const int pair0 = bx * NL;
   const int npairs = (a.rows + 1) / 2;
-  const int nl = min(NL, npairs - pair0);
+  const int nl = NL == 1 ? 1 : min(NL, npairs - pair0);
   fx_zero<W>(s_mx);
   fx_zero<W>(s_key);
   __syncthreads();
-  auto spec_row = [&](int row) -> const double2* {
-    return a.S + ((size_t)(row / a.rows_per_plane) * a.plane_stride + row % a.rows_per_plane) * a.H;
-  };
+  const SpecRows spec(2 * pair0, a.rows_per_plane, a.plane_stride, a.H);
   // Staged as they are: xa[k] at k and xb[k] at L - k for 0 < k < L/2; at
   // k = 0 and L/2 the sum xa + i xb itself (both by the thread of k = 0).
   const int tot = nl * hL;
@@ -551,11 +549,11 @@ __device__ __forceinline__ void fx_body_rows_inv(const RowsInvArgs<double>& a, i
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int e = e0 + u * THREADS;
-      const int ra = 2 * (pair0 + (e >> (lg - 1))), k = e & (hL - 1);
+      const int dr = 2 * (e >> (lg - 1)), k = e & (hL - 1);
       va[u] = vb[u] = make_double2(0.0, 0.0);
       if (e < tot) {
-        va[u] = spec_row(ra)[k];
-        if (ra + 1 < a.rows) vb[u] = spec_row(ra + 1)[k];
+        va[u] = a.S[spec(dr) + k];
+        if (2 * pair0 + dr + 1 < a.rows) vb[u] = a.S[spec(dr + 1) + k];
       }
     }
 #pragma unroll
@@ -567,9 +565,8 @@ __device__ __forceinline__ void fx_body_rows_inv(const RowsInvArgs<double>& a, i
         const SBuf<Fx> lb = buf.at(q * ls);
         double2 xa = va[u], xb = vb[u];
         if (k == 0) {
-          const int ra = 2 * (pair0 + q);
-          const double2 ya = spec_row(ra)[hL];
-          const double2 yb = ra + 1 < a.rows ? spec_row(ra + 1)[hL] : make_double2(0.0, 0.0);
+          const double2 ya = a.S[spec(2 * q) + hL];
+          const double2 yb = 2 * (pair0 + q) + 1 < a.rows ? a.S[spec(2 * q + 1) + hL] : make_double2(0.0, 0.0);
           xa = make_double2(xa.x - xb.y, xa.y + xb.x);
           xb = make_double2(ya.x - yb.y, ya.y + yb.x);
         }

@@ -116,14 +116,13 @@ __device__ __forceinline__ double cta_sum_partials(const double* FL_RESTRICT par
 // Minimum resident CTAs per SM asked of the compiler for a pass kernel of
 // THREADS threads.  The passes are latency-bound: the 128-thread FP32 row
 // passes keep at least 7 CTAs (28 warps) per SM (<= 73 registers), the
-// 256- and 512-thread passes at least 2 CTAs.
+// 256-thread ones 4 (64 registers), the 512-thread passes 2.
 // The wide instantiations for the longest lines (LGLO > 4: one line of 4096
 // or 8192 points per CTA) ask for one CTA only, so that the compiler keeps
 // the row bodies' registers.
-// FP64 passes: four CTAs of 256 threads or two of 512 (64 registers).
 template <typename T = float>
 constexpr int min_ctas(int threads, int lglo = 4) {
-  return lglo > 4 ? 1 : (threads <= 128 ? FL_ROW_MIN_CTAS : (sizeof(T) == 8 && threads == 256 ? 4 : 2));
+  return lglo > 4 ? 1 : (threads <= 128 ? FL_ROW_MIN_CTAS : (threads == 256 ? 4 : 2));
 }
 
 // Column tiles: at most 2^kMaxLtx columns; a CTA of THREADS x VPT values
@@ -187,10 +186,10 @@ __device__ __forceinline__ double cta_sum_ff(float hi, float lo, double* red) {
 
 // Per-thread accumulator of a CG dot product.  GB300 issues FP64 at a small
 // fraction of the FP32 rate, so the FP32 passes keep FP64 off the per-element
-// path: products and runs of up to 16 terms are summed in FP32, each run is
-// added into a float-float (two-sum) total, the warp tree is float-float
-// and the sums across warps and CTAs are FP64.  FP64 passes accumulate in
-// FP64 throughout.
+// path: the FP32 products are added into a float-float (two-sum) total, the
+// warp tree is float-float and the sums across warps and CTAs are FP64.  The
+// sum of the products is then exact to ~2^-46 however a launch shape groups
+// them.  FP64 passes accumulate in FP64 throughout.
 template <typename T>
 struct DotAcc {
   double acc = 0.0;
@@ -200,23 +199,13 @@ struct DotAcc {
 };
 template <>
 struct DotAcc<float> {
-  float hi = 0.f, lo = 0.f, run = 0.f;
-  int cnt = 0;
+  float hi = 0.f, lo = 0.f;
   __device__ __forceinline__ void add(float v) {
-    run += v;
-    if (++cnt == 16) flush();
-  }
-  __device__ __forceinline__ void flush() {
     float e;
-    hi = two_sum(hi, run, e);
+    hi = two_sum(hi, v, e);
     lo = __fadd_rn(lo, e);
-    run = 0.f;
-    cnt = 0;
   }
-  __device__ __forceinline__ double cta_total(double* red) {
-    flush();
-    return cta_sum_ff(hi, lo, red);
-  }
+  __device__ __forceinline__ double cta_total(double* red) const { return cta_sum_ff(hi, lo, red); }
 };
 
 // Every CTA of a pass calls this once, after its partial is stored; it
@@ -261,6 +250,22 @@ __device__ __forceinline__ void pcg_step(PcgState* st, double rr, double rz) {
   }
 }
 
+// Spectrum rows of a CTA's field rows row0, row0 + 1, ...: one division per
+// CTA instead of one per element.
+struct SpecRows {
+  int plane, rem, rpp, ps, H;
+  __device__ __forceinline__ SpecRows(int row0, int rows_per_plane, int plane_stride, int h)
+      : plane(row0 / rows_per_plane), rem(row0 % rows_per_plane), rpp(rows_per_plane), ps(plane_stride), H(h) {}
+  __device__ __forceinline__ size_t operator()(int dr) const {
+    int p = plane, r = rem + dr;
+    while (r >= rpp) {
+      r -= rpp;
+      ++p;
+    }
+    return ((size_t)p * ps + r) * H;
+  }
+};
+
 // ---------------------------------------------------------------------------
 // Operator pass 1: masked real-to-complex FFT along the last axis.
 // Two real rows ra, rb are packed as ra + i rb, zero-padded to L and
@@ -293,7 +298,7 @@ __device__ __forceinline__ void body_rows_fwd_at(const RowsFwdArgs<T>& a, int bx
   const int NL = (VPT * THREADS) / L;       // complex lines (row pairs) per CTA
   const int pair0 = bx * NL;
   const int npairs = (a.rows + 1) / 2;
-  const int nl = min(NL, npairs - pair0);
+  const int nl = NL == 1 ? 1 : min(NL, npairs - pair0);
   const T beta = (a.pre == PRE_PUPDATE) ? (T)a.st->beta : (T)0;
   // loads first (U elements per thread in flight), then the stores.  Only
   // the lower half of each line is written (n <= L/2); the transform's first
@@ -359,22 +364,21 @@ __device__ __forceinline__ void body_rows_fwd_at(const RowsFwdArgs<T>& a, int bx
                                                        true, st, true);
   }
   __syncthreads();
-  for (int q = 0; q < nl; ++q) {
-    const int ra = 2 * (pair0 + q), rb = ra + 1;
-    const bool hb = rb < a.rows;
-    typename Cplx<T>::type* FL_RESTRICT Sa =
-        a.S + ((size_t)(ra / a.rows_per_plane) * a.plane_stride + ra % a.rows_per_plane) * a.H;
-    typename Cplx<T>::type* FL_RESTRICT Sb =
-        hb ? a.S + ((size_t)(rb / a.rows_per_plane) * a.plane_stride + rb % a.rows_per_plane) * a.H
-           : nullptr;
+  // all lines of the CTA in one index space (a loop over lines cost a CTA of
+  // 16 lines of 128 points 2900 instructions per warp, most of them idle
+  // lanes' loop overhead); k = L/2 afterwards
+  const SpecRows spec(2 * pair0, a.rows_per_plane, a.plane_stride, a.H);
+  auto put = [&](int q, int k) {
     const SBuf<C> lb = buf.at(q * ls);
-    for (int k = threadIdx.x; k < a.H; k += THREADS) {
-      const C z = lb[k];
-      const C w = cconj(lb[(L - k) & (L - 1)]);
-      Sa[k] = cmake<C>((z.x + w.x) * (T)0.5, (z.y + w.y) * (T)0.5);
-      if (hb) Sb[k] = cmake<C>((z.y - w.y) * (T)0.5, (w.x - z.x) * (T)0.5);
-    }
-  }
+    const C z = lb[k];
+    const C w = cconj(lb[(L - k) & (L - 1)]);
+    a.S[spec(2 * q) + k] = cmake<C>((z.x + w.x) * (T)0.5, (z.y + w.y) * (T)0.5);
+    if (2 * (pair0 + q) + 1 < a.rows)
+      a.S[spec(2 * q + 1) + k] = cmake<C>((z.y - w.y) * (T)0.5, (w.x - z.x) * (T)0.5);
+  };
+#pragma unroll 4
+  for (int e = threadIdx.x; e < tot; e += THREADS) put(e >> (lg - 1), e & (hL - 1));
+  for (int q = threadIdx.x; q < nl; q += THREADS) put(q, hL);
 }
 
 // body_rows_fwd with the line length 2^LG .. 2^LGHI as a compile-time
@@ -605,52 +609,41 @@ __device__ __forceinline__ void body_rows_inv_at(const RowsInvArgs<T>& a, int bx
   const int NL = (VPT * THREADS) / L;
   const int pair0 = bx * NL;
   const int npairs = (a.rows + 1) / 2;
-  const int nl = min(NL, npairs - pair0);
+  const int nl = NL == 1 ? 1 : min(NL, npairs - pair0);
   // Z[k] = Xa[k] + i Xb[k];  Z[L-k] = conj(Xa[k]) + i conj(Xb[k]) for the
   // row pair (ra, rb) = (2p, 2p + 1) of line q
-  auto spec_row = [&](int row) -> const C* {
-    return a.S + ((size_t)(row / a.rows_per_plane) * a.plane_stride + row % a.rows_per_plane) * a.H;
-  };
+  const SpecRows spec(2 * pair0, a.rows_per_plane, a.plane_stride, a.H);
   auto put = [&](int q, int k, C xa, C xb) {
     const SBuf<C> lb = buf.at(q * ls);
     lb[k] = cmake<C>(xa.x - xb.y, xa.y + xb.x);
     if (k > 0 && k < a.H - 1) lb[L - k] = cmake<C>(xa.x + xb.y, xb.x - xa.y);
   };
-  constexpr int QB = 4;
-  if (NL >= QB) {
-    // several row pairs per CTA (short lines): the pairs' loads of one
-    // column range are issued together, one round trip per THREADS
-    // columns instead of one per pair
-    for (int q0 = 0; q0 < nl; q0 += QB) {
-      const C* Sa[QB];
-      const C* Sb[QB];
+  // all lines of the CTA in one index space, U spectrum pairs in flight per
+  // thread; k = L/2 afterwards
+  const int hL = L >> 1;
+  const int tot = nl * hL;
+  constexpr int U = 4;
+  for (int e0 = threadIdx.x; e0 < tot; e0 += THREADS * U) {
+    C xa[U], xb[U];
 #pragma unroll
-      for (int qq = 0; qq < QB; ++qq) {
-        const int ra = 2 * (pair0 + q0 + qq);
-        Sa[qq] = spec_row(ra);
-        Sb[qq] = (q0 + qq < nl && ra + 1 < a.rows) ? spec_row(ra + 1) : nullptr;
-      }
-      for (int k = threadIdx.x; k < a.H; k += THREADS) {
-        C xa[QB], xb[QB];
-#pragma unroll
-        for (int qq = 0; qq < QB; ++qq) {
-          xa[qq] = q0 + qq < nl ? Sa[qq][k] : cmake<C>((T)0, (T)0);
-          xb[qq] = Sb[qq] ? Sb[qq][k] : cmake<C>((T)0, (T)0);
-        }
-#pragma unroll
-        for (int qq = 0; qq < QB; ++qq)
-          if (q0 + qq < nl) put(q0 + qq, k, xa[qq], xb[qq]);
+    for (int u = 0; u < U; ++u) {
+      const int e = e0 + u * THREADS;
+      const int dr = 2 * (e >> (lg - 1)), k = e & (hL - 1);
+      xa[u] = xb[u] = cmake<C>((T)0, (T)0);
+      if (e < tot) {
+        xa[u] = a.S[spec(dr) + k];
+        if (2 * pair0 + dr + 1 < a.rows) xb[u] = a.S[spec(dr + 1) + k];
       }
     }
-  } else {
-    for (int q = 0; q < nl; ++q) {
-      const int ra = 2 * (pair0 + q);
-      const C* FL_RESTRICT Sa = spec_row(ra);
-      const C* FL_RESTRICT Sb = ra + 1 < a.rows ? spec_row(ra + 1) : nullptr;
-#pragma unroll 4
-      for (int k = threadIdx.x; k < a.H; k += THREADS)
-        put(q, k, Sa[k], Sb ? Sb[k] : cmake<C>((T)0, (T)0));
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int e = e0 + u * THREADS;
+      if (e < tot) put(e >> (lg - 1), e & (hL - 1), xa[u], xb[u]);
     }
+  }
+  for (int q = threadIdx.x; q < nl; q += THREADS) {
+    const bool hb = 2 * (pair0 + q) + 1 < a.rows;
+    put(q, hL, a.S[spec(2 * q) + hL], hb ? a.S[spec(2 * q + 1) + hL] : cmake<C>((T)0, (T)0));
   }
   __syncthreads();
   fft_smem<VPT, false, LGHI, LGLO>(buf, lg, ls, 0, nl, a.tw, a.lgmax, true);
@@ -661,22 +654,23 @@ __device__ __forceinline__ void body_rows_inv_at(const RowsInvArgs<T>& a, int bx
   T* FL_RESTRICT out = a.out;
   float* FL_RESTRICT out32 = a.out32;
   const T cm = (T)a.cm, cx = (T)a.cx, cb = (T)a.cb;
-  for (int q = 0; q < 2 * nl; ++q) {
-    const int row = 2 * pair0 + q;
-    if (row >= a.rows) break;
-    const int half = q & 1;
-    const SBuf<C> lb = buf.at((q >> 1) * ls);
-    const size_t base = (size_t)row * a.n;
-#pragma unroll 4
-    for (int j = threadIdx.x; j < a.n; j += THREADS) {
-      const size_t idx = base + j;
-      const C z = lb[j];
-      const T mx = (a.mask && !a.mask[idx]) ? (T)0 : (half ? z.y : z.x);
+#pragma unroll 2
+  for (int e = threadIdx.x; e < tot; e += THREADS) {
+    const int q = e >> (lg - 1), j = e & (hL - 1);
+    if (j >= a.n) continue;
+    const int row = 2 * (pair0 + q);
+    const C z = buf[q * ls + j];
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      if (half && row + 1 >= a.rows) break;
+      const size_t idx = ((size_t)row + half) * a.n + j;
+      const bool off = a.mask && !a.mask[idx];
+      const T mx = off ? (T)0 : (half ? z.y : z.x);
       if (a.outm) a.outm[idx] = mx;
       T v = mx * cm;
       if (xin) v += cx * xin[idx];
       if (bin) v += cb * bin[idx];
-      if (a.mask && !a.mask[idx]) v = (T)0;
+      if (off) v = (T)0;
       if (out) out[idx] = v;
       if (out32) out32[idx] = (float)v;
       if (a.partials) part.add(win ? v * win[idx] : v * v);

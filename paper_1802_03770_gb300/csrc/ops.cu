@@ -501,7 +501,7 @@ cudaError_t launch_apply(const Geo& g, const Tables<T>& tb, cudaStream_t s, cons
   const int Lx = g.L[g.d - 1];
   FL_KERNEL((sizeof(T) == 4 ? "rows_fwd" "<f32>" : "rows_fwd" "<f64>"), s,
             if constexpr (sizeof(T) == 4) {
-              if (rows_w8(tb, Lx)) launch_rows_fwd_w8(ch.fwd, ch.row_blocks, ch.row_smem, s);
+              if (rows_w8(tb, Lx, ch.row_blocks)) launch_rows_fwd_w8(ch.fwd, ch.row_blocks, ch.row_smem, s);
               else FL_ROWS_LAUNCH(k_rows_fwd, T, Lx, ch.row_blocks, ch.row_smem, s, ch.fwd);
             } else {
               FL_ROWS_LAUNCH(k_rows_fwd, T, Lx, ch.row_blocks, ch.row_smem, s, ch.fwd);
@@ -514,7 +514,7 @@ cudaError_t launch_apply(const Geo& g, const Tables<T>& tb, cudaStream_t s, cons
                              ch.cols[j]));
   FL_KERNEL((sizeof(T) == 4 ? "rows_inv" "<f32>" : "rows_inv" "<f64>"), s,
             if constexpr (sizeof(T) == 4) {
-              if (rows_w8(tb, Lx)) launch_rows_inv_w8(ch.inv, ch.row_blocks, ch.row_smem, s);
+              if (rows_w8(tb, Lx, ch.row_blocks)) launch_rows_inv_w8(ch.inv, ch.row_blocks, ch.row_smem, s);
               else FL_ROWS_LAUNCH(k_rows_inv, T, Lx, ch.row_blocks, ch.row_smem, s, ch.inv);
             } else {
               FL_ROWS_LAUNCH(k_rows_inv, T, Lx, ch.row_blocks, ch.row_smem, s, ch.inv);
@@ -622,7 +622,7 @@ cudaError_t launch_precond(const Geo& g, const Tables<T>& tb, cudaStream_t s, co
   const int Lx = g.L[g.d - 1];
   FL_KERNEL((sizeof(T) == 4 ? "dst_rows" "<f32>" : "dst_rows" "<f64>"), s,
             if constexpr (sizeof(T) == 4) {
-              if (rows_w8(tb, Lx)) launch_dst_rows_w8(ch.first, ch.row_blocks, ch.row_smem, s);
+              if (rows_w8(tb, Lx, ch.row_blocks)) launch_dst_rows_w8(ch.first, ch.row_blocks, ch.row_smem, s);
               else FL_ROWS_LAUNCH(k_dst_rows, T, Lx, ch.row_blocks, ch.row_smem, s, ch.first);
             } else {
               FL_ROWS_LAUNCH(k_dst_rows, T, Lx, ch.row_blocks, ch.row_smem, s, ch.first);
@@ -639,7 +639,7 @@ cudaError_t launch_precond(const Geo& g, const Tables<T>& tb, cudaStream_t s, co
   }
   FL_KERNEL((sizeof(T) == 4 ? "dst_rows" "<f32>" : "dst_rows" "<f64>"), s,
             if constexpr (sizeof(T) == 4) {
-              if (rows_w8(tb, Lx)) launch_dst_rows_w8(ch.last, ch.row_blocks, ch.row_smem, s);
+              if (rows_w8(tb, Lx, ch.row_blocks)) launch_dst_rows_w8(ch.last, ch.row_blocks, ch.row_smem, s);
               else FL_ROWS_LAUNCH(k_dst_rows, T, Lx, ch.row_blocks, ch.row_smem, s, ch.last);
             } else {
               FL_ROWS_LAUNCH(k_dst_rows, T, Lx, ch.row_blocks, ch.row_smem, s, ch.last);

@@ -1722,7 +1722,7 @@ fl_status solve_batched_mixed(fl_plan* const* plans, int count, const double* co
   // tuned (or set) row shape is that one (fl_plan_set_row_shape)
   if (!persist) {
     bool w8 = true;
-    for (int i = 0; i < count && w8; ++i) w8 = rows_w8(plans[i]->t32, plans[i]->g.L[plans[i]->g.d - 1]);
+    for (int i = 0; i < count && w8; ++i) w8 = plans[i]->t32.rshape == 1;
     if (w8) {
       for (BatchPass* bp : {&A32.fwd, &A32.inv, &PI.first, &PI.last, &PS.first, &PS.last}) bp->w8 = 1;
     }

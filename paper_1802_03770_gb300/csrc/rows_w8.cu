@@ -2,10 +2,11 @@
 // instead of 128 x 16 (the same lines per CTA, so the same grids, shared
 // memory and partial-sum counts), radix-8 stages instead of radix-16.  Half
 // the values per thread shortens each CTA's dependent chain, which pays on
-// grids of few rows (a pass over 64 rows of 2048 points: 14.5 -> 12.3 us)
-// and costs on many (1024 rows: 18.9 -> 27.4 us); fl_plan_autotune times
-// both shapes per plan and keeps the faster.  Compiled apart from ops.cu so
-// that the two build in parallel.
+// grids of up to two CTAs per SM and costs on larger ones; rows_w8 (chain.cuh)
+// holds the rule and its measurements, fl_plan_autotune times both shapes per
+// plan and may ask for this one throughout.  64 registers, four CTAs per SM
+// (at two it cost twice as much on full grids).  Compiled apart from ops.cu
+// so that the two build in parallel.
 #include "chain.cuh"
 
 namespace fl {
