@@ -244,7 +244,7 @@ class Plan:
 
     def set_tiles(self, tx):
         """Column-tile widths of the strided passes: six ints (FP32 axes 0..2,
-        FP64 axes 0..2; 0 = the widest tile)."""
+        FP64 axes 0..2; 0 = the default)."""
         arr = (ctypes.c_int * 6)(*[int(v) for v in tx])
         L.check(self._lib.fl_plan_set_tiles(self._h, arr), "fl_plan_set_tiles")
 

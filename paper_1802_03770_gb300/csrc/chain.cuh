@@ -93,10 +93,22 @@ template <typename T> inline int col_tx(int L) {
 template <typename T> inline int min_tx() {
   return std::max(1, 16 / (int)sizeof(typename Cplx<T>::type));
 }
+// Default column-tile width of a strided pass along `axis`: the widest tile
+// that fits the CTA; in FP32 3D passes half of it (CTAs of 256 threads, twice
+// as many resident, whose loads and transforms overlap) where a tile keeps 64
+// contiguous bytes per line element and the spectrum stays in L2.  Measured,
+// widest -> half: apply 64^3 37.5 -> 34.0 us, 96 x 135 x 75 114 -> 109, 128^3
+// (33 MB) 76 -> 68; 256^3 (270 MB, streamed) 734 -> 760; 2D 511^2 22.3 -> 23.0,
+// 1024^2 33.0 -> 40.4.
+template <typename T> inline int default_tx(const Geo& g, int axis) {
+  const int L = g.L[axis], widest = col_tx<T>(L);
+  const bool in_l2 = g.spec * (long long)sizeof(float2) <= 96ll << 20;
+  return sizeof(T) == 4 && g.d == 3 && widest >= 16 && in_l2 ? widest / 2 : widest;
+}
 // column-tile width of a strided pass along `axis`: the plan's tuned width
-// if set, else the widest tile that fits the CTA
-template <typename T> inline int plan_tx(const Tables<T>& tb, int axis, int L) {
-  return tb.tx[axis] > 0 ? tb.tx[axis] : col_tx<T>(L);
+// if set, else the default
+template <typename T> inline int plan_tx(const Geo& g, const Tables<T>& tb, int axis) {
+  return tb.tx[axis] > 0 ? tb.tx[axis] : default_tx<T>(g, axis);
 }
 // a column-tile width tx narrowed to what a CTA of ct threads holds (ct = 0:
 // tx unchanged)
@@ -112,20 +124,21 @@ template <typename T> inline size_t smem_bytes(int lines, int L) {
 template <typename T> inline size_t tile_bytes(int tx, int L) {
   return (size_t)sbuf_elems((long long)tx * L) * sizeof(typename Cplx<T>::type);
 }
-// shared-memory bytes of a strided pass: the FFT tile, then (FP32) the
-// line length's twiddle table
-template <typename T> inline size_t cols_bytes(int tx, int L) {
-  return tile_bytes<T>(tx, L) + (sizeof(T) == 4 ? (size_t)L * sizeof(typename Cplx<T>::type) : 0);
-}
-// ... and for a convolution pass, then the symbol's rows 0..L/2 for the
-// tile's columns
-template <typename T> inline size_t conv_tile_bytes(int tx, int L) {
-  return cols_bytes<T>(tx, L) + (size_t)(L / 2 + 1) * tx * sizeof(T);
-}
 inline int ilog2i(int v) {
   int l = 0;
   while ((1 << l) < v) ++l;
   return l;
+}
+// shared-memory bytes of a strided pass: the FFT tile, then (FP32) the
+// stages' twiddle tables
+template <typename T> inline size_t cols_bytes(int tx, int L) {
+  return tile_bytes<T>(tx, L) + (sizeof(T) == 4 ? (size_t)place_table_len(ilog2i(L)) * sizeof(typename Cplx<T>::type) : 0);
+}
+// ... and for a convolution pass, then the symbol's rows 0..L/2 for the
+// tile's columns (FP32: with a pad row after every 16)
+template <typename T> inline size_t conv_tile_bytes(int tx, int L) {
+  const int rows = L / 2 + 1 + (sizeof(T) == 4 ? L / 32 : 0);
+  return cols_bytes<T>(tx, L) + (size_t)rows * tx * sizeof(T);
 }
 
 // One operator apply: the row pass, one (2D) or three (3D) strided passes

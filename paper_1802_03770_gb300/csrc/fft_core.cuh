@@ -43,6 +43,16 @@ template <typename T> struct Cplx;
 template <> struct Cplx<float> { typedef float2 type; };
 template <> struct Cplx<double> { typedef double2 type; };
 
+// Asynchronous global -> shared copies of 4, 8 or 16 bytes (no registers
+// held while in flight); cp_async_wait_all() waits for the calling thread's
+// own copies, a barrier then makes them visible to the CTA.
+template <int BYTES>
+__device__ __forceinline__ void cp_async(void* smem, const void* gmem) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(sa), "l"(gmem), "n"(BYTES) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // Complex buffer in shared memory with one pad element after every 16: the
 // logical index i is stored at i + i/16.  The first Stockham stage writes the
 // R legs of a butterfly to R consecutive logical places (a stride of R
@@ -74,6 +84,7 @@ template <> __device__ __forceinline__ float2 csub<float2>(float2 a, float2 b) {
 template <typename C> __device__ __forceinline__ C cmul(C a, C b) {
   return cmake<C>(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
+template <typename C> __device__ __forceinline__ C cswap(C a) { return cmake<C>(a.y, a.x); }
 template <typename C> __device__ __forceinline__ C cconj(C a) { return cmake<C>(a.x, -a.y); }
 template <typename C, typename T> __device__ __forceinline__ C cscale(C a, T s) { return cmake<C>(a.x * s, a.y * s); }
 // multiply by -i (forward) or +i (inverse)
@@ -431,5 +442,231 @@ __device__ __forceinline__ void fft_smem(SBuf<C> buf, int lg, int ls, int ltx, i
   fft_io<VPT, IL, false, LGHI, LGLO, TWT>(buf, lg, ls, ltx, nlines, tw, lgmax, inv, ld, true, st, true);
   __syncthreads();
 }
+
+// ---------------------------------------------------------------------------
+// In-place transforms with the frequencies in digit-reversed places: decimation
+// in frequency forward, its mirror image back.  A stage reads and writes the
+// same places of its own thread, so one barrier separates two stages (the
+// autosort stages need two).  A convolution never needs natural order: the
+// last forward stage, the product and the first inverse stage share their
+// values in registers, the first forward stage takes its legs from load and
+// the last inverse stage hands its outputs on, so that S stages each way take
+// 2 (S - 1) trips through shared memory and as many barriers instead of 2 S
+// (and the staging of the input) and 4 S.
+//
+// Stage s has radix R_s on blocks of B_s = L / (R_0 .. R_{s-1}) places,
+// M_s = B_s / R_s: butterfly (block, j) has its legs at block B_s + j + r M_s;
+// output d is multiplied by exp(-2 pi i j d / B_s) and stored at leg d.  The
+// place (d_0, d_1, ..) = d_0 B_1 + d_1 B_2 + .. then holds the frequency
+// d_0 + R_0 d_1 + R_0 R_1 d_2 + ...  The inverse is run on swapped values
+// with the same twiddles, multiplied before the butterfly.
+
+// Frequency at place p of a line of 2^lg with the stage plan of `vpt` values
+// per thread (FftPlan), and the log2 of its radices.
+__host__ __device__ __forceinline__ int plan_lg_radix(int lg, int vpt, int s) {
+  const int n16 = vpt >= 16 ? (lg % 4 == 1 && lg >= 5 ? lg / 4 - 1 : lg / 4) : 0;
+  const int n8 = (lg - 4 * n16) / 3;
+  return s < n16 ? 4 : (s < n16 + n8 ? 3 : lg - 4 * n16 - 3 * n8);
+}
+__host__ __device__ __forceinline__ int place_frequency(int p, int lg, int vpt) {
+  int k = 0, lgb = lg, lgk = 0;
+  for (int s = 0; lgb > 0; ++s) {
+    const int lr = plan_lg_radix(lg, vpt, s);
+    lgb -= lr;
+    k += (p >> lgb) << lgk;
+    p &= (1 << lgb) - 1;
+    lgk += lr;
+  }
+  return k;
+}
+
+template <int V> struct IntC { static constexpr int v = V; };
+
+// Twiddles of stage ST at offset j: exp(-2 pi i j r / B), B its block length.
+// TWT: from a table per stage in shared memory, one after another (stage s:
+// B_s entries; read at a stride of 16 places, the table of the whole line had
+// eight-way bank conflicts), place_table_len entries in all.
+__host__ __device__ __forceinline__ int place_table_len(int lg) { return (1 << lg) + (1 << lg) / 4; }
+// entry m of the concatenated tables as a power of exp(-2 pi i / 2^lg), below 2^lg
+inline int place_table_power(int m, int lg, int vpt) {
+  int lgb = lg;
+  for (int s = 0; m >= (1 << lgb) && lgb > 0; ++s) {
+    m -= 1 << lgb;
+    lgb -= plan_lg_radix(lg, vpt, s);
+  }
+  return lgb > 0 ? m << (lg - lgb) : 0;   // (the rest of the table is not read)
+}
+template <int LG, int VPT>
+__host__ __device__ constexpr int place_table_at(int st) {
+  int at = 0, lgb = LG;
+  for (int s = 0; s < st; ++s) {
+    at += 1 << lgb;
+    lgb -= clog2(FftPlan<LG, VPT>::radix(s));
+  }
+  return at;
+}
+template <int R, bool TWT, int LG, int VPT, int ST, typename C>
+__device__ __forceinline__ void place_twiddles(const C* FL_RESTRICT tw, int j, int lgmax, C* w) {
+  constexpr int LGB = LG - clog2(FftPlan<LG, VPT>::ns(ST));
+  if constexpr (TWT) twiddles<R, true>(tw + place_table_at<LG, VPT>(ST), j, false, w, LGB);
+  else twiddles<R, false>(tw, j << (lgmax - LGB), false, w, lgmax);
+}
+
+enum { PLACE_FWD = 0, PLACE_INV = 1, PLACE_CONV = 2 };
+// What a stage does with its values: forward or inverse butterfly, legs from
+// load (IN) or the buffer, outputs to out (OUT) or the buffer; CONV is the
+// middle stage of a convolution (forward, product, inverse).
+template <int LG, int VPT, bool IL, bool HALF, bool HOUT, bool TWT, int ST, int KIND, bool IN, bool OUT, typename C,
+          typename Load, typename Mid, typename Out>
+__device__ __forceinline__ void place_stage(SBuf<C> buf, int ls, int ltx, int nlines, const C* FL_RESTRICT tw,
+                                            int lgmax, Load& load, Mid& mid, Out& out) {
+  typedef FftPlan<LG, VPT> P;
+  constexpr int R = P::radix(ST);
+  constexpr int LR = LogR<R>::v;
+  constexpr int NB = VPT / R;
+  constexpr int LGB = LG - clog2(P::ns(ST));   // log2 of the block length
+  constexpr int LGM = LGB - LR;
+  constexpr int LGQ = LG - LR;                 // log2 of the butterflies of a line
+  const int total = IL ? ((1 << LGQ) << ltx) : (nlines << LGQ);
+  const int S = IL ? ((1 << LGM) << ltx) : (1 << LGM);   // logical leg stride
+  // the middle product or the first twiddles may read what the pass copied to
+  // shared memory: legs first, then the copies' barrier
+  constexpr bool WAIT = IN && (KIND == PLACE_CONV || (KIND == PLACE_FWD && TWT && LGM > 0));
+  C v[NB][R];
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    const int g = threadIdx.x + b * blockDim.x;
+    if (g < total) {
+      const int line = IL ? (g & ((1 << ltx) - 1)) : (g >> LGQ);
+      const int q = IL ? (g >> ltx) : (g & ((1 << LGQ) - 1));
+      const int pos = ((q >> LGM) << LGB) + (q & ((1 << LGM) - 1));
+      if (IN) {
+        load(line, pos, IntC<LGM>(), IntC<(HALF ? R / 2 : R)>(), v[b]);
+        if (HALF) {
+#pragma unroll
+          for (int r = R / 2; r < R; ++r) v[b][r] = cmake<C>(0, 0);
+        }
+      } else {
+        const C* p0 = buf.p + sbuf_phys(IL ? ((pos << ltx) + line) : (line * ls + pos));
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[b][r] = p0[sbuf_phys(r * S)];
+      }
+      if constexpr (KIND == PLACE_INV && LGM > 0) {
+        C w[R];
+        place_twiddles<R, TWT, LG, VPT, ST>(tw, q & ((1 << LGM) - 1), lgmax, w);
+#pragma unroll
+        for (int r = 1; r < R; ++r) v[b][r] = cmul(v[b][r], w[r]);
+      }
+      if constexpr (HALF && IN && R == 16) dft16<true>(v[b], false);
+      else dftR<R>(v[b], false);
+    }
+  }
+  if (IN) cp_async_wait_all();
+  if (WAIT) __syncthreads();
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    const int g = threadIdx.x + b * blockDim.x;
+    if (g < total) {
+      const int line = IL ? (g & ((1 << ltx) - 1)) : (g >> LGQ);
+      const int q = IL ? (g >> ltx) : (g & ((1 << LGQ) - 1));
+      const int j = q & ((1 << LGM) - 1);
+      const int pos = ((q >> LGM) << LGB) + j;
+      if constexpr (KIND == PLACE_CONV) {
+        // the last stage (M = 1): frequencies kb + r L/R of block q
+        int kb = 0, rem = q, lgr = LGQ, lgk = 0;
+#pragma unroll
+        for (int s = 0; s < ST; ++s) {
+          lgr -= clog2(P::radix(s));
+          kb += (rem >> lgr) << lgk;
+          rem &= (1 << lgr) - 1;
+          lgk += clog2(P::radix(s));
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[b][r] = mid(line, kb + (r << LGQ), pos + r, v[b][r]);
+        dftR<R>(v[b], false);
+      }
+      if constexpr (KIND == PLACE_FWD && LGM > 0) {
+        C w[R];
+        place_twiddles<R, TWT, LG, VPT, ST>(tw, j, lgmax, w);
+#pragma unroll
+        for (int r = 1; r < R; ++r) v[b][r] = cmul(v[b][r], w[r]);
+      }
+      if (OUT) {
+#pragma unroll
+        for (int r = 0; r < (HOUT ? R / 2 : R); ++r) out(line, pos + (r << LGM), v[b][r]);
+      } else {
+        C* p0 = buf.p + sbuf_phys(IL ? ((pos << ltx) + line) : (line * ls + pos));
+#pragma unroll
+        for (int r = 0; r < R; ++r) p0[sbuf_phys(r * S)] = v[b][r];
+      }
+    }
+  }
+  if (!OUT) __syncthreads();
+}
+
+template <int LG, int VPT, bool IL, bool TWT, int ST, int KIND, typename C, typename Load, typename Mid, typename Out>
+__device__ __forceinline__ void place_stages(SBuf<C> buf, int ls, int ltx, int nlines, const C* FL_RESTRICT tw,
+                                             int lgmax, Load& load, Mid& mid, Out& out) {
+  typedef FftPlan<LG, VPT> P;
+  constexpr int LAST = P::S - 1;
+  if constexpr (KIND == PLACE_FWD) {
+    // natural order (upper half zero) to places
+    place_stage<LG, VPT, IL, ST == 0, false, TWT, ST, PLACE_FWD, ST == 0, ST == LAST>(buf, ls, ltx, nlines, tw, lgmax,
+                                                                                    load, mid, out);
+    if constexpr (ST < LAST)
+      place_stages<LG, VPT, IL, TWT, ST + 1, KIND>(buf, ls, ltx, nlines, tw, lgmax, load, mid, out);
+  } else if constexpr (KIND == PLACE_INV) {
+    // places to natural order (lower half)
+    place_stage<LG, VPT, IL, false, ST == 0, TWT, ST, PLACE_INV, ST == LAST, ST == 0>(buf, ls, ltx, nlines, tw, lgmax,
+                                                                                     load, mid, out);
+    if constexpr (ST > 0)
+      place_stages<LG, VPT, IL, TWT, ST - 1, KIND>(buf, ls, ltx, nlines, tw, lgmax, load, mid, out);
+  } else {
+    // forward stages before the last, the middle, and back
+    if constexpr (ST < LAST) {
+      place_stage<LG, VPT, IL, ST == 0, false, TWT, ST, PLACE_FWD, ST == 0, false>(buf, ls, ltx, nlines, tw, lgmax,
+                                                                                  load, mid, out);
+      place_stages<LG, VPT, IL, TWT, ST + 1, KIND>(buf, ls, ltx, nlines, tw, lgmax, load, mid, out);
+      place_stage<LG, VPT, IL, false, ST == 0, TWT, ST, PLACE_INV, false, ST == 0>(buf, ls, ltx, nlines, tw, lgmax,
+                                                                                  load, mid, out);
+    } else {
+      place_stage<LG, VPT, IL, LAST == 0, LAST == 0, TWT, ST, PLACE_CONV, LAST == 0, LAST == 0>(
+          buf, ls, ltx, nlines, tw, lgmax, load, mid, out);
+    }
+  }
+}
+
+// load(line, n, IntC<lg stride>, IntC<count>, v) gives the values of `count`
+// places n, n + stride, .. of a line.  KIND PLACE_CONV: out(line, n, swapped
+// value) for n < L/2 of the circular convolution of the zero-padded input (n <
+// L/2), with mid(line, k, place, v) returning the swapped product at frequency k.
+// PLACE_FWD: the transform of the zero-padded input, out(line, place, v).
+// PLACE_INV: load gives swapped values by place, out(line, n, swapped value)
+// for n < L/2.  What the CTA's asynchronous copies wrote to shared memory may
+// be read by mid and as twiddles.
+#define FL_PLACE_LEN(LGV)                                                                                   \
+  if constexpr (LGV >= LGLO && LGV <= LGHI) {                                                               \
+    if (lg == LGV) {                                                                                        \
+      constexpr int ST0 = KIND == PLACE_INV ? FftPlan<LGV, VPT>::S - 1 : 0;                                 \
+      place_stages<LGV, VPT, IL, TWT, ST0, KIND>(buf, ls, ltx, nlines, tw, lgmax, load, mid, out);          \
+      return;                                                                                               \
+    }                                                                                                       \
+  }
+template <int KIND, int VPT, bool IL, int LGHI, int LGLO, bool TWT, typename C, typename Load, typename Mid,
+          typename Out>
+__device__ __forceinline__ void fft_places(SBuf<C> buf, int lg, int ls, int ltx, int nlines, const C* FL_RESTRICT tw,
+                                           int lgmax, Load load, Mid mid, Out out) {
+  FL_PLACE_LEN(13)
+  FL_PLACE_LEN(12)
+  FL_PLACE_LEN(11)
+  FL_PLACE_LEN(10)
+  FL_PLACE_LEN(9)
+  FL_PLACE_LEN(8)
+  FL_PLACE_LEN(7)
+  FL_PLACE_LEN(6)
+  FL_PLACE_LEN(5)
+  FL_PLACE_LEN(4)
+}
+#undef FL_PLACE_LEN
 
 }  // namespace fl

@@ -48,9 +48,11 @@ struct Tables {
   FxW* fchirp[3] = {nullptr, nullptr, nullptr};
   FxW* fbhat[3] = {nullptr, nullptr, nullptr};   // / 2^bexp
   int bexp[3] = {0, 0, 0};
+  C* ptw[3] = {nullptr, nullptr, nullptr};     // FP32: twiddle tables of the strided passes' stages
   // FP32 DST tables
   C* chirp[3] = {nullptr, nullptr, nullptr};
-  C* bhat[3] = {nullptr, nullptr, nullptr};
+  C* bhat[3] = {nullptr, nullptr, nullptr};   // by place of the 16-value stage plan
+  C* bhat8 = nullptr;         // last axis, by place of the 8-value plan
   C* S = nullptr;             // operator spectrum workspace
   T* t = nullptr;             // preconditioner workspace (N)
   T* mu[3] = {nullptr, nullptr, nullptr};  // eigenvalues of C h^d L per axis

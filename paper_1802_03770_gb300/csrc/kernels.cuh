@@ -46,16 +46,6 @@ __device__ __forceinline__ void pdl_release() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// Asynchronous global -> shared copies of 4, 8 or 16 bytes (no registers
-// held while in flight); cp_async_wait_all() waits for the calling thread's
-// own copies, a barrier then makes them visible to the CTA.
-template <int BYTES>
-__device__ __forceinline__ void cp_async(void* smem, const void* gmem) {
-  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(sa), "l"(gmem), "n"(BYTES) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
 // Device-resident state of one CG solve (all reductions in FP64).
 struct PcgState {
   double rz;       // r^T z of the current iterate
@@ -420,8 +410,8 @@ __global__ void __launch_bounds__(THREADS, min_ctas<T>(THREADS, LGLO)) k_rows_fw
 template <typename T>
 struct ColsArgs {
   typename Cplx<T>::type* S;
-  const typename Cplx<T>::type* tw;
-  const T* sig;            // COLS_CONV: symbol
+  const typename Cplx<T>::type* ptw;   // FP32: the stages' twiddle tables (place_twiddles)
+  const T* sig;            // FP32, COLS_CONV: symbol
   const PcgState* st;
   int H, lg, lgmax;
   int rows_in, rows_out;
@@ -439,14 +429,26 @@ struct ColsArgs {
   int sig_exp;
 };
 
-// The tile is kept in its natural layout, buf[r * TX + c] (row r of the line,
-// column c), and transformed with the interleaved-line FFT; global loads are
-// issued U at a time so that several are in flight per thread.
+// Row of the staged symbol that holds frequency kk: one pad row after every
+// 16, since neighbouring blocks of the middle stage are 16 frequencies apart
+// (the same bank without the pad).
+__device__ __forceinline__ int sig_row(int kk) { return kk + (kk >> 4); }
+
+// FP32.  The tile keeps its natural layout, buf[r * TX + c] (row r of the line,
+// column c); its transforms are in place (fft_places): legs of the first stage
+// come from global memory, outputs of the last stage go there.  A convolution
+// (forward transform, symbol, inverse) takes 2 (S - 1) trips through shared
+// memory for S stages.  In 3D the middle axis is kept in the places of its
+// transform between its forward and inverse passes (place_frequency).
+//
+// Bound by instruction issue and shared memory.  Against autosort stages with
+// the tile staged first: 256^3 convolution pass 367 -> 337 us, middle-axis
+// passes 157, 160 -> 116, 133 us, 1024^2 convolution 24.5 -> 22.4 us (between
+// events).
 template <typename T, int THREADS, int VPT, int LGLO, int LGHI>
 __device__ __forceinline__ void body_cols_at(const ColsArgs<T>& a, int kx0, int by, const int lg,
                                              const int ltx) {
   typedef typename Cplx<T>::type C;
-  constexpr int U = 8;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const SBuf<C> buf{reinterpret_cast<C*>(smem_raw)};
   if (a.st && a.st->done) return;
@@ -455,74 +457,52 @@ __device__ __forceinline__ void body_cols_at(const ColsArgs<T>& a, int kx0, int 
   const int o = by;
   const int ncol = min(TX, a.H - kx0);
   C* base = a.S + (size_t)o * a.ostride + kx0;
-  // the convolution's input has rows_in <= L/2 rows: only the lower half of
-  // the tile is written, the transform's first stage reads the rest as zeros
-  const int hL = L >> 1;
-  const int total = TX * (a.mode == COLS_CONV ? hL : L);
-  // convolution: the symbol's rows kk = 0..L/2 for the tile's columns are
-  // staged in shared memory beside the FFT tile (ssig[kk * TX + c]) by
-  // asynchronous copies issued before the tile's loads, so that the forward
-  // transform's last stage multiplies without a global load in flight
-  // FP32: the twiddles of this line length, exp(-2 pi i m / L) for m < L
-  // (every 2^(lgmax - lg)-th entry of the plan's table), are copied to
-  // shared memory beside the tile (stw): the stages then load every power
-  // of a butterfly's twiddle instead of computing it
-  constexpr bool TWT = sizeof(T) == 4;
+  // the stages' twiddles (place_twiddles) beside the tile, and for a convolution
+  // the symbol's rows kk = 0..L/2 for the tile's columns (row sig_row(kk) of TX
+  // values): asynchronous copies that run beside the first stage's loads
   C* stw = reinterpret_cast<C*>(smem_raw + sbuf_elems((long long)TX * L) * sizeof(C));
-  T* ssig = reinterpret_cast<T*>(smem_raw + (sbuf_elems((long long)TX * L) + (TWT ? L : 0)) * sizeof(C));
-  const C* twp = TWT ? stw : a.tw;
-  const int twlg = TWT ? lg : a.lgmax;
-  if constexpr (TWT)
-    for (int m = threadIdx.x; m < L; m += THREADS) cp_async<sizeof(C)>(&stw[m], &a.tw[m << (a.lgmax - lg)]);
-  const T* FL_RESTRICT sig = a.sig + kx0;
-  if (a.mode == COLS_CONV && a.Lo) sig += (size_t)min(o, a.Lo - o) * a.sig_outer;
-  const int nsym = a.mode == COLS_CONV ? ((hL + 1) << ltx) : 0;
-  for (int e = threadIdx.x; e < nsym; e += THREADS) {
-    const int kk = e >> ltx, c = e & (TX - 1);
-    if (c < ncol) cp_async<sizeof(T)>(&ssig[e], &sig[(size_t)kk * a.sig_line + c]);
-    else ssig[e] = (T)0;
-  }
-  for (int e0 = threadIdx.x; e0 < total; e0 += THREADS * U) {
-    C v[U];
+  const int ntw = place_table_len(lg);
+  T* ssig = reinterpret_cast<T*>(smem_raw + (sbuf_elems((long long)TX * L) + ntw) * sizeof(C));
+  for (int m = threadIdx.x; m < ntw; m += THREADS) cp_async<sizeof(C)>(&stw[m], &a.ptw[m]);
+  const int rows_in = a.rows_in, rows_out = a.rows_out;
+  const long long lstride = a.lstride;
+  auto mid = [=](int c, int k, int, C v) -> C { return cscale(cswap(v), ssig[(sig_row(min(k, L - k)) << ltx) + c]); };
+  auto out = [=](int c, int n, C v) {
+    if (c < ncol && n < rows_out) base[(size_t)n * lstride + c] = cswap(v);
+  };
+  auto ld = [=](int c, int n0, auto lgs, auto cnt, C* v) {
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int e = e0 + u * THREADS;
-      const int r = e >> ltx, c = e & (TX - 1);
-      v[u] = cmake<C>((T)0, (T)0);
-      if (e < total && r < a.rows_in && c < ncol) v[u] = base[(size_t)r * a.lstride + c];
+    for (int r = 0; r < decltype(cnt)::v; ++r) {
+      const int n = n0 + (r << decltype(lgs)::v);
+      v[r] = (c < ncol && n < rows_in) ? base[(size_t)n * lstride + c] : cmake<C>((T)0, (T)0);
     }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int e = e0 + u * THREADS;
-      if (e < total) buf[e] = v[u];
-    }
-  }
-  cp_async_wait_all();
-  __syncthreads();
+  };
   if (a.mode == COLS_CONV) {
-    // forward FFT whose last stage multiplies by the staged symbol on the
-    // way out (columns beyond ncol are scaled by 0 and never stored)
-    auto ld = [=](int c, int k) -> C { return k < hL ? buf[(k << ltx) + c] : cmake<C>((T)0, (T)0); };
-    auto epi = [=](int c, int k, C v) { buf[(k << ltx) + c] = cscale(v, ssig[(min(k, L - k) << ltx) + c]); };
-    fft_io<VPT, true, true, LGHI, LGLO, TWT>(buf, lg, 0, ltx, TX, twp, twlg, false, ld, true, epi,
-                                            true);
-    __syncthreads();
-    // inverse FFT whose last stage writes the kept rows to global
-    const int rows_out = a.rows_out;
-    const long long lstride = a.lstride;
-    auto ld2 = [=](int c, int k) -> C { return buf[(k << ltx) + c]; };
-    auto epi2 = [=](int c, int k, C v) {
-      if (c < ncol && k < rows_out) base[(size_t)k * lstride + c] = v;
+    const T* FL_RESTRICT sig = a.sig + kx0;
+    if (a.Lo) {
+      const int f = place_frequency(o, 31 - __clz(a.Lo), VPT);
+      sig += (size_t)min(f, a.Lo - f) * a.sig_outer;
+    }
+    const int nsym = ((L >> 1) + 1) << ltx;
+    for (int e = threadIdx.x; e < nsym; e += THREADS) {
+      const int kk = e >> ltx, c = e & (TX - 1);
+      T* d = ssig + (sig_row(kk) << ltx) + c;
+      if (c < ncol) cp_async<sizeof(T)>(d, &sig[(size_t)kk * a.sig_line + c]);
+      else *d = (T)0;
+    }
+    fft_places<PLACE_CONV, VPT, true, LGHI, LGLO, true>(buf, lg, 0, ltx, TX, stw, lg, ld, mid, out);
+  } else if (a.mode == COLS_FWD) {
+    auto outp = [=](int c, int p, C v) {
+      if (c < ncol) base[(size_t)p * lstride + c] = v;
     };
-    fft_io<VPT, true, false, LGHI, LGLO, TWT>(buf, lg, 0, ltx, TX, twp, twlg, true, ld2, true, epi2,
-                                             false);
-    return;
-  }
-  fft_smem<VPT, true, LGHI, LGLO, TWT>(buf, lg, 0, ltx, TX, twp, twlg, a.mode == COLS_INV);
-  const int tout = TX * a.rows_out;
-  for (int e = threadIdx.x; e < tout; e += THREADS) {
-    const int r = e >> ltx, c = e & (TX - 1);
-    if (c < ncol) base[(size_t)r * a.lstride + c] = buf[e];
+    fft_places<PLACE_FWD, VPT, true, LGHI, LGLO, true>(buf, lg, 0, ltx, TX, stw, lg, ld, mid, outp);
+  } else {
+    auto ldi = [=](int c, int p0, auto lgs, auto cnt, C* v) {
+#pragma unroll
+      for (int r = 0; r < decltype(cnt)::v; ++r)
+        v[r] = c < ncol ? cswap(base[(size_t)(p0 + (r << decltype(lgs)::v)) * lstride + c]) : cmake<C>((T)0, (T)0);
+    };
+    fft_places<PLACE_INV, VPT, true, LGHI, LGLO, true>(buf, lg, 0, ltx, TX, stw, lg, ldi, mid, out);
   }
 }
 
@@ -721,20 +701,6 @@ __global__ void __launch_bounds__(THREADS, min_ctas<T>(THREADS, LGLO)) k_rows_in
   pdl_release();
 }
 
-// In place on 2^ltx interleaved lines of length L = 2^lg in shared memory
-// (element j of line c at j * 2^ltx + c): y = IFFT(FFT(v) * bhat), the
-// chirp-z convolution of the DST-I (bhat already holds the 1/L); the
-// multiply is done by the forward transform's last stage.
-template <int VPT, int LGHI, bool TWT = false, typename C>
-__device__ __forceinline__ void chirp_conv_il(SBuf<C> buf, int ltx, int L, int lg, int lgmax,
-                                              const C* FL_RESTRICT tw, const C* FL_RESTRICT bhat) {
-  auto ld = [=](int c, int k) -> C { return buf[(k << ltx) + c]; };
-  auto epi = [=](int c, int k, C v) { buf[(k << ltx) + c] = cmul(v, bhat[k]); };
-  fft_io<VPT, true, false, LGHI, 4, TWT>(buf, lg, 0, ltx, 1 << ltx, tw, lgmax, false, ld, true, epi, true);
-  __syncthreads();
-  fft_smem<VPT, true, LGHI, 4, TWT>(buf, lg, 0, ltx, 1 << ltx, tw, lgmax, true);
-}
-
 // ---------------------------------------------------------------------------
 // Preconditioner: DST-I along the last axis (rows of length n), by chirp-z.
 // DPRE_UPDATE fuses the CG update before the transform:
@@ -748,7 +714,10 @@ struct DstRowsArgs {
   T* out;
   const typename Cplx<T>::type* tw;
   const typename Cplx<T>::type* chirp;   // c_{j+1}, j = 0..n-1
-  const typename Cplx<T>::type* bhat;    // FFT_L of conj(c_m) embedded circularly, / L
+  // FFT_L of conj(c_m) embedded circularly, / L, by place (place_frequency) of
+  // the stage plans with 16 and with 8 values per thread
+  const typename Cplx<T>::type* bhat;
+  const typename Cplx<T>::type* bhat8;
   PcgState* st;            // DPRE_UPDATE: alpha from here; FIN_STEP: updated
   // DPRE_UPDATE
   T* x; T* r; const T* p; const T* q;
@@ -791,93 +760,70 @@ __device__ __forceinline__ void body_dst_rows_at(const DstRowsArgs<T>& a, int bx
   const int NL = (VPT * THREADS) / L;
   const int row0 = bx * NL;
   const int nl = min(NL, a.rows - row0);
-  // Only the lower half of each line is written (n <= L/2); the transform's
-  // first stage reads the upper half as zeros.
-  DotAcc<T> rr;
-  const int hL = L >> 1;
-  const int tot = nl * hL;
-  if (a.pre == DPRE_UPDATE) {
-    const T al = (T)a.st->alpha;
-    T* FL_RESTRICT xv = a.x;
-    T* FL_RESTRICT rv = a.r;
-    const T* FL_RESTRICT pv = a.p;
-    const T* FL_RESTRICT qv = a.q;
-    constexpr int U = 4;   // elements in flight per thread
-    for (int e0 = threadIdx.x; e0 < tot; e0 += THREADS * U) {
-      T xo[U], ro[U], po[U], qo[U];
+  // Both transforms in place (fft_places), the first stage's legs from global
+  // memory with all loads before the first use, the sine coefficients from
+  // the last stage's registers: 256^3 213 -> 157 us (DST along the middle axis
+  // 204 -> 130), 255^2 preconditioner 14.1 -> 10.8 us, 1024^2 rows unchanged
+  // (18.6: one wave, bound by its loads and one CTA's chain).
+  DotAcc<T> rr, dp;
+  const bool update = a.pre == DPRE_UPDATE;
+  const T al = update ? (T)a.st->alpha : (T)0;
+  const C* FL_RESTRICT chirp = a.chirp;
+  const C* FL_RESTRICT bhat = VPT == 8 ? a.bhat8 : a.bhat;
+  const int n = a.n;
+  auto ld = [&](int q, int n0, auto lgs, auto cnt, C* v) {
+    constexpr int N = decltype(cnt)::v, LGS = decltype(lgs)::v;
+    const size_t row = (size_t)(row0 + q) * n;
+    T xo[N], ro[N], po[N], qo[N];
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int e = e0 + u * THREADS;
-        const int q = e >> (lg - 1), j = e & (hL - 1);
-        xo[u] = ro[u] = po[u] = qo[u] = (T)0;
-        if (e < tot && j < a.n) {
-          const size_t idx = (size_t)(row0 + q) * a.n + j;
-          xo[u] = xv[idx];
-          ro[u] = rv[idx];
-          po[u] = pv[idx];
-          qo[u] = qv[idx];
+    for (int r = 0; r < N; ++r) {
+      const int j = n0 + (r << LGS);
+      xo[r] = ro[r] = po[r] = qo[r] = (T)0;
+      if (j < n) {
+        if (update) {
+          xo[r] = a.x[row + j];
+          ro[r] = a.r[row + j];
+          po[r] = a.p[row + j];
+          qo[r] = a.q[row + j];
+        } else if (!a.mask_in || a.mask_in[row + j]) {
+          ro[r] = a.in[row + j];
         }
       }
+    }
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int e = e0 + u * THREADS;
-        if (e >= tot) continue;
-        const int q = e >> (lg - 1), j = e & (hL - 1);
-        C v = cmake<C>((T)0, (T)0);
-        if (j < a.n) {
-          const size_t idx = (size_t)(row0 + q) * a.n + j;
-          const T rn = ro[u] - al * qo[u];
-          xv[idx] = xo[u] + al * po[u];
-          rv[idx] = rn;
+    for (int r = 0; r < N; ++r) {
+      const int j = n0 + (r << LGS);
+      v[r] = cmake<C>((T)0, (T)0);
+      if (j < n) {
+        T rn = ro[r];
+        if (update) {
+          rn = ro[r] - al * qo[r];
+          a.x[row + j] = xo[r] + al * po[r];
+          a.r[row + j] = rn;
           rr.add(rn * rn);
-          v = cscale(a.chirp[j], rn);
         }
-        buf[q * ls + j] = v;
+        v[r] = cscale(chirp[j], rn);
       }
     }
-  } else {
-#pragma unroll 4
-    for (int e = threadIdx.x; e < tot; e += THREADS) {
-      const int q = e >> (lg - 1), j = e & (hL - 1);
-      C v = cmake<C>((T)0, (T)0);
-      if (j < a.n) {
-        const size_t idx = (size_t)(row0 + q) * a.n + j;
-        if (!a.mask_in || a.mask_in[idx]) v = cscale(a.chirp[j], a.in[idx]);
-      }
-      buf[q * ls + j] = v;
-    }
-  }
-  __syncthreads();
+  };
+  auto mid = [=](int q, int, int p, C v) -> C { return cswap(cmul(v, bhat[p])); };
   {
-    // forward FFT whose last stage multiplies by bhat on the way out
-    const C* FL_RESTRICT bhat = a.bhat;
-    auto ld = [=](int q, int k) -> C { return k < hL ? buf[q * ls + k] : cmake<C>((T)0, (T)0); };
-    auto epi = [=](int q, int k, C v) { buf[q * ls + k] = cmul(v, bhat[k]); };
-    fft_io<VPT, false, true, LGHI, LGLO>(buf, lg, ls, 0, nl, a.tw, a.lgmax, false, ld,
-                                                       true, epi, true);
-  }
-  __syncthreads();
-  DotAcc<T> dp;
-  {
-    // inverse FFT whose last stage writes the DST coefficients to global
     const T post = (T)a.post;
-    const C* FL_RESTRICT chirp = a.chirp;
     T* FL_RESTRICT outp = a.out;
     const T* FL_RESTRICT dw = a.dotw;
     const uint8_t* FL_RESTRICT mask = a.mask_out;
     const T* FL_RESTRICT add = a.add;
-    const int n = a.n;
-    auto ld = [=](int q, int k) -> C { return buf[q * ls + k]; };
-    auto epi = [=, &dp](int q, int k, C v) {
+    // v is swapped: Im(chirp conv) of the value itself
+    auto out = [=, &dp](int q, int k, C v) {
       if (k < n) {
         const size_t idx = (size_t)(row0 + q) * n + k;
-        const T o = (!mask || mask[idx]) ? cmul(chirp[k], v).y * post + (add ? add[idx] : (T)0) : (T)0;
+        const C c = chirp[k];
+        const T o = (!mask || mask[idx]) ? (c.x * v.x + c.y * v.y) * post + (add ? add[idx] : (T)0) : (T)0;
         outp[idx] = o;
         if (dw) dp.add(o * dw[idx]);
       }
     };
-    fft_io<VPT, false, false, LGHI, LGLO>(buf, lg, ls, 0, nl, a.tw, a.lgmax, true, ld,
-                                                        true, epi, false);
+    fft_places<PLACE_CONV, VPT, false, LGHI, LGLO, false>(buf, lg, ls, 0, nl, a.tw, a.lgmax, ld, mid, out);
   }
   if (a.pre == DPRE_UPDATE) {
     const double s = rr.cta_total(red);
@@ -933,7 +879,7 @@ __global__ void __launch_bounds__(THREADS, min_ctas<T>(THREADS, LGLO)) k_dst_row
 template <typename T>
 struct DstColsArgs {
   T* v;
-  const typename Cplx<T>::type* tw;
+  const typename Cplx<T>::type* ptw;   // FP32: the stages' twiddle tables
   const typename Cplx<T>::type* chirp;
   const typename Cplx<T>::type* bhat;
   const PcgState* st;
@@ -951,7 +897,6 @@ template <typename T, int THREADS, int VPT, int LGLO, int LGHI>
 __device__ __forceinline__ void body_dst_cols_at(const DstColsArgs<T>& a, int c0, int by, const int lg,
                                                  const int ltx) {
   typedef typename Cplx<T>::type C;
-  constexpr int U = 8;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const SBuf<C> buf{reinterpret_cast<C*>(smem_raw)};
   if (a.st && a.st->done) return;
@@ -960,40 +905,36 @@ __device__ __forceinline__ void body_dst_cols_at(const DstColsArgs<T>& a, int c0
   const int o = by;
   const int ncol = min(TX, a.ncols - c0);
   T* base = a.v + (size_t)o * a.ostride + c0;
-  const int total = TX * L;
-  // FP32: the line length's twiddles in shared memory (as in body_cols_at)
-  constexpr bool TWT = sizeof(T) == 4;
+  // the stages' twiddles in shared memory (as in body_cols_at)
   C* stw = reinterpret_cast<C*>(smem_raw + sbuf_elems((long long)TX * L) * sizeof(C));
-  if constexpr (TWT)
-    for (int m = threadIdx.x; m < L; m += THREADS) cp_async<sizeof(C)>(&stw[m], &a.tw[m << (a.lgmax - lg)]);
-  for (int e0 = threadIdx.x; e0 < total; e0 += THREADS * U) {
-    T v[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int e = e0 + u * THREADS;
-      const int r = e >> ltx, c = e & (TX - 1);
-      v[u] = (T)0;
-      if (e < total && r < a.n && c < ncol) v[u] = base[(size_t)r * a.lstride + c];
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int e = e0 + u * THREADS;
-      const int r = e >> ltx;
-      if (e < total) buf[e] = r < a.n ? cscale(a.chirp[r], v[u]) : cmake<C>((T)0, (T)0);
-    }
-  }
-  cp_async_wait_all();
-  __syncthreads();
-  chirp_conv_il<VPT, LGHI, TWT>(buf, ltx, L, lg, TWT ? lg : a.lgmax, TWT ? stw : a.tw, a.bhat);
-  const int tout = TX * a.n;
+  for (int m = threadIdx.x; m < place_table_len(lg); m += THREADS) cp_async<sizeof(C)>(&stw[m], &a.ptw[m]);
+  const int n = a.n;
+  const long long lstride = a.lstride;
+  const C* FL_RESTRICT chirp = a.chirp;
+  const C* FL_RESTRICT bhat = a.bhat;
   const T post = (T)a.post;
-  for (int e = threadIdx.x; e < tout; e += THREADS) {
-    const int r = e >> ltx, c = e & (TX - 1);
-    if (c < ncol) {
-      const C y = cmul(a.chirp[r], buf[e]);
-      base[(size_t)r * a.lstride + c] = y.y * post;
+  auto ld = [=](int c, int n0, auto lgs, auto cnt, C* v) {
+    constexpr int N = decltype(cnt)::v, LGS = decltype(lgs)::v;
+    T x[N];
+#pragma unroll
+    for (int r = 0; r < N; ++r) {
+      const int j = n0 + (r << LGS);
+      x[r] = (c < ncol && j < n) ? base[(size_t)j * lstride + c] : (T)0;
     }
-  }
+#pragma unroll
+    for (int r = 0; r < N; ++r) {
+      const int j = n0 + (r << LGS);
+      v[r] = j < n ? cscale(chirp[j], x[r]) : cmake<C>((T)0, (T)0);
+    }
+  };
+  auto mid = [=](int c, int, int p, C v) -> C { return cswap(cmul(v, bhat[p])); };
+  auto out = [=](int c, int k, C v) {
+    if (c < ncol && k < n) {
+      const C w = chirp[k];   // v is swapped
+      base[(size_t)k * lstride + c] = (w.x * v.x + w.y * v.y) * post;
+    }
+  };
+  fft_places<PLACE_CONV, VPT, true, LGHI, LGLO, true>(buf, lg, 0, ltx, TX, stw, lg, ld, mid, out);
 }
 
 template <typename T, int THREADS, int VPT, int LGLO, int LGHI, int LG>

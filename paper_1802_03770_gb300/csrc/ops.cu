@@ -32,8 +32,17 @@ namespace fl {
   } while (0)
 #define FL_ROWS_LAUNCH(KERNEL, T, L, grid, smem, s, arg) \
   FL_SHAPED_LAUNCH(KERNEL, T, Cfg<T>::RT, Cfg<T>::RV, L, grid, smem, s, arg)
-#define FL_COLS_LAUNCH(KERNEL, T, L, grid, smem, s, arg) \
-  FL_SHAPED_LAUNCH(KERNEL, T, Cfg<T>::CT, Cfg<T>::CV, L, grid, smem, s, arg)
+// Strided passes: FP32 tiles of half the widest or less take CTAs of half the
+// threads.
+#define FL_COLS_LAUNCH(KERNEL, T, L, grid, smem, s, arg)                                     \
+  do {                                                                                      \
+    constexpr int hc_ = Cfg<T>::CT / 2;                                                     \
+    if (sizeof(T) == 4 && ((L) << (arg).ltx) <= hc_ * Cfg<T>::CV) {                         \
+      if constexpr (sizeof(T) == 4) pdl_launch(KERNEL<T, hc_, Cfg<T>::CV>, grid, hc_, smem, s, arg); \
+    } else {                                                                                \
+      FL_SHAPED_LAUNCH(KERNEL, T, Cfg<T>::CT, Cfg<T>::CV, L, grid, smem, s, arg);           \
+    }                                                                                       \
+  } while (0)
 
 // ---------------------------------------------------------------------------
 // CG vector kernels (grid-stride, kVecBlocks CTAs, one partial per CTA).
@@ -352,6 +361,8 @@ cudaError_t configure_kernels() {
   FL_SET(k_cols<float, Cfg<float>::CT, Cfg<float>::CV>);
   FL_SET(k_dst_rows<float, Cfg<float>::RT, Cfg<float>::RV>);
   FL_SET(k_dst_cols<float, Cfg<float>::CT, Cfg<float>::CV>);
+  FL_SET(k_cols<float, Cfg<float>::CT / 2, Cfg<float>::CV>);
+  FL_SET(k_dst_cols<float, Cfg<float>::CT / 2, Cfg<float>::CV>);
   // the wide instantiations of the longest lines
   FL_SET(k_rows_fwd<float, 256, 16, 12>);
   FL_SET(k_rows_fwd<float, 512, 16, 13>);
@@ -459,13 +470,13 @@ ApplyChain<T> build_apply(const Geo& g, const Tables<T>& tb, const ApplyIO<T>& i
   auto cols = [&](int axis, int mode, int rows_in, int rows_out, long long lstride,
                   long long ostride, int nouter, long long sig_line, long long sig_outer, int Lo) {
     ColsArgs<T>& a = ch.cols[ch.ncols];
-    a.S = tb.S; a.tw = tb.tw; a.sig = tb.sig; a.st = io.st;
+    a.S = tb.S; a.ptw = tb.ptw[axis]; a.sig = tb.sig; a.st = io.st;
     a.ftw = tb.ftw; a.fsig = tb.fsig; a.sig_exp = tb.sig_exp;
     a.H = g.H; a.lg = g.lg[axis]; a.lgmax = g.lgmax;
     a.rows_in = rows_in; a.rows_out = rows_out; a.lstride = lstride; a.ostride = ostride;
     a.nouter = nouter; a.mode = mode; a.sig_line = sig_line; a.sig_outer = sig_outer; a.Lo = Lo;
     const int L = g.L[axis];
-    const int tx = tile_at<T>(plan_tx<T>(tb, axis, L), L, io.col_threads);
+    const int tx = tile_at<T>(plan_tx<T>(g, tb, axis), L, io.col_threads);
     a.ltx = ilog2i(tx);
     ch.cols_grid[ch.ncols] = dim3((g.H + tx - 1) / tx, nouter);
     ch.cols_smem[ch.ncols] = mode == COLS_CONV ? conv_tile_bytes<T>(tx, L) : cols_bytes<T>(tx, L);
@@ -536,7 +547,7 @@ PrecChain<T> build_precond(const Geo& g, const Tables<T>& tb, const PrecIO<T>& i
   for (int i = 1; i < d; ++i) post *= 2.0 / (g.n[i] + 1.0);
   {
     DstRowsArgs<T>& a = ch.first;
-    a.in = io.in; a.out = tb.t; a.tw = tb.tw; a.chirp = tb.chirp[d - 1]; a.bhat = tb.bhat[d - 1];
+    a.in = io.in; a.out = tb.t; a.tw = tb.tw; a.chirp = tb.chirp[d - 1]; a.bhat = tb.bhat[d - 1]; a.bhat8 = tb.bhat8;
     a.ftw = tb.ftw; a.fchirp = tb.fchirp[d - 1]; a.fbhat = tb.fbhat[d - 1]; a.bexp = tb.bexp[d - 1];
     a.st = io.st; a.x = io.x; a.r = io.r; a.p = io.p; a.q = io.q;
     a.rr_part = io.rr_part;
@@ -548,13 +559,13 @@ PrecChain<T> build_precond(const Geo& g, const Tables<T>& tb, const PrecIO<T>& i
   ch.ncols = 0;
   auto cols = [&](int axis, long long lstride, long long ostride, int nouter) {
     DstColsArgs<T>& a = ch.cols[ch.ncols];
-    a.v = tb.t; a.tw = tb.tw; a.chirp = tb.chirp[axis]; a.bhat = tb.bhat[axis]; a.st = io.st;
+    a.v = tb.t; a.ptw = tb.ptw[axis]; a.chirp = tb.chirp[axis]; a.bhat = tb.bhat[axis]; a.st = io.st;
     a.ftw = tb.ftw; a.fchirp = tb.fchirp[axis]; a.fbhat = tb.fbhat[axis]; a.bexp = tb.bexp[axis];
     a.post = 1.0;
     a.n = g.n[axis]; a.ncols = nx; a.lg = g.lg[axis]; a.lgmax = g.lgmax;
     a.ostride = ostride; a.lstride = lstride;
     const int L = g.L[axis];
-    const int tx = tile_at<T>(plan_tx<T>(tb, axis, L), L, io.col_threads);
+    const int tx = tile_at<T>(plan_tx<T>(g, tb, axis), L, io.col_threads);
     a.ltx = ilog2i(tx);
     ch.cols_grid[ch.ncols] = dim3((nx + tx - 1) / tx, nouter);
     ch.cols_smem[ch.ncols] = cols_bytes<T>(tx, L);
@@ -581,7 +592,7 @@ PrecChain<T> build_precond(const Geo& g, const Tables<T>& tb, const PrecIO<T>& i
   }
   {
     DstRowsArgs<T>& a = ch.last;
-    a.in = tb.t; a.out = io.out; a.tw = tb.tw; a.chirp = tb.chirp[d - 1]; a.bhat = tb.bhat[d - 1];
+    a.in = tb.t; a.out = io.out; a.tw = tb.tw; a.chirp = tb.chirp[d - 1]; a.bhat = tb.bhat[d - 1]; a.bhat8 = tb.bhat8;
     a.ftw = tb.ftw; a.fchirp = tb.fchirp[d - 1]; a.fbhat = tb.fbhat[d - 1]; a.bexp = tb.bexp[d - 1];
     a.st = io.st; a.x = nullptr; a.r = nullptr; a.p = nullptr; a.q = nullptr;
     a.rr_part = nullptr;

@@ -283,11 +283,23 @@ fl_status build_tables(fl_plan* p) {
       bx[k] = fix_const(ldexpl(v.real(), -bexp), ldexpl(v.imag(), -bexp));
       b32[k] = make_float2((float)v.real(), (float)v.imag());
     }
+    // FP32: in the order in which the transforms hold the frequencies
+    std::vector<float2> b16(L), b8(L);
+    for (int k = 0; k < L; ++k) {
+      b16[k] = b32[place_frequency(k, g.lg[ax], 16)];
+      b8[k] = b32[place_frequency(k, g.lg[ax], 8)];
+    }
+    std::vector<float2> pt(place_table_len(g.lg[ax]));
+    for (size_t m = 0; m < pt.size(); ++m)
+      pt[m] = tw32[(size_t)place_table_power((int)m, g.lg[ax], Cfg<float>::CV) << (g.lgmax - g.lg[ax])];
+    us = upload_table(p, &p->t32.ptw[ax], pt);
+    if (us != FL_OK) return us;
     p->t64.bexp[ax] = bexp;
     us = upload_table(p, &p->t64.fchirp[ax], cx);
     if (us == FL_OK) us = upload_table(p, &p->t64.fbhat[ax], bx);
     if (us == FL_OK) us = upload_table(p, &p->t32.chirp[ax], c32);
-    if (us == FL_OK) us = upload_table(p, &p->t32.bhat[ax], b32);
+    if (us == FL_OK) us = upload_table(p, &p->t32.bhat[ax], b16);
+    if (us == FL_OK && ax == g.d - 1) us = upload_table(p, &p->t32.bhat8, b8);
     if (us != FL_OK) return us;
     // eigenvalues of C h^d L along this axis: c (-a) 4 sin^2(pi k / (2 (n+1)))
     std::vector<double> mu(n);
@@ -1220,8 +1232,8 @@ fl_status fl_plan_autotune(fl_plan* p, int tx_out[6]) {
     const int na = strided_axes(p->g, axes);
     for (int ia = 0; ia < na; ++ia) {
       const int ax = axes[ia];
-      tx_out[ax] = plan_tx<float>(p->t32, ax, p->g.L[ax]);
-      tx_out[3 + ax] = plan_tx<double>(p->t64, ax, p->g.L[ax]);
+      tx_out[ax] = plan_tx<float>(p->g, p->t32, ax);
+      tx_out[3 + ax] = plan_tx<double>(p->g, p->t64, ax);
     }
   }
   return FL_OK;
