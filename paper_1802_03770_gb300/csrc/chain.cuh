@@ -260,7 +260,7 @@ cudaError_t configure_batched_kernels();
 constexpr int kRowsW8Threads = 256;
 void launch_rows_fwd_w8(const RowsFwdArgs<float>& a, int grid, size_t smem, cudaStream_t s);
 void launch_rows_inv_w8(const RowsInvArgs<float>& a, int grid, size_t smem, cudaStream_t s);
-void launch_dst_rows_w8(const DstRowsArgs<float>& a, int grid, size_t smem, cudaStream_t s);
+void launch_dst_rows_w8(const DstRowsArgs<float>& a, int grid, size_t smem, cudaStream_t s);   // either form
 cudaError_t configure_rows_w8();
 // Whether a plan's FP32 row pass of `ctas` CTAs on lines of L points takes
 // the 256 x 8 shape: where the plan asks for it, and by default where the
@@ -275,6 +275,13 @@ template <typename T> inline bool rows_w8(const Tables<T>& tb, int L, int ctas) 
   if (sizeof(T) != 4 || L < 256 || L > 2048) return false;
   if (tb.rshape == 1) return true;
   return ctas <= (L >= 512 ? 304 : 152);
+}
+
+// Whether a DST along an axis takes the odd extension (its points n = 2^k - 1).
+inline bool dst_odd(const Geo& g, int axis) { return g.L[axis] == 2 * (g.n[axis] + 1); }
+// rows of the last axis per CTA of a DST row pass (rt: threads, 0: the Cfg shape)
+template <typename T> inline int dst_row_lines(const Geo& g, int rt) {
+  return row_lines_at<T>(g.L[g.d - 1], rt) * (dst_odd(g, g.d - 1) ? 2 : 1);
 }
 
 template <typename T>

@@ -755,19 +755,110 @@ __device__ __forceinline__ void fx_body_dst_rows(const DstRowsArgs<double>& a, i
   DotAcc<double> dp;
   fx_fft<VPT, false, false, true, LGLO, LGHI>(buf, lg, ls, 0, nl, a.ftw, a.lgmax, mx2, NL, mx2 + NL,
                                               FxLoadFix{buf, ls, 0, false}, true, FxDstRowsEpi{a, s_x, dp, row0, 0}, false);
-  if (update) {
-    const double s = rr.cta_total(red);
-    if (threadIdx.x == 0) a.rr_part[bx] = s;
+  dst_rows_finish(a, bx, rr, dp, red);
+}
+
+// sine coefficients of a pair of rows: Z = -2 i (S_a + i S_b)
+struct FxDstOddEpi {
+  static constexpr bool kNote = false;
+  const DstRowsArgs<double>& a;
+  DotAcc<double>& dp;
+  int pair0, X;
+  __device__ __forceinline__ void begin(int q, int dX, unsigned key) { X = fx_x0(fx_line_field(key)) + dX - 1; }
+  __device__ __forceinline__ unsigned operator()(int q, int k, Fx v) {
+    if (k < 1 || k > a.n) return 0u;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int row = 2 * (pair0 + q) + h;
+      if (row >= a.rows) break;
+      const size_t idx = (size_t)row * a.n + k - 1;
+      double o = 0.0;
+      if (!a.mask_out || a.mask_out[idx]) {
+        o = fx_to(h ? v.x : -v.y, X);
+        if (a.post != 1.0) o *= a.post;
+        if (a.add) o += a.add[idx];
+      }
+      a.out[idx] = o;
+      if (a.dotw) dp.add(o * a.dotw[idx]);
+    }
+    return 0u;
   }
-  if (a.dotw) {
-    const double s = dp.cta_total(red);
-    if (threadIdx.x == 0) a.dot_part[bx] = s;
-    if (a.fin == FIN_STEP && arrive_last(&a.st->arrive, a.nparts)) {
-      const double rrv = cta_sum_partials(a.rr_in, a.rr_count, red);
-      const double rz = cta_sum_partials(a.dot_part, a.nparts, red);
-      if (threadIdx.x == 0) pcg_step(a.st, rrv, rz);
+};
+
+// --- preconditioner rows, n + 1 = L/2 (see body_dst_rows_odd_at) -----------------------
+template <int THREADS, int VPT, int LGLO, int LGHI>
+__device__ __forceinline__ void fx_body_dst_rows_odd(const DstRowsArgs<double>& a, int bx) {
+  constexpr int W = fx_words(THREADS, VPT, LGLO);
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ unsigned s_mx[W];
+  __shared__ double red[32];
+  const SBuf<Fx> buf{reinterpret_cast<Fx*>(smem_raw)};
+  if (a.st && a.st->done) return;
+  const int lg = a.lg, L = 1 << lg, ls = L, hL = L >> 1;
+  const int NL = (VPT * THREADS) >> lg;
+  const int pair0 = bx * NL;
+  const int nl = NL == 1 ? 1 : min(NL, (a.rows + 1) / 2 - pair0);
+  fx_zero<W>(s_mx);
+  __syncthreads();
+  DotAcc<double> rr, dp;
+  const int tot = nl * hL;
+  const bool update = a.pre == DPRE_UPDATE;
+  const double al = update ? a.st->alpha : 0.0;
+  constexpr int U = 2;   // pairs in flight per thread
+  for (int e0 = threadIdx.x; e0 < tot; e0 += THREADS * U) {
+    double xo[2 * U], ro[2 * U], po[2 * U], qo[2 * U];
+#pragma unroll
+    for (int u = 0; u < 2 * U; ++u) {
+      const int e = e0 + (u >> 1) * THREADS;
+      const int row = 2 * (pair0 + (e >> (lg - 1))) + (u & 1), i = e & (hL - 1);
+      xo[u] = ro[u] = po[u] = qo[u] = 0.0;
+      if (e < tot && i > 0 && row < a.rows) {
+        const size_t idx = (size_t)row * a.n + i - 1;
+        if (update) {
+          xo[u] = a.x[idx];
+          ro[u] = a.r[idx];
+          po[u] = a.p[idx];
+          qo[u] = a.q[idx];
+        } else if (!a.mask_in || a.mask_in[idx]) {
+          ro[u] = a.in[idx];
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 2 * U; ++u) {
+      const int e = e0 + (u >> 1) * THREADS;
+      const int row = 2 * (pair0 + (e >> (lg - 1))) + (u & 1), i = e & (hL - 1);
+      if (update && e < tot && i > 0 && row < a.rows) {
+        const size_t idx = (size_t)row * a.n + i - 1;
+        ro[u] -= al * qo[u];
+        a.x[idx] = xo[u] + al * po[u];
+        a.r[idx] = ro[u];
+        rr.add(ro[u] * ro[u]);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int e = e0 + u * THREADS;
+      const int q = e >> (lg - 1), i = e & (hL - 1);
+      const double va = ro[2 * u], vb = ro[2 * u + 1];
+      unsigned key = max(fx_key(va), fx_key(vb));
+      if (e < tot) {
+        buf[q * ls + i] = Fx{__double_as_longlong(va), __double_as_longlong(vb)};   // i = 0: zero, and at L/2
+        buf[q * ls + (i > 0 ? L - i : hL)] = Fx{__double_as_longlong(-va), __double_as_longlong(-vb)};
+      }
+      if (hL >= 32) {
+        key = __reduce_max_sync(0xffffffffu, key);
+        if (e < tot && (threadIdx.x & 31) == 0 && key) atomicMax(s_mx + q, key);
+      } else if (e < tot && key) {
+        atomicMax(s_mx + q, key);
+      }
     }
   }
+  __syncthreads();
+  fx_fft<VPT, false, false, true, LGLO, LGHI>(buf, lg, ls, 0, nl, a.ftw, a.lgmax, s_mx, NL, s_mx + NL,
+                                              FxLoadRaw{buf, ls, 0, false, false}, true,
+                                              FxDstOddEpi{a, dp, pair0, 0}, false);
+  dst_rows_finish(a, bx, rr, dp, red);
 }
 
 // sine coefficients of a column tile

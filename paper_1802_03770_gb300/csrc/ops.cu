@@ -360,6 +360,7 @@ cudaError_t configure_kernels() {
   FL_SET(k_rows_inv<float, Cfg<float>::RT, Cfg<float>::RV>);
   FL_SET(k_cols<float, Cfg<float>::CT, Cfg<float>::CV>);
   FL_SET(k_dst_rows<float, Cfg<float>::RT, Cfg<float>::RV>);
+  FL_SET(k_dst_rows_odd<float, Cfg<float>::RT, Cfg<float>::RV>);
   FL_SET(k_dst_cols<float, Cfg<float>::CT, Cfg<float>::CV>);
   FL_SET(k_cols<float, Cfg<float>::CT / 2, Cfg<float>::CV>);
   FL_SET(k_dst_cols<float, Cfg<float>::CT / 2, Cfg<float>::CV>);
@@ -369,7 +370,9 @@ cudaError_t configure_kernels() {
   FL_SET(k_rows_inv<float, 256, 16, 12>);
   FL_SET(k_rows_inv<float, 512, 16, 13>);
   FL_SET(k_dst_rows<float, 256, 16, 12>);
+  FL_SET(k_dst_rows_odd<float, 256, 16, 12>);
   FL_SET(k_dst_rows<float, 512, 16, 13>);
+  FL_SET(k_dst_rows_odd<float, 512, 16, 13>);
 #undef FL_SET
   return e;
 }
@@ -382,13 +385,16 @@ cudaError_t configure_kernels_f64() {
   FL_SET(k_rows_inv<double, Cfg<double>::RT, Cfg<double>::RV>);
   FL_SET(k_cols<double, Cfg<double>::CT, Cfg<double>::CV>);
   FL_SET(k_dst_rows<double, Cfg<double>::RT, Cfg<double>::RV>);
+  FL_SET(k_dst_rows_odd<double, Cfg<double>::RT, Cfg<double>::RV>);
   FL_SET(k_dst_cols<double, Cfg<double>::CT, Cfg<double>::CV>);
   FL_SET(k_rows_fwd<double, 512, 8, 12>);
   FL_SET(k_rows_inv<double, 512, 8, 12>);
   FL_SET(k_dst_rows<double, 512, 8, 12>);
+  FL_SET(k_dst_rows_odd<double, 512, 8, 12>);
   FL_SET(k_rows_fwd<double, 1024, 8, 13>);
   FL_SET(k_rows_inv<double, 1024, 8, 13>);
   FL_SET(k_dst_rows<double, 1024, 8, 13>);
+  FL_SET(k_dst_rows_odd<double, 1024, 8, 13>);
   FL_SET(k_cols<double, 1024, 8, 13>);
   FL_SET(k_dst_cols<double, 1024, 8, 13>);
   FL_SET(k_rows_c2c<kSymT, kSymV>);
@@ -444,7 +450,7 @@ int apply_partials(const Geo& g) {
 template <typename T>
 int precond_partials(const Geo& g) {
   const long long rows = g.N / g.n[g.d - 1];
-  const int NL = row_lines<T>(g.L[g.d - 1]);
+  const int NL = dst_row_lines<T>(g, 0);
   return (int)((rows + NL - 1) / NL);
 }
 
@@ -539,16 +545,17 @@ PrecChain<T> build_precond(const Geo& g, const Tables<T>& tb, const PrecIO<T>& i
   const int d = g.d;
   const int nx = g.n[d - 1], Lx = g.L[d - 1];
   const long long rows = g.N / nx;
-  const int NL = row_lines_at<T>(Lx, io.row_threads);
+  const int NL = dst_row_lines<T>(g, io.row_threads);
+  const int odd = dst_odd(g, d - 1) ? 1 : 0;
   ch.row_blocks = (int)((rows + NL - 1) / NL);
-  ch.row_smem = smem_bytes<T>(NL, Lx);
+  ch.row_smem = smem_bytes<T>(row_lines_at<T>(Lx, io.row_threads), Lx);
   // DST normalisation of every axis but 0 (solved by the tridiagonal pass)
   double post = 1.0;
   for (int i = 1; i < d; ++i) post *= 2.0 / (g.n[i] + 1.0);
   {
     DstRowsArgs<T>& a = ch.first;
     a.in = io.in; a.out = tb.t; a.tw = tb.tw; a.chirp = tb.chirp[d - 1]; a.bhat = tb.bhat[d - 1]; a.bhat8 = tb.bhat8;
-    a.ftw = tb.ftw; a.fchirp = tb.fchirp[d - 1]; a.fbhat = tb.fbhat[d - 1]; a.bexp = tb.bexp[d - 1];
+    a.ftw = tb.ftw; a.fchirp = tb.fchirp[d - 1]; a.fbhat = tb.fbhat[d - 1]; a.bexp = tb.bexp[d - 1]; a.odd = odd;
     a.st = io.st; a.x = io.x; a.r = io.r; a.p = io.p; a.q = io.q;
     a.rr_part = io.rr_part;
     a.dotw = nullptr; a.dot_part = nullptr; a.post = 1.0;
@@ -593,7 +600,7 @@ PrecChain<T> build_precond(const Geo& g, const Tables<T>& tb, const PrecIO<T>& i
   {
     DstRowsArgs<T>& a = ch.last;
     a.in = tb.t; a.out = io.out; a.tw = tb.tw; a.chirp = tb.chirp[d - 1]; a.bhat = tb.bhat[d - 1]; a.bhat8 = tb.bhat8;
-    a.ftw = tb.ftw; a.fchirp = tb.fchirp[d - 1]; a.fbhat = tb.fbhat[d - 1]; a.bexp = tb.bexp[d - 1];
+    a.ftw = tb.ftw; a.fchirp = tb.fchirp[d - 1]; a.fbhat = tb.fbhat[d - 1]; a.bexp = tb.bexp[d - 1]; a.odd = odd;
     a.st = io.st; a.x = nullptr; a.r = nullptr; a.p = nullptr; a.q = nullptr;
     a.rr_part = nullptr;
     a.dotw = io.dotw; a.dot_part = io.dot_part; a.post = post;
@@ -631,12 +638,15 @@ cudaError_t launch_precond(const Geo& g, const Tables<T>& tb, cudaStream_t s, co
   if (tb.tri_shift != io.shift || tb.tri_scale != io.scale) return cudaErrorInvalidValue;
   const PrecChain<T> ch = build_precond<T>(g, tb, io);
   const int Lx = g.L[g.d - 1];
+  const bool odd = dst_odd(g, g.d - 1);
   FL_KERNEL((sizeof(T) == 4 ? "dst_rows" "<f32>" : "dst_rows" "<f64>"), s,
             if constexpr (sizeof(T) == 4) {
               if (rows_w8(tb, Lx, ch.row_blocks)) launch_dst_rows_w8(ch.first, ch.row_blocks, ch.row_smem, s);
+              else if (odd) FL_ROWS_LAUNCH(k_dst_rows_odd, T, Lx, ch.row_blocks, ch.row_smem, s, ch.first);
               else FL_ROWS_LAUNCH(k_dst_rows, T, Lx, ch.row_blocks, ch.row_smem, s, ch.first);
             } else {
-              FL_ROWS_LAUNCH(k_dst_rows, T, Lx, ch.row_blocks, ch.row_smem, s, ch.first);
+              if (odd) FL_ROWS_LAUNCH(k_dst_rows_odd, T, Lx, ch.row_blocks, ch.row_smem, s, ch.first);
+              else FL_ROWS_LAUNCH(k_dst_rows, T, Lx, ch.row_blocks, ch.row_smem, s, ch.first);
             });
   for (int j = 0; j <= ch.ncols; ++j) {
     if (j == ch.tri_after)
@@ -651,9 +661,11 @@ cudaError_t launch_precond(const Geo& g, const Tables<T>& tb, cudaStream_t s, co
   FL_KERNEL((sizeof(T) == 4 ? "dst_rows" "<f32>" : "dst_rows" "<f64>"), s,
             if constexpr (sizeof(T) == 4) {
               if (rows_w8(tb, Lx, ch.row_blocks)) launch_dst_rows_w8(ch.last, ch.row_blocks, ch.row_smem, s);
+              else if (odd) FL_ROWS_LAUNCH(k_dst_rows_odd, T, Lx, ch.row_blocks, ch.row_smem, s, ch.last);
               else FL_ROWS_LAUNCH(k_dst_rows, T, Lx, ch.row_blocks, ch.row_smem, s, ch.last);
             } else {
-              FL_ROWS_LAUNCH(k_dst_rows, T, Lx, ch.row_blocks, ch.row_smem, s, ch.last);
+              if (odd) FL_ROWS_LAUNCH(k_dst_rows_odd, T, Lx, ch.row_blocks, ch.row_smem, s, ch.last);
+              else FL_ROWS_LAUNCH(k_dst_rows, T, Lx, ch.row_blocks, ch.row_smem, s, ch.last);
             });
   return launch_status();
 }

@@ -59,7 +59,11 @@ __device__ void persist_rows_inv(const PItem& it, int i, int l) {
 __device__ void persist_dst_rows(const PItem& it, int i, int l) {
   const DstRowsArgs<float> a = static_cast<const DstRowsArgs<float>*>(it.args)[i];
   const int gx = it.gx[i];
-  FL_PERSIST_LG_SWITCH(a.lg, (body_dst_rows_at<float, kPT, kPV, kPLo, kPHi>(a, l % gx, l / gx, LG)))
+  if (a.odd) {
+    FL_PERSIST_LG_SWITCH(a.lg, (body_dst_rows_odd_at<float, kPT, kPV, kPLo, kPHi>(a, l % gx, LG)))
+  } else {
+    FL_PERSIST_LG_SWITCH(a.lg, (body_dst_rows_at<float, kPT, kPV, kPLo, kPHi>(a, l % gx, l / gx, LG)))
+  }
 }
 __device__ void persist_dst_cols(const PItem& it, int i, int l) {
   const DstColsArgs<float> a = static_cast<const DstColsArgs<float>*>(it.args)[i];

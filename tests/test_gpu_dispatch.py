@@ -66,3 +66,18 @@ def test_interface_solve_sizes(k, shift, scale):
     for dtype, tol in ((torch.float64, 1e-11), (torch.float32, 2e-5)):
         z = p.precond(dev(r, dtype), shift=shift, scale=scale).cpu().numpy()
         assert rel(z, np.where(mask, ref, 0.0)) <= tol
+
+
+# last axis 2^k - 1 (sines by the odd extension, two rows per line), odd and even numbers of rows, and its neighbours
+@pytest.mark.parametrize("n", [(1, 7), (5, 7), (4, 15), (7, 31), (33, 63), (9, 127), (64, 255), (3, 511), (6, 1023),
+                               (5, 2047), (2, 4095), (5, 126), (5, 128), (5, 9, 31), (4, 31, 31)])
+def test_odd_extension_rows(n):
+    d = len(n)
+    h = 1.0 / (max(n) + 1)
+    op, p = OPlan(d, n, h, 1.3), Plan(d, n, h, 1.3)
+    r = np.random.default_rng(8).standard_normal(n).astype(np.float32).astype(np.float64)
+    for shift, scale in ((0.0, 1.0), (1.0, 1e-3)):
+        ref = oprec.solve_box(op, r, shift, scale)
+        for dtype, tol in ((torch.float64, 1e-11), (torch.float32, 2e-5)):
+            z = p.precond(dev(r, dtype), shift=shift, scale=scale).cpu().numpy()
+            assert rel(z, ref) <= tol, (dtype, rel(z, ref))
