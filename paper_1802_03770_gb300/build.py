@@ -20,12 +20,13 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # code, device-linked together (each body function is register-allocated on
 # its own; 80 registers keep three 256-thread CTAs per SM)
 RDC = ["-rdc=true", "-maxrregcount=80"]
-# (source, extra flags, object): ops.cu and batch.cu are compiled in two
-# halves each (FP32 and FP64 instantiations) so that their largest parts run
-# in parallel
+# (source, extra flags, object): ops.cu and batch.cu are compiled in parts
+# (FP32 and FP64, the preconditioner passes apart) so that their largest parts
+# run in parallel
 CUDA_SOURCES = [("ops.cu", ["-DFL_OPS_PART=1"], "ops_f32.o"), ("ops.cu", ["-DFL_OPS_PART=2"], "ops_f64.o"),
+                ("ops.cu", ["-DFL_OPS_PART=3"], "ops_prec_f32.o"), ("ops.cu", ["-DFL_OPS_PART=4"], "ops_prec_f64.o"),
                 ("plan.cu", [], "plan.o"), ("batch.cu", ["-DFL_BATCH_PART=1"], "batch_f32.o"),
-                ("batch.cu", ["-DFL_BATCH_PART=2"], "batch_f64.o"), ("unet.cu", [], "unet.o"),
+                ("batch.cu", ["-DFL_BATCH_PART=2"], "batch_f64.o"), ("batch.cu", ["-DFL_BATCH_PART=3"], "batch_prec_f32.o"), ("unet.cu", [], "unet.o"),
                 ("learned.cu", [], "learned.o"), ("domain.cu", [], "domain.o"),
                 ("rows_w8.cu", [], "rows_w8.o"),
                 ("persist.cu", RDC, "persist.o"), ("persist_body.cu", RDC, "persist_body.o")]

@@ -91,9 +91,10 @@ __global__ void __launch_bounds__(kVecThreads) kb_noprec_update(const BVecArgs<T
   body_b_noprec<T>(args[i], blockIdx.x - off[i], off[i + 1] - off[i]);
 }
 
-// This file is compiled in two halves (FL_BATCH_PART 1: the FP32 passes and
-// the precision-free kernels, 2: the FP64 passes) so that its template
-// instantiations compile in parallel; without FL_BATCH_PART it holds both.
+// This file is compiled in three parts (FL_BATCH_PART 1: the FP32 apply passes
+// and the precision-free kernels, 2: the FP64 apply passes, 3: the FP32
+// preconditioner passes and CG vector kernels) so that its template
+// instantiations compile in parallel; without FL_BATCH_PART it holds all.
 #if !defined(FL_BATCH_PART) || FL_BATCH_PART == 1
 // FP64 right-hand side to the FP32 inner right-hand side (masked), with
 // partials of ||b||^2 -- the residual of the zero initial guess.
@@ -156,6 +157,53 @@ __global__ void kb_sum(const BScalarArgs* __restrict__ args, double* out, int np
 
 // --- launchers --------------------------------------------------------------
 
+// The preconditioner's passes and the CG vector kernels (FP32).
+cudaError_t launch_batched_prec(const BatchPass& bp, cudaStream_t s);
+#if !defined(FL_BATCH_PART) || FL_BATCH_PART == 3
+cudaError_t launch_batched_prec(const BatchPass& bp, cudaStream_t s) {
+  typedef float T;
+  typedef Cfg<T> K;
+  switch (bp.kind) {
+    case BK_DST_ROWS:
+      if (bp.w8) {
+        FL_KERNEL("b_dst_rows<f32>", s,
+                  pdl_launch(kb_dst_rows<T, kRowsW8Threads, 8>, bp.blocks, kRowsW8Threads, bp.smem, s,
+                             (const DstRowsArgs<T>*)bp.args, bp.off, bp.gx, bp.nprob));
+        break;
+      }
+      FL_KERNEL("b_dst_rows<f32>", s,
+                pdl_launch(kb_dst_rows<T, K::RT, K::RV>, bp.blocks, K::RT, bp.smem, s,
+                           (const DstRowsArgs<T>*)bp.args, bp.off, bp.gx, bp.nprob));
+      break;
+    case BK_DST_COLS:
+      FL_KERNEL("b_dst_cols<f32>", s,
+                pdl_launch(kb_dst_cols<T, K::CT, K::CV>, bp.blocks, K::CT, bp.smem, s,
+                           (const DstColsArgs<T>*)bp.args, bp.off, bp.gx, bp.nprob));
+      break;
+    case BK_TRI_COLS:
+      FL_KERNEL("b_tri_cols<f32>", s,
+                pdl_launch(kb_tri_cols<T>, bp.blocks, kTriCols<T> * kTriSeg, 0, s,
+                           (const TriArgs<T>*)bp.args, bp.off, bp.nprob));
+      break;
+    case BK_CG_START:
+      FL_KERNEL("b_cg_start<f32>", s,
+                pdl_launch(kb_cg_start<T>, bp.blocks, kVecThreads, 0, s,
+                           (const BVecArgs<T>*)bp.args, bp.off,
+                           bp.nprob));
+      break;
+    case BK_NOPREC:
+      FL_KERNEL("b_noprec_update<f32>", s,
+                pdl_launch(kb_noprec_update<T>, bp.blocks, kVecThreads, 0, s,
+                           (const BVecArgs<T>*)bp.args, bp.off,
+                           bp.nprob));
+      break;
+    default:
+      return cudaErrorInvalidValue;
+  }
+  return launch_status();
+}
+#endif
+
 template <typename T>
 cudaError_t launch_batched(const BatchPass& bp, cudaStream_t s) {
   typedef Cfg<T> K;
@@ -193,40 +241,13 @@ cudaError_t launch_batched(const BatchPass& bp, cudaStream_t s) {
                            (const RowsInvArgs<T>*)bp.args, bp.off, bp.gx, bp.nprob));
       break;
     case BK_DST_ROWS:
-      if constexpr (sizeof(T) == 4) {
-        if (bp.w8) {
-          FL_KERNEL("b_dst_rows<f32>", s,
-                    pdl_launch(kb_dst_rows<T, kRowsW8Threads, 8>, bp.blocks, kRowsW8Threads, bp.smem, s,
-                               (const DstRowsArgs<T>*)bp.args, bp.off, bp.gx, bp.nprob));
-          break;
-        }
-      }
-      FL_KERNEL(sizeof(T) == 4 ? "b_dst_rows<f32>" : "b_dst_rows<f64>", s,
-                pdl_launch(kb_dst_rows<T, K::RT, K::RV>, bp.blocks, K::RT, bp.smem, s,
-                           (const DstRowsArgs<T>*)bp.args, bp.off, bp.gx, bp.nprob));
-      break;
     case BK_DST_COLS:
-      FL_KERNEL(sizeof(T) == 4 ? "b_dst_cols<f32>" : "b_dst_cols<f64>", s,
-                pdl_launch(kb_dst_cols<T, K::CT, K::CV>, bp.blocks, K::CT, bp.smem, s,
-                           (const DstColsArgs<T>*)bp.args, bp.off, bp.gx, bp.nprob));
-      break;
     case BK_TRI_COLS:
-      FL_KERNEL(sizeof(T) == 4 ? "b_tri_cols<f32>" : "b_tri_cols<f64>", s,
-                pdl_launch(kb_tri_cols<T>, bp.blocks, kTriCols<T> * kTriSeg, 0, s,
-                           (const TriArgs<T>*)bp.args, bp.off, bp.nprob));
-      break;
     case BK_CG_START:
-      FL_KERNEL(sizeof(T) == 4 ? "b_cg_start<f32>" : "b_cg_start<f64>", s,
-                pdl_launch(kb_cg_start<T>, bp.blocks, kVecThreads, 0, s,
-                           (const BVecArgs<T>*)bp.args, bp.off,
-                           bp.nprob));
-      break;
     case BK_NOPREC:
-      FL_KERNEL(sizeof(T) == 4 ? "b_noprec_update<f32>" : "b_noprec_update<f64>", s,
-                pdl_launch(kb_noprec_update<T>, bp.blocks, kVecThreads, 0, s,
-                           (const BVecArgs<T>*)bp.args, bp.off,
-                           bp.nprob));
-      break;
+      // FP32 only: FP64 batches run the residual's applies
+      if constexpr (sizeof(T) == 4) return launch_batched_prec(bp, s);
+      return cudaErrorInvalidValue;
     default:
       return cudaErrorInvalidValue;
   }
@@ -263,23 +284,33 @@ static cudaError_t set_batched_smem(const void* f) {
 }
 
 cudaError_t configure_batched_kernels_f64();
+cudaError_t configure_batched_prec();
 
 #if !defined(FL_BATCH_PART) || FL_BATCH_PART == 1
 cudaError_t configure_batched_kernels() {
   cudaError_t e = configure_batched_kernels_f64();
+  if (e == cudaSuccess) e = configure_batched_prec();
   for (const void* f : {reinterpret_cast<const void*>(&kb_rows_fwd<float, Cfg<float>::RT, Cfg<float>::RV>),
                         reinterpret_cast<const void*>(&kb_rows_inv<float, Cfg<float>::RT, Cfg<float>::RV>),
                         reinterpret_cast<const void*>(&kb_cols<float, Cfg<float>::CT, Cfg<float>::CV>),
-                        reinterpret_cast<const void*>(&kb_dst_rows<float, Cfg<float>::RT, Cfg<float>::RV>),
-                        reinterpret_cast<const void*>(&kb_dst_cols<float, Cfg<float>::CT, Cfg<float>::CV>),
                         reinterpret_cast<const void*>(&kb_rows_fwd<float, kRowsW8Threads, 8>),
-                        reinterpret_cast<const void*>(&kb_rows_inv<float, kRowsW8Threads, 8>),
-                        reinterpret_cast<const void*>(&kb_dst_rows<float, kRowsW8Threads, 8>)})
+                        reinterpret_cast<const void*>(&kb_rows_inv<float, kRowsW8Threads, 8>)})
     if (e == cudaSuccess) e = set_batched_smem(f);
   return e;
 }
 
 template cudaError_t launch_batched<float>(const BatchPass&, cudaStream_t);
+#endif
+
+#if !defined(FL_BATCH_PART) || FL_BATCH_PART == 3
+cudaError_t configure_batched_prec() {
+  cudaError_t e = cudaSuccess;
+  for (const void* f : {reinterpret_cast<const void*>(&kb_dst_rows<float, Cfg<float>::RT, Cfg<float>::RV>),
+                        reinterpret_cast<const void*>(&kb_dst_cols<float, Cfg<float>::CT, Cfg<float>::CV>),
+                        reinterpret_cast<const void*>(&kb_dst_rows<float, kRowsW8Threads, 8>)})
+    if (e == cudaSuccess) e = set_batched_smem(f);
+  return e;
+}
 #endif
 
 #if !defined(FL_BATCH_PART) || FL_BATCH_PART == 2

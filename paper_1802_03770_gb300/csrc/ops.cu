@@ -1,9 +1,10 @@
 // Kernel launchers: the operator apply chain, the preconditioner chain, CG
 // vector and scalar kernels, and the plan-time symbol build.
 //
-// The file is compiled twice (in parallel): FL_OPS_PART=1 holds the FP32
+// The file is compiled four times (in parallel): FL_OPS_PART=1 holds the FP32
 // instantiations and the precision-free kernels, FL_OPS_PART=2 the FP64
-// instantiations and the plan-time symbol build.
+// instantiations and the plan-time symbol build, 3 and 4 the preconditioner
+// passes in FP32 and FP64.
 #include <algorithm>
 
 #ifndef FL_OPS_PART
@@ -350,25 +351,57 @@ static cudaError_t set_smem(const void* f) {
 
 #if FL_OPS_PART == 1
 cudaError_t configure_kernels_f64();
+cudaError_t configure_precond_f32();
+cudaError_t configure_precond_f64();
 
 cudaError_t configure_kernels() {
   cudaError_t e = configure_kernels_f64();
+  if (e == cudaSuccess) e = configure_precond_f32();
+  if (e == cudaSuccess) e = configure_precond_f64();
   if (e == cudaSuccess) e = configure_rows_w8();
 #define FL_SET(...)                                                         \
   if (e == cudaSuccess) e = set_smem(reinterpret_cast<const void*>(&__VA_ARGS__));
   FL_SET(k_rows_fwd<float, Cfg<float>::RT, Cfg<float>::RV>);
   FL_SET(k_rows_inv<float, Cfg<float>::RT, Cfg<float>::RV>);
   FL_SET(k_cols<float, Cfg<float>::CT, Cfg<float>::CV>);
-  FL_SET(k_dst_rows<float, Cfg<float>::RT, Cfg<float>::RV>);
-  FL_SET(k_dst_rows_odd<float, Cfg<float>::RT, Cfg<float>::RV>);
-  FL_SET(k_dst_cols<float, Cfg<float>::CT, Cfg<float>::CV>);
   FL_SET(k_cols<float, Cfg<float>::CT / 2, Cfg<float>::CV>);
-  FL_SET(k_dst_cols<float, Cfg<float>::CT / 2, Cfg<float>::CV>);
   // the wide instantiations of the longest lines
   FL_SET(k_rows_fwd<float, 256, 16, 12>);
   FL_SET(k_rows_fwd<float, 512, 16, 13>);
   FL_SET(k_rows_inv<float, 256, 16, 12>);
   FL_SET(k_rows_inv<float, 512, 16, 13>);
+#undef FL_SET
+  return e;
+}
+#elif FL_OPS_PART == 2
+cudaError_t configure_kernels_f64() {
+  cudaError_t e = cudaSuccess;
+#define FL_SET(...)                                                         \
+  if (e == cudaSuccess) e = set_smem(reinterpret_cast<const void*>(&__VA_ARGS__));
+  FL_SET(k_rows_fwd<double, Cfg<double>::RT, Cfg<double>::RV>);
+  FL_SET(k_rows_inv<double, Cfg<double>::RT, Cfg<double>::RV>);
+  FL_SET(k_cols<double, Cfg<double>::CT, Cfg<double>::CV>);
+  FL_SET(k_rows_fwd<double, 512, 8, 12>);
+  FL_SET(k_rows_inv<double, 512, 8, 12>);
+  FL_SET(k_rows_fwd<double, 1024, 8, 13>);
+  FL_SET(k_rows_inv<double, 1024, 8, 13>);
+  FL_SET(k_cols<double, 1024, 8, 13>);
+  FL_SET(k_rows_c2c<kSymT, kSymV>);
+  FL_SET(k_rows_c2c<2 * kSymT, kSymV>);
+  FL_SET(k_cols_c2c<kSymT, kSymV>);
+  FL_SET(k_cols_c2c<2 * kSymT, kSymV, 13>);
+#undef FL_SET
+  return e;
+}
+#elif FL_OPS_PART == 3
+cudaError_t configure_precond_f32() {
+  cudaError_t e = cudaSuccess;
+#define FL_SET(...)                                                         \
+  if (e == cudaSuccess) e = set_smem(reinterpret_cast<const void*>(&__VA_ARGS__));
+  FL_SET(k_dst_rows<float, Cfg<float>::RT, Cfg<float>::RV>);
+  FL_SET(k_dst_rows_odd<float, Cfg<float>::RT, Cfg<float>::RV>);
+  FL_SET(k_dst_cols<float, Cfg<float>::CT, Cfg<float>::CV>);
+  FL_SET(k_dst_cols<float, Cfg<float>::CT / 2, Cfg<float>::CV>);
   FL_SET(k_dst_rows<float, 256, 16, 12>);
   FL_SET(k_dst_rows_odd<float, 256, 16, 12>);
   FL_SET(k_dst_rows<float, 512, 16, 13>);
@@ -377,30 +410,18 @@ cudaError_t configure_kernels() {
   return e;
 }
 #else
-cudaError_t configure_kernels_f64() {
+cudaError_t configure_precond_f64() {
   cudaError_t e = cudaSuccess;
 #define FL_SET(...)                                                         \
   if (e == cudaSuccess) e = set_smem(reinterpret_cast<const void*>(&__VA_ARGS__));
-  FL_SET(k_rows_fwd<double, Cfg<double>::RT, Cfg<double>::RV>);
-  FL_SET(k_rows_inv<double, Cfg<double>::RT, Cfg<double>::RV>);
-  FL_SET(k_cols<double, Cfg<double>::CT, Cfg<double>::CV>);
   FL_SET(k_dst_rows<double, Cfg<double>::RT, Cfg<double>::RV>);
   FL_SET(k_dst_rows_odd<double, Cfg<double>::RT, Cfg<double>::RV>);
   FL_SET(k_dst_cols<double, Cfg<double>::CT, Cfg<double>::CV>);
-  FL_SET(k_rows_fwd<double, 512, 8, 12>);
-  FL_SET(k_rows_inv<double, 512, 8, 12>);
   FL_SET(k_dst_rows<double, 512, 8, 12>);
   FL_SET(k_dst_rows_odd<double, 512, 8, 12>);
-  FL_SET(k_rows_fwd<double, 1024, 8, 13>);
-  FL_SET(k_rows_inv<double, 1024, 8, 13>);
   FL_SET(k_dst_rows<double, 1024, 8, 13>);
   FL_SET(k_dst_rows_odd<double, 1024, 8, 13>);
-  FL_SET(k_cols<double, 1024, 8, 13>);
   FL_SET(k_dst_cols<double, 1024, 8, 13>);
-  FL_SET(k_rows_c2c<kSymT, kSymV>);
-  FL_SET(k_rows_c2c<2 * kSymT, kSymV>);
-  FL_SET(k_cols_c2c<kSymT, kSymV>);
-  FL_SET(k_cols_c2c<2 * kSymT, kSymV, 13>);
 #undef FL_SET
   return e;
 }
@@ -711,7 +732,7 @@ cudaError_t launch_mask_copy_dot(long long N, cudaStream_t s, const T* src, cons
 }
 #if FL_OPS_PART == 1
 template cudaError_t launch_mask_copy_dot<float>(long long, cudaStream_t, const float*, const uint8_t*, float*, double*, int*);
-#else
+#elif FL_OPS_PART == 2
 template cudaError_t launch_mask_copy_dot<double>(long long, cudaStream_t, const double*, const uint8_t*, double*, double*, int*);
 #endif
 
@@ -849,23 +870,25 @@ template PrecChain<float> build_precond<float>(const Geo&, const Tables<float>&,
 template int apply_partials<float>(const Geo&);
 template int precond_partials<float>(const Geo&);
 template cudaError_t prepare_precond<float>(const Geo&, Tables<float>&, double, double, cudaStream_t);
-template cudaError_t launch_precond<float>(const Geo&, const Tables<float>&, cudaStream_t, const PrecIO<float>&);
 template cudaError_t launch_noprec_update<float>(long long, cudaStream_t, PcgState*, float*, float*, const float*, const float*, double*, int, int*);
 template cudaError_t launch_dot<float>(long long, cudaStream_t, const float*, const float*, double*, int*);
 template cudaError_t launch_copy_cast<float>(long long, cudaStream_t, const double*, float*);
 template cudaError_t launch_axpby<float>(long long, cudaStream_t, double, const float*, double, float*);
-#else
+#elif FL_OPS_PART == 2
 template cudaError_t launch_apply<double>(const Geo&, const Tables<double>&, cudaStream_t, const ApplyIO<double>&);
 template ApplyChain<double> build_apply<double>(const Geo&, const Tables<double>&, const ApplyIO<double>&);
 template PrecChain<double> build_precond<double>(const Geo&, const Tables<double>&, const PrecIO<double>&);
 template int apply_partials<double>(const Geo&);
 template int precond_partials<double>(const Geo&);
 template cudaError_t prepare_precond<double>(const Geo&, Tables<double>&, double, double, cudaStream_t);
-template cudaError_t launch_precond<double>(const Geo&, const Tables<double>&, cudaStream_t, const PrecIO<double>&);
 template cudaError_t launch_noprec_update<double>(long long, cudaStream_t, PcgState*, double*, double*, const double*, const double*, double*, int, int*);
 template cudaError_t launch_dot<double>(long long, cudaStream_t, const double*, const double*, double*, int*);
 template cudaError_t launch_copy_cast<double>(long long, cudaStream_t, const double*, double*);
 template cudaError_t launch_axpby<double>(long long, cudaStream_t, double, const double*, double, double*);
+#elif FL_OPS_PART == 3
+template cudaError_t launch_precond<float>(const Geo&, const Tables<float>&, cudaStream_t, const PrecIO<float>&);
+#else
+template cudaError_t launch_precond<double>(const Geo&, const Tables<double>&, cudaStream_t, const PrecIO<double>&);
 #endif
 
 }  // namespace fl
