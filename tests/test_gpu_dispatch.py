@@ -81,3 +81,13 @@ def test_odd_extension_rows(n):
         for dtype, tol in ((torch.float64, 1e-11), (torch.float32, 2e-5)):
             z = p.precond(dev(r, dtype), shift=shift, scale=scale).cpu().numpy()
             assert rel(z, ref) <= tol, (dtype, rel(z, ref))
+
+
+# iterations between reads of the device state: caps inside, at and past the captured graph's four
+@pytest.mark.parametrize("cap", [1, 3, 4, 5, 7, 8, 13, 40])
+def test_iteration_cap(cap):
+    n = (31, 40)
+    p = Plan(2, n, 1.0 / 41, 1.3)
+    b = dev(np.random.default_rng(9).standard_normal(n), torch.float64)
+    _, info = p.solve(b, tol=1e-300, maxit=cap, mode=0, raise_on_fail=False)
+    assert info["iterations"] == cap
