@@ -279,9 +279,22 @@ template <typename T> inline bool rows_w8(const Tables<T>& tb, int L, int ctas) 
 
 // Whether a DST along an axis takes the odd extension (its points n = 2^k - 1).
 inline bool dst_odd(const Geo& g, int axis) { return g.L[axis] == 2 * (g.n[axis] + 1); }
+// Whether an FP32 DST along an axis is Rader's convolution of half the length
+// (n + 1 an odd prime; lines of 16 points are the shortest), and the length of
+// the DST's transforms.
+template <typename T> inline bool dst_prime(const Geo& g, int axis) {
+  const int q = g.n[axis] + 1;
+  if (sizeof(T) != 4 || g.L[axis] < 32 || q % 2 == 0) return false;
+  for (int f = 3; f * f <= q; f += 2)
+    if (q % f == 0) return false;
+  return true;
+}
+template <typename T> inline int dst_len(const Geo& g, int axis) {
+  return dst_prime<T>(g, axis) ? g.L[axis] / 2 : g.L[axis];
+}
 // rows of the last axis per CTA of a DST row pass (rt: threads, 0: the Cfg shape)
 template <typename T> inline int dst_row_lines(const Geo& g, int rt) {
-  return row_lines_at<T>(g.L[g.d - 1], rt) * (dst_odd(g, g.d - 1) ? 2 : 1);
+  return row_lines_at<T>(dst_len<T>(g, g.d - 1), rt) * (dst_odd(g, g.d - 1) ? 2 : 1);
 }
 
 template <typename T>

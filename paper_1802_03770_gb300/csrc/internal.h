@@ -49,6 +49,9 @@ struct Tables {
   FxW* fbhat[3] = {nullptr, nullptr, nullptr};   // / 2^bexp
   int bexp[3] = {0, 0, 0};
   C* ptw[3] = {nullptr, nullptr, nullptr};     // FP32: twiddle tables of the strided passes' stages
+  // FP32 axes with n + 1 prime: orders and stage twiddles of Rader's convolution (dst_prime)
+  short* perm[3] = {nullptr, nullptr, nullptr};
+  C* dptw[3] = {nullptr, nullptr, nullptr};
   // FP32 DST tables
   C* chirp[3] = {nullptr, nullptr, nullptr};
   C* bhat[3] = {nullptr, nullptr, nullptr};   // by place of the 16-value stage plan

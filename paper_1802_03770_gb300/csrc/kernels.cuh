@@ -737,6 +737,9 @@ struct DstRowsArgs {
   const uint8_t* mask_in;
   const uint8_t* mask_out;
   int odd;                 // n + 1 = L/2: two rows per complex line (body_dst_rows_odd_at)
+  // FP32, n + 1 prime: the orders of Rader's convolution (body_dst_rows_prime_at);
+  // lg and bhat are then that convolution's
+  const short* perm;
   // nullable (last pass): added to the transformed value before the output
   // mask, out = mask_out ? (B^{-1} in + add) : 0 (the second half of the
   // capacitance solve on an occluded domain)
@@ -748,6 +751,14 @@ struct DstRowsArgs {
   const FxW* fbhat;
   int bexp;
 };
+
+// u_j + i v_j of the prime-length sines from x_j and x_{p-j} (for j > M the
+// signs are those of the odd continuation)
+template <typename C, typename T>
+__device__ __forceinline__ C rader_fold(T xj, T xm, int j) {
+  const T s = xj + xm;
+  return cmake<C>(xj - xm, (j & 1) ? s : -s);
+}
 
 // The partial sums of a DST row pass, and in its last CTA the CG step.
 template <typename T>
@@ -969,41 +980,188 @@ __device__ __forceinline__ void body_dst_rows_odd_fixed(const DstRowsArgs<T>& a,
   }
 }
 
+// The same where p = n + 1 is an odd prime (192, 256, 640, 768 points), by a
+// convolution of half the length.  With u_j = x_j - x_{p-j}, v_j = (-1)^{j+1}
+// (x_j + x_{p-j}) and M = n/2, the sines are S_{2m} = sum_{j=1..M} u_j
+// sin(2 pi jm/p) and S_{p-2m} the same of v, and for a generator g of the
+// residues modulo p (Rader, Proc. IEEE 56, 1968) the substitution j = g^a, m =
+// g^-b makes both the convolution with the real sequence sin(2 pi g^-d / p): one
+// complex transform pair of length L >= 2M - 1 carries u + i v, no chirp.  perm:
+// g^a mod p for a < M, then for b < M the index 2m (m = +-g^-b in 1..M),
+// negative where the sign is.  The rows go through shared memory in their own
+// order, so global reads and writes are one contiguous run per CTA.
+// @PRIME@
+template <typename T, int THREADS, int VPT, int LGLO, int LGHI>
+__device__ __forceinline__ void body_dst_rows_prime_at(const DstRowsArgs<T>& a, int bx, const int lg) {
+  typedef typename Cplx<T>::type C;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const SBuf<C> buf{reinterpret_cast<C*>(smem_raw)};
+  __shared__ double red[32];
+  if (a.st && a.st->done) return;
+  const int L = 1 << lg;
+  const int ls = L;
+  const int NL = (VPT * THREADS) / L;
+  const int row0 = bx * NL;
+  const int nl = min(NL, a.rows - row0);
+  const int n = a.n, M = n >> 1;
+  T* xs = reinterpret_cast<T*>(smem_raw + sbuf_elems((long long)NL * L) * sizeof(C));   // the CTA's rows
+  const size_t base = (size_t)row0 * n;
+  const int tot = nl * n;
+  constexpr int U = 4;   // elements in flight per thread
+  DotAcc<T> rr, dp;
+  const bool update = a.pre == DPRE_UPDATE;
+  const T al = update ? (T)a.st->alpha : (T)0;
+  for (int e0 = threadIdx.x; e0 < tot; e0 += THREADS * U) {
+    T xo[U], ro[U], po[U], qo[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int e = e0 + u * THREADS;
+      const size_t idx = base + e;
+      xo[u] = ro[u] = po[u] = qo[u] = (T)0;
+      if (e < tot) {
+        if (update) {
+          xo[u] = a.x[idx];
+          ro[u] = a.r[idx];
+          po[u] = a.p[idx];
+          qo[u] = a.q[idx];
+        } else if (!a.mask_in || a.mask_in[idx]) {
+          ro[u] = a.in[idx];
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int e = e0 + u * THREADS;
+      if (e < tot) {
+        if (update) {
+          const size_t idx = base + e;
+          ro[u] -= al * qo[u];
+          a.x[idx] = xo[u] + al * po[u];
+          a.r[idx] = ro[u];
+          rr.add(ro[u] * ro[u]);
+        }
+        xs[e] = ro[u];
+      }
+    }
+  }
+  __syncthreads();
+  {
+    const short* FL_RESTRICT perm = a.perm;
+    const C* FL_RESTRICT bhat = VPT == 8 ? a.bhat8 : a.bhat;
+    const T post = (T)a.post;
+    auto ld = [=](int q, int n0, auto lgs, auto cnt, C* v) {
+      constexpr int N = decltype(cnt)::v, LGS = decltype(lgs)::v;
+      const T* x = xs + q * n;
+#pragma unroll
+      for (int r = 0; r < N; ++r) {
+        const int i = n0 + (r << LGS);
+        v[r] = cmake<C>((T)0, (T)0);
+        if (i < M) {
+          const int j = perm[i];
+          v[r] = rader_fold<C>(x[j - 1], x[n - j], j);
+        }
+      }
+    };
+    auto mid = [=](int, int, int p, C v) -> C { return cswap(cmul(v, bhat[p])); };
+    // every row was read before the first stage's barrier (one thread holds
+    // the whole row where there is one stage only)
+    auto out = [=](int q, int k, C v) {
+      if (k < M) {
+        const int m = perm[M + k], i = abs(m);
+        const T s = m < 0 ? -post : post;
+        xs[q * n + i - 1] = v.y * s;   // v is swapped
+        xs[q * n + n - i] = v.x * s;
+      }
+    };
+    fft_places<PLACE_CONV, VPT, false, LGHI, LGLO, false>(buf, lg, ls, 0, nl, a.tw, a.lgmax, ld, mid, out);
+  }
+  __syncthreads();
+  for (int e0 = threadIdx.x; e0 < tot; e0 += THREADS * U) {
+    T ad[U], dw[U];
+    bool in[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int e = e0 + u * THREADS;
+      const size_t idx = base + e;
+      in[u] = e < tot && (!a.mask_out || a.mask_out[idx]);
+      ad[u] = in[u] && a.add ? a.add[idx] : (T)0;
+      dw[u] = e < tot && a.dotw ? a.dotw[idx] : (T)0;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int e = e0 + u * THREADS;
+      if (e < tot) {
+        const T o = in[u] ? xs[e] + ad[u] : (T)0;
+        a.out[base + e] = o;
+        if (a.dotw) dp.add(o * dw[u]);
+      }
+    }
+  }
+  dst_rows_finish(a, bx, rr, dp, red);
+}
+
+template <typename T, int THREADS, int VPT, int LGLO, int LGHI, int LG>
+__device__ __forceinline__ void body_dst_rows_prime_fixed(const DstRowsArgs<T>& a, int bx) {
+  if constexpr (LG <= LGHI) {
+    if (a.lg == LG) {
+      body_dst_rows_prime_at<T, THREADS, VPT, LGLO, LGHI>(a, bx, LG);
+      return;
+    }
+    body_dst_rows_prime_fixed<T, THREADS, VPT, LGLO, LGHI, LG + 1>(a, bx);
+  } else if constexpr (LGLO < kFixedLgMin) {
+    body_dst_rows_prime_at<T, THREADS, VPT, LGLO, LGHI>(a, bx, a.lg);
+  }
+}
+
 // FP64: fixed-point lines (fix_passes.cuh)
 template <int THREADS, int VPT, int LGLO, int LGHI>
 __device__ __forceinline__ void fx_body_dst_rows(const DstRowsArgs<double>& a, int bx);
 template <int THREADS, int VPT, int LGLO, int LGHI>
 __device__ __forceinline__ void fx_body_dst_rows_odd(const DstRowsArgs<double>& a, int bx);
 
-// either by a chirp convolution per row (ODD = false) or for a.odd
-template <typename T, int THREADS, int VPT, bool ODD, int LGLO = 4, int LGHI = clog2(THREADS * VPT)>
+// by a chirp convolution per row, for a.odd or (FP32) for a.perm
+enum { DST_CHIRP = 0, DST_ODD = 1, DST_PRIME = 2 };
+template <typename T, int THREADS, int VPT, int FORM, int LGLO = 4, int LGHI = clog2(THREADS * VPT)>
 __device__ __forceinline__ void body_dst_rows_as(const DstRowsArgs<T>& a, int bx, int by) {
   constexpr int LG0 = LGLO > kFixedLgMin ? LGLO : kFixedLgMin;
   if constexpr (sizeof(T) == 8) {
-    if constexpr (ODD) fx_body_dst_rows_odd<THREADS, VPT, LGLO, LGHI>(a, bx);
+    if constexpr (FORM == DST_ODD) fx_body_dst_rows_odd<THREADS, VPT, LGLO, LGHI>(a, bx);
     else fx_body_dst_rows<THREADS, VPT, LGLO, LGHI>(a, bx);
   } else {
-    if constexpr (ODD) body_dst_rows_odd_fixed<T, THREADS, VPT, LGLO, LGHI, LG0>(a, bx);
+    if constexpr (FORM == DST_ODD) body_dst_rows_odd_fixed<T, THREADS, VPT, LGLO, LGHI, LG0>(a, bx);
+    else if constexpr (FORM == DST_PRIME) body_dst_rows_prime_fixed<T, THREADS, VPT, LGLO, LGHI, LG0>(a, bx);
     else body_dst_rows_fixed<T, THREADS, VPT, LGLO, LGHI, LG0>(a, bx, by);
   }
 }
 
 template <typename T, int THREADS, int VPT, int LGLO = 4, int LGHI = clog2(THREADS * VPT)>
 __device__ __forceinline__ void body_dst_rows(const DstRowsArgs<T>& a, int bx, int by) {
-  if (a.odd) body_dst_rows_as<T, THREADS, VPT, true, LGLO, LGHI>(a, bx, by);
-  else body_dst_rows_as<T, THREADS, VPT, false, LGLO, LGHI>(a, bx, by);
+  if constexpr (sizeof(T) == 4) {
+    if (a.perm) {
+      body_dst_rows_as<T, THREADS, VPT, DST_PRIME, LGLO, LGHI>(a, bx, by);
+      return;
+    }
+  }
+  if (a.odd) body_dst_rows_as<T, THREADS, VPT, DST_ODD, LGLO, LGHI>(a, bx, by);
+  else body_dst_rows_as<T, THREADS, VPT, DST_CHIRP, LGLO, LGHI>(a, bx, by);
 }
 
 template <typename T, int THREADS, int VPT, int LGLO = 4>
 __global__ void __launch_bounds__(THREADS, min_ctas<T>(THREADS, LGLO)) k_dst_rows(DstRowsArgs<T> a) {
   pdl_wait();
-  body_dst_rows_as<T, THREADS, VPT, false, LGLO>(a, blockIdx.x, blockIdx.y);
+  body_dst_rows_as<T, THREADS, VPT, DST_CHIRP, LGLO>(a, blockIdx.x, blockIdx.y);
   pdl_release();
 }
 template <typename T, int THREADS, int VPT, int LGLO = 4>
 __global__ void __launch_bounds__(THREADS, min_ctas<T>(THREADS, LGLO)) k_dst_rows_odd(DstRowsArgs<T> a) {
   pdl_wait();
-  body_dst_rows_as<T, THREADS, VPT, true, LGLO>(a, blockIdx.x, blockIdx.y);
+  body_dst_rows_as<T, THREADS, VPT, DST_ODD, LGLO>(a, blockIdx.x, blockIdx.y);
+  pdl_release();
+}
+template <typename T, int THREADS, int VPT, int LGLO = 4>
+__global__ void __launch_bounds__(THREADS, min_ctas<T>(THREADS, LGLO)) k_dst_rows_prime(DstRowsArgs<T> a) {
+  pdl_wait();
+  body_dst_rows_as<T, THREADS, VPT, DST_PRIME, LGLO>(a, blockIdx.x, blockIdx.y);
   pdl_release();
 }
 
@@ -1022,13 +1180,14 @@ struct DstColsArgs {
   int n, ncols, lg, lgmax;
   long long ostride, lstride;
   int ltx;
+  const short* perm;       // as in DstRowsArgs
   const FxW* ftw;          // FP64: as in DstRowsArgs
   const FxW* fchirp;
   const FxW* fbhat;
   int bexp;
 };
 
-template <typename T, int THREADS, int VPT, int LGLO, int LGHI>
+template <typename T, int THREADS, int VPT, bool PRIME, int LGLO, int LGHI>
 __device__ __forceinline__ void body_dst_cols_at(const DstColsArgs<T>& a, int c0, int by, const int lg,
                                                  const int ltx) {
   typedef typename Cplx<T>::type C;
@@ -1048,8 +1207,26 @@ __device__ __forceinline__ void body_dst_cols_at(const DstColsArgs<T>& a, int c0
   const C* FL_RESTRICT chirp = a.chirp;
   const C* FL_RESTRICT bhat = a.bhat;
   const T post = (T)a.post;
+  const short* FL_RESTRICT perm = a.perm;
+  const int M = n >> 1;
   auto ld = [=](int c, int n0, auto lgs, auto cnt, C* v) {
     constexpr int N = decltype(cnt)::v, LGS = decltype(lgs)::v;
+    if constexpr (PRIME) {
+      // both rows of a fold once, each a contiguous run of the tile's columns
+      T x[N], y[N];
+      int j[N];
+#pragma unroll
+      for (int r = 0; r < N; ++r) {
+        const int i = n0 + (r << LGS);
+        j[r] = i < M ? perm[i] : 0;
+        const bool in = c < ncol && i < M;
+        x[r] = in ? base[(size_t)(j[r] - 1) * lstride + c] : (T)0;
+        y[r] = in ? base[(size_t)(n - j[r]) * lstride + c] : (T)0;
+      }
+#pragma unroll
+      for (int r = 0; r < N; ++r) v[r] = rader_fold<C>(x[r], y[r], j[r]);
+      return;
+    }
     T x[N];
 #pragma unroll
     for (int r = 0; r < N; ++r) {
@@ -1064,7 +1241,14 @@ __device__ __forceinline__ void body_dst_cols_at(const DstColsArgs<T>& a, int c0
   };
   auto mid = [=](int c, int, int p, C v) -> C { return cswap(cmul(v, bhat[p])); };
   auto out = [=](int c, int k, C v) {
-    if (c < ncol && k < n) {
+    if constexpr (PRIME) {
+      if (c < ncol && k < M) {
+        const int m = perm[M + k], i = abs(m);
+        const T s = m < 0 ? -post : post;
+        base[(size_t)(i - 1) * lstride + c] = v.y * s;   // v is swapped
+        base[(size_t)(n - i) * lstride + c] = v.x * s;
+      }
+    } else if (c < ncol && k < n) {
       const C w = chirp[k];   // v is swapped
       base[(size_t)k * lstride + c] = (w.x * v.x + w.y * v.y) * post;
     }
@@ -1072,17 +1256,17 @@ __device__ __forceinline__ void body_dst_cols_at(const DstColsArgs<T>& a, int c0
   fft_places<PLACE_CONV, VPT, true, LGHI, LGLO, true>(buf, lg, 0, ltx, TX, stw, lg, ld, mid, out);
 }
 
-template <typename T, int THREADS, int VPT, int LGLO, int LGHI, int LG>
+template <typename T, int THREADS, int VPT, bool PRIME, int LGLO, int LGHI, int LG>
 __device__ __forceinline__ void body_dst_cols_fixed(const DstColsArgs<T>& a, int bx, int by) {
   if constexpr (LG <= LGHI) {
     constexpr int W = widest_ltx(THREADS, VPT, LG);
     if (a.lg == LG && a.ltx == W && ((bx + 1) << W) <= a.ncols) {
-      body_dst_cols_at<T, THREADS, VPT, LGLO, LGHI>(a, bx << W, by, LG, W);
+      body_dst_cols_at<T, THREADS, VPT, PRIME, LGLO, LGHI>(a, bx << W, by, LG, W);
       return;
     }
-    body_dst_cols_fixed<T, THREADS, VPT, LGLO, LGHI, LG + 1>(a, bx, by);
+    body_dst_cols_fixed<T, THREADS, VPT, PRIME, LGLO, LGHI, LG + 1>(a, bx, by);
   } else {
-    body_dst_cols_at<T, THREADS, VPT, LGLO, LGHI>(a, bx << a.ltx, by, a.lg, block_ltx(a.ltx, bx, a.ncols));
+    body_dst_cols_at<T, THREADS, VPT, PRIME, LGLO, LGHI>(a, bx << a.ltx, by, a.lg, block_ltx(a.ltx, bx, a.ncols));
   }
 }
 
@@ -1090,16 +1274,34 @@ __device__ __forceinline__ void body_dst_cols_fixed(const DstColsArgs<T>& a, int
 template <int THREADS, int VPT, int LGLO, int LGHI>
 __device__ __forceinline__ void fx_body_dst_cols(const DstColsArgs<double>& a, int bx, int by);
 
+template <typename T, int THREADS, int VPT, bool PRIME, int LGLO = 4, int LGHI = clog2(THREADS * VPT)>
+__device__ __forceinline__ void body_dst_cols_as(const DstColsArgs<T>& a, int bx, int by) {
+  if constexpr (sizeof(T) == 8) fx_body_dst_cols<THREADS, VPT, LGLO, LGHI>(a, bx, by);
+  else
+    body_dst_cols_fixed<T, THREADS, VPT, PRIME, LGLO, LGHI, (LGLO > kFixedLgMin ? LGLO : kFixedLgMin)>(a, bx, by);
+}
+
 template <typename T, int THREADS, int VPT, int LGLO = 4, int LGHI = clog2(THREADS * VPT)>
 __device__ __forceinline__ void body_dst_cols(const DstColsArgs<T>& a, int bx, int by) {
-  if constexpr (sizeof(T) == 8) fx_body_dst_cols<THREADS, VPT, LGLO, LGHI>(a, bx, by);
-  else body_dst_cols_fixed<T, THREADS, VPT, LGLO, LGHI, (LGLO > kFixedLgMin ? LGLO : kFixedLgMin)>(a, bx, by);
+  if constexpr (sizeof(T) == 4) {
+    if (a.perm) {
+      body_dst_cols_as<T, THREADS, VPT, true, LGLO, LGHI>(a, bx, by);
+      return;
+    }
+  }
+  body_dst_cols_as<T, THREADS, VPT, false, LGLO, LGHI>(a, bx, by);
 }
 
 template <typename T, int THREADS, int VPT, int LGLO = 4>
 __global__ void __launch_bounds__(THREADS, min_ctas<T>(THREADS, LGLO)) k_dst_cols(DstColsArgs<T> a) {
   pdl_wait();
-  body_dst_cols<T, THREADS, VPT, LGLO>(a, blockIdx.x, blockIdx.y);
+  body_dst_cols_as<T, THREADS, VPT, false, LGLO>(a, blockIdx.x, blockIdx.y);
+  pdl_release();
+}
+template <typename T, int THREADS, int VPT, int LGLO = 4>
+__global__ void __launch_bounds__(THREADS, min_ctas<T>(THREADS, LGLO)) k_dst_cols_prime(DstColsArgs<T> a) {
+  pdl_wait();
+  body_dst_cols_as<T, THREADS, VPT, true, LGLO>(a, blockIdx.x, blockIdx.y);
   pdl_release();
 }
 

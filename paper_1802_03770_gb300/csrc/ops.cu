@@ -400,12 +400,17 @@ cudaError_t configure_precond_f32() {
   if (e == cudaSuccess) e = set_smem(reinterpret_cast<const void*>(&__VA_ARGS__));
   FL_SET(k_dst_rows<float, Cfg<float>::RT, Cfg<float>::RV>);
   FL_SET(k_dst_rows_odd<float, Cfg<float>::RT, Cfg<float>::RV>);
+  FL_SET(k_dst_rows_prime<float, Cfg<float>::RT, Cfg<float>::RV>);
   FL_SET(k_dst_cols<float, Cfg<float>::CT, Cfg<float>::CV>);
   FL_SET(k_dst_cols<float, Cfg<float>::CT / 2, Cfg<float>::CV>);
+  FL_SET(k_dst_cols_prime<float, Cfg<float>::CT, Cfg<float>::CV>);
+  FL_SET(k_dst_cols_prime<float, Cfg<float>::CT / 2, Cfg<float>::CV>);
   FL_SET(k_dst_rows<float, 256, 16, 12>);
   FL_SET(k_dst_rows_odd<float, 256, 16, 12>);
+  FL_SET(k_dst_rows_prime<float, 256, 16, 12>);
   FL_SET(k_dst_rows<float, 512, 16, 13>);
   FL_SET(k_dst_rows_odd<float, 512, 16, 13>);
+  FL_SET(k_dst_rows_prime<float, 512, 16, 13>);
 #undef FL_SET
   return e;
 }
@@ -564,12 +569,15 @@ template <typename T>
 PrecChain<T> build_precond(const Geo& g, const Tables<T>& tb, const PrecIO<T>& io) {
   PrecChain<T> ch;
   const int d = g.d;
-  const int nx = g.n[d - 1], Lx = g.L[d - 1];
+  const int nx = g.n[d - 1];
   const long long rows = g.N / nx;
   const int NL = dst_row_lines<T>(g, io.row_threads);
   const int odd = dst_odd(g, d - 1) ? 1 : 0;
   ch.row_blocks = (int)((rows + NL - 1) / NL);
-  ch.row_smem = smem_bytes<T>(row_lines_at<T>(Lx, io.row_threads), Lx);
+  const bool prime = dst_prime<T>(g, d - 1);
+  const int Ld = dst_len<T>(g, d - 1);
+  ch.row_smem = smem_bytes<T>(row_lines_at<T>(Ld, io.row_threads), Ld);
+  if (prime) ch.row_smem += (size_t)NL * nx * sizeof(T);   // the CTA's rows
   // DST normalisation of every axis but 0 (solved by the tridiagonal pass)
   double post = 1.0;
   for (int i = 1; i < d; ++i) post *= 2.0 / (g.n[i] + 1.0);
@@ -577,22 +585,25 @@ PrecChain<T> build_precond(const Geo& g, const Tables<T>& tb, const PrecIO<T>& i
     DstRowsArgs<T>& a = ch.first;
     a.in = io.in; a.out = tb.t; a.tw = tb.tw; a.chirp = tb.chirp[d - 1]; a.bhat = tb.bhat[d - 1]; a.bhat8 = tb.bhat8;
     a.ftw = tb.ftw; a.fchirp = tb.fchirp[d - 1]; a.fbhat = tb.fbhat[d - 1]; a.bexp = tb.bexp[d - 1]; a.odd = odd;
+    a.perm = prime ? tb.perm[d - 1] : nullptr;
     a.st = io.st; a.x = io.x; a.r = io.r; a.p = io.p; a.q = io.q;
     a.rr_part = io.rr_part;
     a.dotw = nullptr; a.dot_part = nullptr; a.post = 1.0;
-    a.rows = (int)rows; a.n = nx; a.lg = g.lg[d - 1]; a.lgmax = g.lgmax; a.pre = io.pre;
+    a.rows = (int)rows; a.n = nx; a.lg = ilog2i(Ld); a.lgmax = g.lgmax; a.pre = io.pre;
     a.fin = FIN_NONE; a.nparts = ch.row_blocks; a.rr_in = nullptr; a.rr_count = 0;
     a.mask_in = io.input_unmasked ? nullptr : io.mask; a.mask_out = nullptr; a.add = nullptr;
   }
   ch.ncols = 0;
   auto cols = [&](int axis, long long lstride, long long ostride, int nouter) {
     DstColsArgs<T>& a = ch.cols[ch.ncols];
-    a.v = tb.t; a.ptw = tb.ptw[axis]; a.chirp = tb.chirp[axis]; a.bhat = tb.bhat[axis]; a.st = io.st;
+    const bool cprime = dst_prime<T>(g, axis);
+    a.perm = cprime ? tb.perm[axis] : nullptr;
+    a.v = tb.t; a.ptw = cprime ? tb.dptw[axis] : tb.ptw[axis]; a.chirp = tb.chirp[axis]; a.bhat = tb.bhat[axis]; a.st = io.st;
     a.ftw = tb.ftw; a.fchirp = tb.fchirp[axis]; a.fbhat = tb.fbhat[axis]; a.bexp = tb.bexp[axis];
     a.post = 1.0;
-    a.n = g.n[axis]; a.ncols = nx; a.lg = g.lg[axis]; a.lgmax = g.lgmax;
+    const int L = dst_len<T>(g, axis);
+    a.n = g.n[axis]; a.ncols = nx; a.lg = ilog2i(L); a.lgmax = g.lgmax;
     a.ostride = ostride; a.lstride = lstride;
-    const int L = g.L[axis];
     const int tx = tile_at<T>(plan_tx<T>(g, tb, axis), L, io.col_threads);
     a.ltx = ilog2i(tx);
     ch.cols_grid[ch.ncols] = dim3((nx + tx - 1) / tx, nouter);
@@ -622,10 +633,11 @@ PrecChain<T> build_precond(const Geo& g, const Tables<T>& tb, const PrecIO<T>& i
     DstRowsArgs<T>& a = ch.last;
     a.in = tb.t; a.out = io.out; a.tw = tb.tw; a.chirp = tb.chirp[d - 1]; a.bhat = tb.bhat[d - 1]; a.bhat8 = tb.bhat8;
     a.ftw = tb.ftw; a.fchirp = tb.fchirp[d - 1]; a.fbhat = tb.fbhat[d - 1]; a.bexp = tb.bexp[d - 1]; a.odd = odd;
+    a.perm = prime ? tb.perm[d - 1] : nullptr;
     a.st = io.st; a.x = nullptr; a.r = nullptr; a.p = nullptr; a.q = nullptr;
     a.rr_part = nullptr;
     a.dotw = io.dotw; a.dot_part = io.dot_part; a.post = post;
-    a.rows = (int)rows; a.n = nx; a.lg = g.lg[d - 1]; a.lgmax = g.lgmax; a.pre = DPRE_NONE;
+    a.rows = (int)rows; a.n = nx; a.lg = ilog2i(Ld); a.lgmax = g.lgmax; a.pre = DPRE_NONE;
     // the CG step needs r.z partials (dotw), the update pass's ||r||^2
     // partials and a state
     const bool step = io.fin == FIN_STEP && io.dotw && io.dot_part && io.rr_part && io.st;
@@ -658,12 +670,13 @@ cudaError_t launch_precond(const Geo& g, const Tables<T>& tb, cudaStream_t s, co
   // the tridiagonal pass's table must hold this shift and scale
   if (tb.tri_shift != io.shift || tb.tri_scale != io.scale) return cudaErrorInvalidValue;
   const PrecChain<T> ch = build_precond<T>(g, tb, io);
-  const int Lx = g.L[g.d - 1];
+  const int Lx = dst_len<T>(g, g.d - 1);
   const bool odd = dst_odd(g, g.d - 1);
   FL_KERNEL((sizeof(T) == 4 ? "dst_rows" "<f32>" : "dst_rows" "<f64>"), s,
             if constexpr (sizeof(T) == 4) {
               if (rows_w8(tb, Lx, ch.row_blocks)) launch_dst_rows_w8(ch.first, ch.row_blocks, ch.row_smem, s);
               else if (odd) FL_ROWS_LAUNCH(k_dst_rows_odd, T, Lx, ch.row_blocks, ch.row_smem, s, ch.first);
+              else if (ch.first.perm) FL_ROWS_LAUNCH(k_dst_rows_prime, T, Lx, ch.row_blocks, ch.row_smem, s, ch.first);
               else FL_ROWS_LAUNCH(k_dst_rows, T, Lx, ch.row_blocks, ch.row_smem, s, ch.first);
             } else {
               if (odd) FL_ROWS_LAUNCH(k_dst_rows_odd, T, Lx, ch.row_blocks, ch.row_smem, s, ch.first);
@@ -676,13 +689,23 @@ cudaError_t launch_precond(const Geo& g, const Tables<T>& tb, cudaStream_t s, co
                 pdl_launch(tri, ch.tri_blocks, kTriCols<T> * kTriSeg, 0, s, ch.tri));
     if (j < ch.ncols)
       FL_KERNEL((sizeof(T) == 4 ? "dst_cols" "<f32>" : "dst_cols" "<f64>"), s,
-                FL_COLS_LAUNCH(k_dst_cols, T, 1 << ch.cols[j].lg, ch.cols_grid[j], ch.cols_smem[j], s,
-                               ch.cols[j]));
+                if constexpr (sizeof(T) == 4) {
+                  if (ch.cols[j].perm)
+                    FL_COLS_LAUNCH(k_dst_cols_prime, T, 1 << ch.cols[j].lg, ch.cols_grid[j], ch.cols_smem[j], s,
+                                   ch.cols[j]);
+                  else
+                    FL_COLS_LAUNCH(k_dst_cols, T, 1 << ch.cols[j].lg, ch.cols_grid[j], ch.cols_smem[j], s,
+                                   ch.cols[j]);
+                } else {
+                  FL_COLS_LAUNCH(k_dst_cols, T, 1 << ch.cols[j].lg, ch.cols_grid[j], ch.cols_smem[j], s,
+                                 ch.cols[j]);
+                });
   }
   FL_KERNEL((sizeof(T) == 4 ? "dst_rows" "<f32>" : "dst_rows" "<f64>"), s,
             if constexpr (sizeof(T) == 4) {
               if (rows_w8(tb, Lx, ch.row_blocks)) launch_dst_rows_w8(ch.last, ch.row_blocks, ch.row_smem, s);
               else if (odd) FL_ROWS_LAUNCH(k_dst_rows_odd, T, Lx, ch.row_blocks, ch.row_smem, s, ch.last);
+              else if (ch.last.perm) FL_ROWS_LAUNCH(k_dst_rows_prime, T, Lx, ch.row_blocks, ch.row_smem, s, ch.last);
               else FL_ROWS_LAUNCH(k_dst_rows, T, Lx, ch.row_blocks, ch.row_smem, s, ch.last);
             } else {
               if (odd) FL_ROWS_LAUNCH(k_dst_rows_odd, T, Lx, ch.row_blocks, ch.row_smem, s, ch.last);

@@ -59,7 +59,9 @@ __device__ void persist_rows_inv(const PItem& it, int i, int l) {
 __device__ void persist_dst_rows(const PItem& it, int i, int l) {
   const DstRowsArgs<float> a = static_cast<const DstRowsArgs<float>*>(it.args)[i];
   const int gx = it.gx[i];
-  if (a.odd) {
+  if (a.perm) {
+    FL_PERSIST_LG_SWITCH(a.lg, (body_dst_rows_prime_at<float, kPT, kPV, kPLo, kPHi>(a, l % gx, LG)))
+  } else if (a.odd) {
     FL_PERSIST_LG_SWITCH(a.lg, (body_dst_rows_odd_at<float, kPT, kPV, kPLo, kPHi>(a, l % gx, LG)))
   } else {
     FL_PERSIST_LG_SWITCH(a.lg, (body_dst_rows_at<float, kPT, kPV, kPLo, kPHi>(a, l % gx, l / gx, LG)))
@@ -70,7 +72,11 @@ __device__ void persist_dst_cols(const PItem& it, int i, int l) {
   const int gx = it.gx[i];
   const int bx = l % gx, by = l / gx;
   const int w = block_ltx(a.ltx, bx, a.ncols);
-  FL_PERSIST_LG_SWITCH(a.lg, (body_dst_cols_at<float, kPT, kPV, kPLo, kPHi>(a, bx << a.ltx, by, LG, w)))
+  if (a.perm) {
+    FL_PERSIST_LG_SWITCH(a.lg, (body_dst_cols_at<float, kPT, kPV, true, kPLo, kPHi>(a, bx << a.ltx, by, LG, w)))
+  } else {
+    FL_PERSIST_LG_SWITCH(a.lg, (body_dst_cols_at<float, kPT, kPV, false, kPLo, kPHi>(a, bx << a.ltx, by, LG, w)))
+  }
 }
 __device__ void persist_tri_cols(const PItem& it, int i, int l) {
   const TriArgs<float> a = static_cast<const TriArgs<float>*>(it.args)[i];

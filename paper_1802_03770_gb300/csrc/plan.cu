@@ -283,11 +283,47 @@ fl_status build_tables(fl_plan* p) {
       bx[k] = fix_const(ldexpl(v.real(), -bexp), ldexpl(v.imag(), -bexp));
       b32[k] = make_float2((float)v.real(), (float)v.imag());
     }
-    // FP32: in the order in which the transforms hold the frequencies
-    std::vector<float2> b16(L), b8(L);
-    for (int k = 0; k < L; ++k) {
-      b16[k] = b32[place_frequency(k, g.lg[ax], 16)];
-      b8[k] = b32[place_frequency(k, g.lg[ax], 8)];
+    // FP32, n + 1 prime: Rader's convolution (body_dst_rows_prime_at)
+    const int Ld = dst_len<float>(g, ax), lgd = ilog2i(Ld);
+    if (dst_prime<float>(g, ax)) {
+      const int q = n + 1, M = n / 2;
+      std::vector<short> perm(n);
+      int gen = 1;
+      for (int a = 0; a < M;) {   // a generator modulo sign: g^a = +-1 for no 0 < a < M
+        ++gen;
+        long long v = gen;
+        for (a = 1; a < M && v != 1 && v != q - 1; ++a) v = v * gen % q;
+      }
+      std::vector<int> pw(n);   // gen^a mod q
+      pw[0] = 1;
+      for (int a = 1; a < n; ++a) pw[a] = (int)((long long)pw[a - 1] * gen % q);
+      // gen^M is -1, or 1 where gen generates the squares only: then the powers
+      // repeat after M, and gen^-d is the same power either way
+      auto inv = [&](int d) { return pw[((n - d) % n + n) % n]; };
+      std::vector<std::complex<long double>> ker(Ld, 0.0L);
+      for (int d = -(M - 1); d <= M - 1; ++d)
+        ker[(d + Ld) % Ld] = sinl(2.0L * pi * (long double)inv(d) / (long double)q);
+      host_fft(ker);
+      for (int k = 0; k < Ld; ++k)
+        b32[k] = make_float2((float)(ker[k].real() / Ld), (float)(ker[k].imag() / Ld));
+      for (int a = 0; a < M; ++a) {
+        const int m = inv(a);
+        perm[a] = (short)pw[a];
+        perm[M + a] = (short)(m <= M ? 2 * m : -2 * (q - m));
+      }
+      us = upload_table(p, &p->t32.perm[ax], perm);
+      if (us != FL_OK) return us;
+      std::vector<float2> dt(place_table_len(lgd));
+      for (size_t m = 0; m < dt.size(); ++m)
+        dt[m] = tw32[(size_t)place_table_power((int)m, lgd, Cfg<float>::CV) << (g.lgmax - lgd)];
+      us = upload_table(p, &p->t32.dptw[ax], dt);
+      if (us != FL_OK) return us;
+    }
+    // in the order in which the transforms hold the frequencies
+    std::vector<float2> b16(Ld), b8(Ld);
+    for (int k = 0; k < Ld; ++k) {
+      b16[k] = b32[place_frequency(k, lgd, 16)];
+      b8[k] = b32[place_frequency(k, lgd, 8)];
     }
     std::vector<float2> pt(place_table_len(g.lg[ax]));
     for (size_t m = 0; m < pt.size(); ++m)

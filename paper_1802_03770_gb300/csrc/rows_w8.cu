@@ -20,8 +20,9 @@ void launch_rows_inv_w8(const RowsInvArgs<float>& a, int grid, size_t smem, cuda
 }
 
 void launch_dst_rows_w8(const DstRowsArgs<float>& a, int grid, size_t smem, cudaStream_t s) {
-  pdl_launch(a.odd ? k_dst_rows_odd<float, kRowsW8Threads, 8> : k_dst_rows<float, kRowsW8Threads, 8>, grid,
-             kRowsW8Threads, smem, s, a);
+  pdl_launch(a.odd ? k_dst_rows_odd<float, kRowsW8Threads, 8>
+             : a.perm ? k_dst_rows_prime<float, kRowsW8Threads, 8> : k_dst_rows<float, kRowsW8Threads, 8>,
+             grid, kRowsW8Threads, smem, s, a);
 }
 
 cudaError_t configure_rows_w8() {
@@ -29,7 +30,8 @@ cudaError_t configure_rows_w8() {
   for (const void* f : {reinterpret_cast<const void*>(&k_rows_fwd<float, kRowsW8Threads, 8>),
                         reinterpret_cast<const void*>(&k_rows_inv<float, kRowsW8Threads, 8>),
                         reinterpret_cast<const void*>(&k_dst_rows<float, kRowsW8Threads, 8>),
-                        reinterpret_cast<const void*>(&k_dst_rows_odd<float, kRowsW8Threads, 8>)}) {
+                        reinterpret_cast<const void*>(&k_dst_rows_odd<float, kRowsW8Threads, 8>),
+                        reinterpret_cast<const void*>(&k_dst_rows_prime<float, kRowsW8Threads, 8>)}) {
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (e == cudaSuccess)

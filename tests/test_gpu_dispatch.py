@@ -91,3 +91,28 @@ def test_iteration_cap(cap):
     b = dev(np.random.default_rng(9).standard_normal(n), torch.float64)
     _, info = p.solve(b, tol=1e-300, maxit=cap, mode=0, raise_on_fail=False)
     assert info["iterations"] == cap
+
+
+# axes with n + 1 prime (FP32: Rader's convolution): the shortest lines, one stage and several, full and partial CTAs and
+# tiles, the last and the middle axis, generators of all residues and of half of them; FP64 stays with its own form
+@pytest.mark.parametrize("n", [(1, 10), (5, 12), (300, 16), (33, 40), (17, 96), (3, 130), (65, 192), (40, 256), (5, 640),
+                               (4, 768), (2, 1012), (3, 2028), (2, 4092), (4, 16, 9), (3, 96, 33), (2, 256, 256),
+                               (3, 192, 35), (2, 12, 1000)])
+@pytest.mark.parametrize("masked", [False, True])
+def test_prime_sines(n, masked):
+    d = len(n)
+    h = 1.0 / (max(n) + 1)
+    rng = np.random.default_rng(10)
+    mask = None
+    if masked:
+        mask = np.ones(n, dtype=bool)
+        mask[(0,) * (d - 1) + (slice(2, 5),)] = False
+    op, p = OPlan(d, n, h, 1.3, mask=mask), Plan(d, n, h, 1.3, mask=mask)
+    r = rng.standard_normal(n).astype(np.float32).astype(np.float64)
+    for shift, scale in ((0.0, 1.0), (1.0, 1e-3)):
+        ref = oprec.solve_domain(op, r, shift, scale) if masked else oprec.solve_box(op, r, shift, scale)
+        if masked:
+            ref = np.where(mask, ref, 0.0)
+        for dtype, tol in ((torch.float64, 1e-11), (torch.float32, 2e-5)):
+            z = p.precond(dev(r, dtype), shift=shift, scale=scale).cpu().numpy()
+            assert rel(z, ref) <= tol, (dtype, rel(z, ref))
