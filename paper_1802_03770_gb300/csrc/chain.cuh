@@ -281,10 +281,13 @@ template <typename T> inline bool rows_w8(const Tables<T>& tb, int L, int ctas) 
 inline bool dst_odd(const Geo& g, int axis) { return g.L[axis] == 2 * (g.n[axis] + 1); }
 // Whether an FP32 DST along an axis is Rader's convolution of half the length
 // (n + 1 an odd prime; lines of 16 points are the shortest), and the length of
-// the DST's transforms.
+// the DST's transforms.  Not where rows of 256 points take the 256 x 8 shape by
+// rows_w8, which lines of 128 do not have (preconditioner 96^2 9.4 us so, 12.8
+// by Rader; 96^3, more CTAs, 54.7 and 38.5).
 template <typename T> inline bool dst_prime(const Geo& g, int axis) {
   const int q = g.n[axis] + 1;
   if (sizeof(T) != 4 || g.L[axis] < 32 || q % 2 == 0) return false;
+  if (axis == g.d - 1 && g.L[axis] == 256 && g.N / g.n[axis] <= 152 * row_lines<T>(256)) return false;
   for (int f = 3; f * f <= q; f += 2)
     if (q % f == 0) return false;
   return true;

@@ -190,50 +190,49 @@ template <> struct LogR<8> { static constexpr int v = 3; };
 template <> struct LogR<16> { static constexpr int v = 4; };
 
 // w[r] = w1^r, r = 0..R-1, for w1 = exp(-2 pi i step / Lmax) (conjugated
-// for the inverse).  FP64, and FP32 with TWT (tw then points to a copy of
-// the table in shared memory): every power is loaded from the long-double
-// table tw (GB300's FP64 rate makes the loads cheaper than products).  FP32: w1 = sincospif(-2 step / Lmax) (the
-// argument is exact), w2, w4, w8 by squaring, the rest by products -- no
-// table load on the stage's critical path (measured 3 % faster solves on
-// the 1024^2 workload than the table, at unchanged iteration counts).
+// for the inverse).  FP64, and FP32 with TWT (tw then points to a copy of the
+// table in shared memory): every power is loaded from the long-double table tw
+// (r * step < Lmax).  FP32 without: w1 = sincospif(-2 step / Lmax) (the argument
+// is exact), w2 and w4 by squaring, w4 brought back to modulus 1 to first order,
+// the rest by products.  Without that w8..w15 have up to fifteen times the
+// modulus error of w1, which the two directions of a convolution add up:
+// preconditioner 640^2, error 5.9e-7, with it 3.3e-7 (18.8 -> 19.2 us, 256^3 380
+// -> 379).  w4 from the table 3.6e-7 (1024^2 32.9 -> 34.1), w1, w2, w4 and w8
+// from it 3.0e-7 (1024^2 35.8, 256^3 403).
 template <int R, bool TWT = false, typename C>
 __device__ __forceinline__ void twiddles(const C* FL_RESTRICT tw, int step, bool inv, C* w, int lgmax) {
   auto ld = [&](int i) {
-    C t;
-    if constexpr (sizeof(t.x) == 4 && !TWT) {
-      float sn, cs;
-      sincospif(-(float)i * ldexpf(1.0f, 1 - lgmax), &sn, &cs);
-      t.x = cs;
-      t.y = sn;
-    } else {
-      t = tw[i];
-    }
+    C t = tw[i];
     if (inv) t.y = -t.y;
     return t;
   };
   w[0] = cmake<C>(1, 0);
   if constexpr (sizeof(w[0].x) == 8 || TWT) {
-    // FP64, and FP32 with a table (TWT): every power straight from the table
-    // (loads instead of products; r * step < Lmax)
 #pragma unroll
     for (int r = 1; r < R; ++r) w[r] = ld(r * step);
-    return;
-  }
-  if (R >= 2) w[1] = ld(step);
-  if (R >= 4) {
-    w[2] = sizeof(w[0].x) == 4 ? cmul(w[1], w[1]) : ld(2 * step);
-    w[3] = cmul(w[1], w[2]);
-  }
-  if (R >= 8) {
-    w[4] = sizeof(w[0].x) == 4 ? cmul(w[2], w[2]) : ld(4 * step);
-    w[5] = cmul(w[4], w[1]);
-    w[6] = cmul(w[4], w[2]);
-    w[7] = cmul(w[4], w[3]);
-  }
-  if (R >= 16) {
-    w[8] = sizeof(w[0].x) == 4 ? cmul(w[4], w[4]) : ld(8 * step);
+  } else {
+    if (R >= 2) {
+      float sn, cs;
+      sincospif(-(float)step * ldexpf(1.0f, 1 - lgmax), &sn, &cs);
+      w[1] = cmake<C>(cs, inv ? -sn : sn);
+    }
+    if (R >= 4) {
+      w[2] = cmul(w[1], w[1]);
+      w[3] = cmul(w[1], w[2]);
+    }
+    if (R >= 8) {
+      w[4] = cmul(w[2], w[2]);
+      const float e = -0.5f * fmaf(w[4].x, w[4].x, fmaf(w[4].y, w[4].y, -1.0f));
+      w[4] = cmake<C>(fmaf(w[4].x, e, w[4].x), fmaf(w[4].y, e, w[4].y));
+      w[5] = cmul(w[4], w[1]);
+      w[6] = cmul(w[4], w[2]);
+      w[7] = cmul(w[4], w[3]);
+    }
+    if (R >= 16) {
+      w[8] = cmul(w[4], w[4]);
 #pragma unroll
-    for (int r = 9; r < 16; ++r) w[r] = cmul(w[8], w[r - 8]);
+      for (int r = 9; r < 16; ++r) w[r] = cmul(w[8], w[r - 8]);
+    }
   }
 }
 
