@@ -685,7 +685,8 @@ cudaError_t launch_precond(const Geo& g, const Tables<T>& tb, cudaStream_t s, co
   for (int j = 0; j <= ch.ncols; ++j) {
     if (j == ch.tri_after)
       FL_KERNEL((sizeof(T) == 4 ? "tri_cols" "<f32>" : "tri_cols" "<f64>"), s,
-                const auto tri = ch.tri.m <= 8 ? k_tri_cols<T, 8> : ch.tri.m <= 16 ? k_tri_cols<T, 16> : k_tri_cols<T, kTriM>;
+                const auto tri = ch.tri.m <= 8 ? k_tri_cols<T, 8> : ch.tri.m <= 16 ? k_tri_cols<T, 16>
+                                 : ch.tri.m <= 24 ? k_tri_cols<T, 24> : k_tri_cols<T, kTriM>;
                 pdl_launch(tri, ch.tri_blocks, kTriCols<T> * kTriSeg, 0, s, ch.tri));
     if (j < ch.ncols)
       FL_KERNEL((sizeof(T) == 4 ? "dst_cols" "<f32>" : "dst_cols" "<f64>"), s,

@@ -116,3 +116,9 @@ def test_prime_sines(n, masked):
         for dtype, tol in ((torch.float64, 1e-11), (torch.float32, 2e-5)):
             z = p.precond(dev(r, dtype), shift=shift, scale=scale).cpu().numpy()
             assert rel(z, ref) <= tol, (dtype, rel(z, ref))
+
+
+# tridiagonal segments about 24 rows
+@pytest.mark.parametrize("n", [(544, 6), (545, 6), (700, 9), (768, 5), (769, 5)])
+def test_tridiagonal_segments_24(n):
+    test_tridiagonal_segments(n, 1.0, 1e-3)
