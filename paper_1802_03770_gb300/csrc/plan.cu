@@ -257,86 +257,89 @@ fl_status build_tables(fl_plan* p) {
   for (int ax = 0; ax < g.d; ++ax) {
     const int n = g.n[ax], L = g.L[ax];
     const long long N1 = n + 1;
-    // c_m = exp(i pi m^2 / (2 N1)), with m^2 reduced mod 4 N1
-    auto chirp = [&](long long m) {
-      const long long m2 = (m * m) % (4 * N1);
-      const long double ang = pi * (long double)m2 / (2.0L * (long double)N1);
-      return std::complex<long double>(cosl(ang), sinl(ang));
-    };
-    std::vector<FxW> cx(n);
-    std::vector<float2> c32(n);
-    for (int j = 0; j < n; ++j) {
-      const auto c = chirp(j + 1);
-      cx[j] = fix_const(c.real(), c.imag());
-      c32[j] = make_float2((float)c.real(), (float)c.imag());
-    }
-    std::vector<std::complex<long double>> b(L, 0.0L);
-    for (int m = -(n - 1); m <= n - 1; ++m) b[(m + L) % L] = std::conj(chirp(m));
-    host_fft(b);
-    std::vector<FxW> bx(L);
-    std::vector<float2> b32(L);
-    long double top = 0.0L;
-    for (int k = 0; k < L; ++k) top = std::max(top, fabsl(b[k].real()) + fabsl(b[k].imag()));
-    const int bexp = std::ilogb(top / (long double)L) + 1;   // moduli below 2^bexp
-    for (int k = 0; k < L; ++k) {
-      const auto v = b[k] / (long double)L;
-      bx[k] = fix_const(ldexpl(v.real(), -bexp), ldexpl(v.imag(), -bexp));
-      b32[k] = make_float2((float)v.real(), (float)v.imag());
-    }
-    // FP32, n + 1 prime: Rader's convolution (body_dst_rows_prime_at)
-    const int Ld = dst_len<float>(g, ax), lgd = ilog2i(Ld);
-    if (dst_prime<float>(g, ax)) {
-      const int q = n + 1, M = n / 2;
-      std::vector<short> perm(n);
-      int gen = 1;
-      for (int a = 0; a < M;) {   // a generator modulo sign: g^a = +-1 for no 0 < a < M
-        ++gen;
-        long long v = gen;
-        for (a = 1; a < M && v != 1 && v != q - 1; ++a) v = v * gen % q;
-      }
-      std::vector<int> pw(n);   // gen^a mod q
-      pw[0] = 1;
-      for (int a = 1; a < n; ++a) pw[a] = (int)((long long)pw[a - 1] * gen % q);
-      // gen^M is -1, or 1 where gen generates the squares only: then the powers
-      // repeat after M, and gen^-d is the same power either way
-      auto inv = [&](int d) { return pw[((n - d) % n + n) % n]; };
-      std::vector<std::complex<long double>> ker(Ld, 0.0L);
-      for (int d = -(M - 1); d <= M - 1; ++d)
-        ker[(d + Ld) % Ld] = sinl(2.0L * pi * (long double)inv(d) / (long double)q);
-      host_fft(ker);
-      for (int k = 0; k < Ld; ++k)
-        b32[k] = make_float2((float)(ker[k].real() / Ld), (float)(ker[k].imag() / Ld));
-      for (int a = 0; a < M; ++a) {
-        const int m = inv(a);
-        perm[a] = (short)pw[a];
-        perm[M + a] = (short)(m <= M ? 2 * m : -2 * (q - m));
-      }
-      us = upload_table(p, &p->t32.perm[ax], perm);
-      if (us != FL_OK) return us;
-      std::vector<float2> dt(place_table_len(lgd));
-      for (size_t m = 0; m < dt.size(); ++m)
-        dt[m] = tw32[(size_t)place_table_power((int)m, lgd, Cfg<float>::CV) << (g.lgmax - lgd)];
-      us = upload_table(p, &p->t32.dptw[ax], dt);
-      if (us != FL_OK) return us;
-    }
-    // in the order in which the transforms hold the frequencies
-    std::vector<float2> b16(Ld), b8(Ld);
-    for (int k = 0; k < Ld; ++k) {
-      b16[k] = b32[place_frequency(k, lgd, 16)];
-      b8[k] = b32[place_frequency(k, lgd, 8)];
-    }
+    // stage twiddles of the strided passes
     std::vector<float2> pt(place_table_len(g.lg[ax]));
     for (size_t m = 0; m < pt.size(); ++m)
       pt[m] = tw32[(size_t)place_table_power((int)m, g.lg[ax], Cfg<float>::CV) << (g.lgmax - g.lg[ax])];
     us = upload_table(p, &p->t32.ptw[ax], pt);
     if (us != FL_OK) return us;
-    p->t64.bexp[ax] = bexp;
-    us = upload_table(p, &p->t64.fchirp[ax], cx);
-    if (us == FL_OK) us = upload_table(p, &p->t64.fbhat[ax], bx);
-    if (us == FL_OK) us = upload_table(p, &p->t32.chirp[ax], c32);
-    if (us == FL_OK) us = upload_table(p, &p->t32.bhat[ax], b16);
-    if (us == FL_OK && ax == g.d - 1) us = upload_table(p, &p->t32.bhat8, b8);
-    if (us != FL_OK) return us;
+    if (ax > 0) {   // axis 0 has no DST (tridiagonal pass)
+      // c_m = exp(i pi m^2 / (2 N1)), with m^2 reduced mod 4 N1
+      auto chirp = [&](long long m) {
+        const long long m2 = (m * m) % (4 * N1);
+        const long double ang = pi * (long double)m2 / (2.0L * (long double)N1);
+        return std::complex<long double>(cosl(ang), sinl(ang));
+      };
+      std::vector<FxW> cx(n);
+      std::vector<float2> c32(n);
+      for (int j = 0; j < n; ++j) {
+        const auto c = chirp(j + 1);
+        cx[j] = fix_const(c.real(), c.imag());
+        c32[j] = make_float2((float)c.real(), (float)c.imag());
+      }
+      std::vector<std::complex<long double>> b(L, 0.0L);
+      for (int m = -(n - 1); m <= n - 1; ++m) b[(m + L) % L] = std::conj(chirp(m));
+      host_fft(b);
+      std::vector<FxW> bx(L);
+      std::vector<float2> b32(L);
+      long double top = 0.0L;
+      for (int k = 0; k < L; ++k) top = std::max(top, fabsl(b[k].real()) + fabsl(b[k].imag()));
+      const int bexp = std::ilogb(top / (long double)L) + 1;   // moduli below 2^bexp
+      for (int k = 0; k < L; ++k) {
+        const auto v = b[k] / (long double)L;
+        bx[k] = fix_const(ldexpl(v.real(), -bexp), ldexpl(v.imag(), -bexp));
+        b32[k] = make_float2((float)v.real(), (float)v.imag());
+      }
+      // FP32, n + 1 prime: Rader's convolution (body_dst_rows_prime_at)
+      const int Ld = dst_len<float>(g, ax), lgd = ilog2i(Ld);
+      if (dst_prime<float>(g, ax)) {
+        const int q = n + 1, M = n / 2;
+        std::vector<short> perm(n);
+        int gen = 1;
+        for (int a = 0; a < M;) {   // a generator modulo sign: g^a = +-1 for no 0 < a < M
+          ++gen;
+          long long v = gen;
+          for (a = 1; a < M && v != 1 && v != q - 1; ++a) v = v * gen % q;
+        }
+        std::vector<int> pw(n);   // gen^a mod q
+        pw[0] = 1;
+        for (int a = 1; a < n; ++a) pw[a] = (int)((long long)pw[a - 1] * gen % q);
+        // gen^M is -1, or 1 where gen generates the squares only: then the powers
+        // repeat after M, and gen^-d is the same power either way
+        auto inv = [&](int d) { return pw[((n - d) % n + n) % n]; };
+        std::vector<std::complex<long double>> ker(Ld, 0.0L);
+        for (int d = -(M - 1); d <= M - 1; ++d)
+          ker[(d + Ld) % Ld] = sinl(2.0L * pi * (long double)inv(d) / (long double)q);
+        host_fft(ker);
+        for (int k = 0; k < Ld; ++k)
+          b32[k] = make_float2((float)(ker[k].real() / Ld), (float)(ker[k].imag() / Ld));
+        for (int a = 0; a < M; ++a) {
+          const int m = inv(a);
+          perm[a] = (short)pw[a];
+          perm[M + a] = (short)(m <= M ? 2 * m : -2 * (q - m));
+        }
+        us = upload_table(p, &p->t32.perm[ax], perm);
+        if (us != FL_OK) return us;
+        std::vector<float2> dt(place_table_len(lgd));
+        for (size_t m = 0; m < dt.size(); ++m)
+          dt[m] = tw32[(size_t)place_table_power((int)m, lgd, Cfg<float>::CV) << (g.lgmax - lgd)];
+        us = upload_table(p, &p->t32.dptw[ax], dt);
+        if (us != FL_OK) return us;
+      }
+      // in the order in which the transforms hold the frequencies
+      std::vector<float2> b16(Ld), b8(Ld);
+      for (int k = 0; k < Ld; ++k) {
+        b16[k] = b32[place_frequency(k, lgd, 16)];
+        b8[k] = b32[place_frequency(k, lgd, 8)];
+      }
+      p->t64.bexp[ax] = bexp;
+      us = upload_table(p, &p->t64.fchirp[ax], cx);
+      if (us == FL_OK) us = upload_table(p, &p->t64.fbhat[ax], bx);
+      if (us == FL_OK) us = upload_table(p, &p->t32.chirp[ax], c32);
+      if (us == FL_OK) us = upload_table(p, &p->t32.bhat[ax], b16);
+      if (us == FL_OK && ax == g.d - 1) us = upload_table(p, &p->t32.bhat8, b8);
+      if (us != FL_OK) return us;
+    }
     // eigenvalues of C h^d L along this axis: c (-a) 4 sin^2(pi k / (2 (n+1)))
     std::vector<double> mu(n);
     for (int k = 0; k < n; ++k) {
