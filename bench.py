@@ -147,7 +147,7 @@ NCU_DRAM_BYTES = {
 
 # the sources that make up the single-plan pass kernels and their launch
 # shapes (the roofline kernel's code and configuration)
-PASS_KERNEL_SOURCES = ("chain.cuh", "fft_core.cuh", "internal.h", "kernels.cuh", "ops.cu")
+PASS_KERNEL_SOURCES = ("chain.cuh", "fft_core.cuh", "fix_core.cuh", "fix_passes.cuh", "internal.h", "kernels.cuh", "ops.cu")
 
 
 def kernel_source_sha():

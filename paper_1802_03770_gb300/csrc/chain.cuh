@@ -45,8 +45,8 @@ inline cudaError_t launch_status() {
 // Launch shapes.  A CTA keeps VPT * THREADS complex values in shared memory:
 // row passes one or two lines of L = 2048 (many small CTAs, up to eight per
 // SM, so that a 1024-line pass fills all 152 SMs several times over);
-// strided passes a tile of 4 (FP32) or 2 (FP64) columns of L = 2048, i.e. at
-// least 32 contiguous bytes per line element.
+// strided passes a tile of 4 (FP32) or 2 (FP64) columns of L = 2048, i.e. 32
+// contiguous bytes per line element.
 template <typename T> struct Cfg;
 template <> struct Cfg<float> {
   static constexpr int RT = 128, RV = 16;   // rows: threads, values per thread

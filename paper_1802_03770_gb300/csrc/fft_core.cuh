@@ -15,10 +15,15 @@
 // number of values a thread holds is VPT = lines * L / blockDim.x, a
 // compile-time bound chosen by the launcher.
 //
+// The FP32 convolution passes use a second form, in place with the
+// frequencies in digit-reversed places (fft_places); the FP64 passes have
+// their own fixed-point transforms (fix_passes.cuh), so the FP64 stages here
+// run in the symbol's set-up only.
+//
 // Twiddles: FP64 stages load every power w^r from a table
-// tw[k] = exp(-2 pi i k / Lmax) computed on the host in long double; FP32
-// stages compute w with sincospif and the even powers by squaring; the
-// other powers are complex products (see twiddles()).
+// tw[k] = exp(-2 pi i k / Lmax) computed on the host in long double, FP32
+// column passes from a copy in shared memory; the other FP32 stages compute
+// them (see twiddles()).
 //
 // Two storage layouts: lines of stride ls (element j of line q at
 // q * ls + j, ls a multiple of 16), and 2^ltx interleaved lines (element j

@@ -22,6 +22,8 @@
 // (2(n+1))), sin(pi jk/(n+1)) = Im(c_j c_k conj(c_{k-j})), so
 // X_k = Im(c_k sum_j (c_j x_j) conj(c_{k-j})) -- a linear convolution of
 // length-n sequences done with FFTs of the operator's length L >= 2n - 1.
+// Rows with n + 1 = 2^k take the odd extension, two per transform, and FP32
+// axes with n + 1 an odd prime Rader's convolution of length L/2.
 #pragma once
 
 #include "fft_core.cuh"
