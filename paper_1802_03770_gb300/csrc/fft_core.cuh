@@ -487,9 +487,10 @@ __host__ __device__ __forceinline__ int place_frequency(int p, int lg, int vpt) 
 template <int V> struct IntC { static constexpr int v = V; };
 
 // Twiddles of stage ST at offset j: exp(-2 pi i j r / B), B its block length.
-// TWT: from a table per stage in shared memory, one after another (stage s:
-// B_s entries; read at a stride of 16 places, the table of the whole line had
-// eight-way bank conflicts), place_table_len entries in all.
+// TW_CALC: computed.  TW_TABLE: from a table per stage in shared memory, one
+// after another (stage s: B_s entries; read at a stride of 16 places, the table
+// of the whole line had eight-way bank conflicts), place_table_len entries in
+// all.
 __host__ __device__ __forceinline__ int place_table_len(int lg) { return (1 << lg) + (1 << lg) / 4; }
 // entry m of the concatenated tables as a power of exp(-2 pi i / 2^lg), below 2^lg
 inline int place_table_power(int m, int lg, int vpt) {
@@ -509,18 +510,48 @@ __host__ __device__ constexpr int place_table_at(int st) {
   }
   return at;
 }
-template <int R, bool TWT, int LG, int VPT, int ST, typename C>
+// TW_ROWS: rows of up to 2^kRowTableLg points, tables in shared memory too, but
+// entry r M + j: neighbouring threads have neighbouring j.  Longer rows, whose
+// tables would be as large as a CTA's lines, compute their twiddles.  With powers
+// of a computed w1 the prime-length preconditioner was less accurate than with
+// the chirps it replaced (relative error 40^2 2.29 -> 2.34e-7, 136^2 2.49 -> 2.67,
+// 256^2 3.00 -> 3.14, 256^3 3.82 -> 4.05), from the tables 1.82, 2.06, 2.46 and
+// 3.73; six powers from the table and one product for each of the others 2.08,
+// 2.31, 2.71 and 4.01.  Longer rows were below the chirps without (640^2 4.26 ->
+// 3.31).
+constexpr int kRowTableLg = 8;
+__host__ __device__ __forceinline__ int row_table_len(int lg) { return lg <= kRowTableLg ? place_table_len(lg) : 0; }
+// entry m of the rows' tables as a power of exp(-2 pi i / 2^lg), below 2^lg
+inline int row_table_power(int m, int lg, int vpt) {
+  int lgb = lg, s = 0;
+  for (; lgb > 0 && m >= (1 << lgb); ++s) {
+    m -= 1 << lgb;
+    lgb -= plan_lg_radix(lg, vpt, s);
+  }
+  if (lgb == 0) return 0;   // (the rest of the table is not read)
+  const int lgm = lgb - plan_lg_radix(lg, vpt, s);
+  return ((m >> lgm) * (m & ((1 << lgm) - 1))) << (lg - lgb);
+}
+enum { TW_CALC = 0, TW_TABLE = 1, TW_ROWS = 2 };
+template <int R, int TW, int LG, int VPT, int ST, typename C>
 __device__ __forceinline__ void place_twiddles(const C* FL_RESTRICT tw, int j, int lgmax, C* w) {
   constexpr int LGB = LG - clog2(FftPlan<LG, VPT>::ns(ST));
-  if constexpr (TWT) twiddles<R, true>(tw + place_table_at<LG, VPT>(ST), j, false, w, LGB);
-  else twiddles<R, false>(tw, j << (lgmax - LGB), false, w, lgmax);
+  if constexpr (TW == TW_TABLE) {
+    twiddles<R, true>(tw + place_table_at<LG, VPT>(ST), j, false, w, LGB);
+  } else if constexpr (TW == TW_ROWS && LG <= kRowTableLg) {
+    const C* FL_RESTRICT t = tw + place_table_at<LG, VPT>(ST) + j;
+#pragma unroll
+    for (int r = 1; r < R; ++r) w[r] = t[r << (LGB - LogR<R>::v)];
+  } else {
+    twiddles<R, false>(tw, j << (lgmax - LGB), false, w, lgmax);
+  }
 }
 
 enum { PLACE_FWD = 0, PLACE_INV = 1, PLACE_CONV = 2 };
 // What a stage does with its values: forward or inverse butterfly, legs from
 // load (IN) or the buffer, outputs to out (OUT) or the buffer; CONV is the
 // middle stage of a convolution (forward, product, inverse).
-template <int LG, int VPT, bool IL, bool HALF, bool HOUT, bool TWT, int ST, int KIND, bool IN, bool OUT, typename C,
+template <int LG, int VPT, bool IL, bool HALF, bool HOUT, int TW, int ST, int KIND, bool IN, bool OUT, typename C,
           typename Load, typename Mid, typename Out>
 __device__ __forceinline__ void place_stage(SBuf<C> buf, int ls, int ltx, int nlines, const C* FL_RESTRICT tw,
                                             int lgmax, Load& load, Mid& mid, Out& out) {
@@ -535,7 +566,7 @@ __device__ __forceinline__ void place_stage(SBuf<C> buf, int ls, int ltx, int nl
   const int S = IL ? ((1 << LGM) << ltx) : (1 << LGM);   // logical leg stride
   // the middle product or the first twiddles may read what the pass copied to
   // shared memory: legs first, then the copies' barrier
-  constexpr bool WAIT = IN && (KIND == PLACE_CONV || (KIND == PLACE_FWD && TWT && LGM > 0));
+  constexpr bool WAIT = IN && (KIND == PLACE_CONV || (KIND == PLACE_FWD && TW == TW_TABLE && LGM > 0));
   C v[NB][R];
 #pragma unroll
   for (int b = 0; b < NB; ++b) {
@@ -557,7 +588,7 @@ __device__ __forceinline__ void place_stage(SBuf<C> buf, int ls, int ltx, int nl
       }
       if constexpr (KIND == PLACE_INV && LGM > 0) {
         C w[R];
-        place_twiddles<R, TWT, LG, VPT, ST>(tw, q & ((1 << LGM) - 1), lgmax, w);
+        place_twiddles<R, TW, LG, VPT, ST>(tw, q & ((1 << LGM) - 1), lgmax, w);
 #pragma unroll
         for (int r = 1; r < R; ++r) v[b][r] = cmul(v[b][r], w[r]);
       }
@@ -591,7 +622,7 @@ __device__ __forceinline__ void place_stage(SBuf<C> buf, int ls, int ltx, int nl
       }
       if constexpr (KIND == PLACE_FWD && LGM > 0) {
         C w[R];
-        place_twiddles<R, TWT, LG, VPT, ST>(tw, j, lgmax, w);
+        place_twiddles<R, TW, LG, VPT, ST>(tw, j, lgmax, w);
 #pragma unroll
         for (int r = 1; r < R; ++r) v[b][r] = cmul(v[b][r], w[r]);
       }
@@ -608,33 +639,33 @@ __device__ __forceinline__ void place_stage(SBuf<C> buf, int ls, int ltx, int nl
   if (!OUT) __syncthreads();
 }
 
-template <int LG, int VPT, bool IL, bool TWT, int ST, int KIND, typename C, typename Load, typename Mid, typename Out>
+template <int LG, int VPT, bool IL, int TW, int ST, int KIND, typename C, typename Load, typename Mid, typename Out>
 __device__ __forceinline__ void place_stages(SBuf<C> buf, int ls, int ltx, int nlines, const C* FL_RESTRICT tw,
                                              int lgmax, Load& load, Mid& mid, Out& out) {
   typedef FftPlan<LG, VPT> P;
   constexpr int LAST = P::S - 1;
   if constexpr (KIND == PLACE_FWD) {
     // natural order (upper half zero) to places
-    place_stage<LG, VPT, IL, ST == 0, false, TWT, ST, PLACE_FWD, ST == 0, ST == LAST>(buf, ls, ltx, nlines, tw, lgmax,
+    place_stage<LG, VPT, IL, ST == 0, false, TW, ST, PLACE_FWD, ST == 0, ST == LAST>(buf, ls, ltx, nlines, tw, lgmax,
                                                                                     load, mid, out);
     if constexpr (ST < LAST)
-      place_stages<LG, VPT, IL, TWT, ST + 1, KIND>(buf, ls, ltx, nlines, tw, lgmax, load, mid, out);
+      place_stages<LG, VPT, IL, TW, ST + 1, KIND>(buf, ls, ltx, nlines, tw, lgmax, load, mid, out);
   } else if constexpr (KIND == PLACE_INV) {
     // places to natural order (lower half)
-    place_stage<LG, VPT, IL, false, ST == 0, TWT, ST, PLACE_INV, ST == LAST, ST == 0>(buf, ls, ltx, nlines, tw, lgmax,
+    place_stage<LG, VPT, IL, false, ST == 0, TW, ST, PLACE_INV, ST == LAST, ST == 0>(buf, ls, ltx, nlines, tw, lgmax,
                                                                                      load, mid, out);
     if constexpr (ST > 0)
-      place_stages<LG, VPT, IL, TWT, ST - 1, KIND>(buf, ls, ltx, nlines, tw, lgmax, load, mid, out);
+      place_stages<LG, VPT, IL, TW, ST - 1, KIND>(buf, ls, ltx, nlines, tw, lgmax, load, mid, out);
   } else {
     // forward stages before the last, the middle, and back
     if constexpr (ST < LAST) {
-      place_stage<LG, VPT, IL, ST == 0, false, TWT, ST, PLACE_FWD, ST == 0, false>(buf, ls, ltx, nlines, tw, lgmax,
+      place_stage<LG, VPT, IL, ST == 0, false, TW, ST, PLACE_FWD, ST == 0, false>(buf, ls, ltx, nlines, tw, lgmax,
                                                                                   load, mid, out);
-      place_stages<LG, VPT, IL, TWT, ST + 1, KIND>(buf, ls, ltx, nlines, tw, lgmax, load, mid, out);
-      place_stage<LG, VPT, IL, false, ST == 0, TWT, ST, PLACE_INV, false, ST == 0>(buf, ls, ltx, nlines, tw, lgmax,
+      place_stages<LG, VPT, IL, TW, ST + 1, KIND>(buf, ls, ltx, nlines, tw, lgmax, load, mid, out);
+      place_stage<LG, VPT, IL, false, ST == 0, TW, ST, PLACE_INV, false, ST == 0>(buf, ls, ltx, nlines, tw, lgmax,
                                                                                   load, mid, out);
     } else {
-      place_stage<LG, VPT, IL, LAST == 0, LAST == 0, TWT, ST, PLACE_CONV, LAST == 0, LAST == 0>(
+      place_stage<LG, VPT, IL, LAST == 0, LAST == 0, TW, ST, PLACE_CONV, LAST == 0, LAST == 0>(
           buf, ls, ltx, nlines, tw, lgmax, load, mid, out);
     }
   }
@@ -652,11 +683,11 @@ __device__ __forceinline__ void place_stages(SBuf<C> buf, int ls, int ltx, int n
   if constexpr (LGV >= LGLO && LGV <= LGHI) {                                                               \
     if (lg == LGV) {                                                                                        \
       constexpr int ST0 = KIND == PLACE_INV ? FftPlan<LGV, VPT>::S - 1 : 0;                                 \
-      place_stages<LGV, VPT, IL, TWT, ST0, KIND>(buf, ls, ltx, nlines, tw, lgmax, load, mid, out);          \
+      place_stages<LGV, VPT, IL, TW, ST0, KIND>(buf, ls, ltx, nlines, tw, lgmax, load, mid, out);          \
       return;                                                                                               \
     }                                                                                                       \
   }
-template <int KIND, int VPT, bool IL, int LGHI, int LGLO, bool TWT, typename C, typename Load, typename Mid,
+template <int KIND, int VPT, bool IL, int LGHI, int LGLO, int TW, typename C, typename Load, typename Mid,
           typename Out>
 __device__ __forceinline__ void fft_places(SBuf<C> buf, int lg, int ls, int ltx, int nlines, const C* FL_RESTRICT tw,
                                            int lgmax, Load load, Mid mid, Out out) {

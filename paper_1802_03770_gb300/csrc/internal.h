@@ -52,6 +52,9 @@ struct Tables {
   // FP32 axes with n + 1 prime: orders and stage twiddles of Rader's convolution (dst_prime)
   short* perm[3] = {nullptr, nullptr, nullptr};
   C* dptw[3] = {nullptr, nullptr, nullptr};
+  // twiddle tables of its rows, for the 16- and the 8-value stage plan (row_table_power)
+  C* rtw = nullptr;
+  C* rtw8 = nullptr;
   // FP32 DST tables
   C* chirp[3] = {nullptr, nullptr, nullptr};
   C* bhat[3] = {nullptr, nullptr, nullptr};   // by place of the 16-value stage plan

@@ -492,19 +492,19 @@ __device__ __forceinline__ void body_cols_at(const ColsArgs<T>& a, int kx0, int 
       if (c < ncol) cp_async<sizeof(T)>(d, &sig[(size_t)kk * a.sig_line + c]);
       else *d = (T)0;
     }
-    fft_places<PLACE_CONV, VPT, true, LGHI, LGLO, true>(buf, lg, 0, ltx, TX, stw, lg, ld, mid, out);
+    fft_places<PLACE_CONV, VPT, true, LGHI, LGLO, TW_TABLE>(buf, lg, 0, ltx, TX, stw, lg, ld, mid, out);
   } else if (a.mode == COLS_FWD) {
     auto outp = [=](int c, int p, C v) {
       if (c < ncol) base[(size_t)p * lstride + c] = v;
     };
-    fft_places<PLACE_FWD, VPT, true, LGHI, LGLO, true>(buf, lg, 0, ltx, TX, stw, lg, ld, mid, outp);
+    fft_places<PLACE_FWD, VPT, true, LGHI, LGLO, TW_TABLE>(buf, lg, 0, ltx, TX, stw, lg, ld, mid, outp);
   } else {
     auto ldi = [=](int c, int p0, auto lgs, auto cnt, C* v) {
 #pragma unroll
       for (int r = 0; r < decltype(cnt)::v; ++r)
         v[r] = c < ncol ? cswap(base[(size_t)(p0 + (r << decltype(lgs)::v)) * lstride + c]) : cmake<C>((T)0, (T)0);
     };
-    fft_places<PLACE_INV, VPT, true, LGHI, LGLO, true>(buf, lg, 0, ltx, TX, stw, lg, ldi, mid, out);
+    fft_places<PLACE_INV, VPT, true, LGHI, LGLO, TW_TABLE>(buf, lg, 0, ltx, TX, stw, lg, ldi, mid, out);
   }
 }
 
@@ -715,6 +715,10 @@ struct DstRowsArgs {
   const T* in;             // DPRE_NONE: input rows
   T* out;
   const typename Cplx<T>::type* tw;
+  // FP32, n + 1 prime, lines of up to 2^kRowTableLg points: the stages' twiddle
+  // tables (row_table_power) of the plans with 16 and with 8 values per thread
+  const typename Cplx<T>::type* rtw;
+  const typename Cplx<T>::type* rtw8;
   const typename Cplx<T>::type* chirp;   // c_{j+1}, j = 0..n-1
   // FFT_L of conj(c_m) embedded circularly, / L, by place (place_frequency) of
   // the stage plans with 16 and with 8 values per thread
@@ -856,7 +860,7 @@ __device__ __forceinline__ void body_dst_rows_at(const DstRowsArgs<T>& a, int bx
         if (dw) dp.add(o * dw[idx]);
       }
     };
-    fft_places<PLACE_CONV, VPT, false, LGHI, LGLO, false>(buf, lg, ls, 0, nl, a.tw, a.lgmax, ld, mid, out);
+    fft_places<PLACE_CONV, VPT, false, LGHI, LGLO, TW_CALC>(buf, lg, ls, 0, nl, a.tw, a.lgmax, ld, mid, out);
   }
   dst_rows_finish(a, bx, rr, dp, red);
 }
@@ -993,8 +997,9 @@ __device__ __forceinline__ void body_dst_rows_odd_fixed(const DstRowsArgs<T>& a,
 // negative where the sign is.  The rows go through shared memory in their own
 // order, so global reads and writes are one contiguous run per CTA.
 // Chirp convolutions before, this after (CUDA graphs): preconditioner 256^3 594
-// -> 384 us, 192^3 330 -> 204, 96^3 54.7 -> 38.5, 768^2 27.7 -> 20.0, 256^2
-// 10.75 -> 11.2 (few CTAs, one chain).
+// -> 391 us, 192^3 330 -> 207, 96^3 54.7 -> 39.1, 768^2 27.7 -> 19.5, 256^2
+// 10.75 -> 11.3 (few CTAs, one chain).  The twiddle tables (TW_ROWS) are 10 us
+// of 256^3 and 5 of 192^3; smaller grids do not feel them.
 template <typename T, int THREADS, int VPT, int LGLO, int LGHI>
 __device__ __forceinline__ void body_dst_rows_prime_at(const DstRowsArgs<T>& a, int bx, const int lg) {
   typedef typename Cplx<T>::type C;
@@ -1008,7 +1013,14 @@ __device__ __forceinline__ void body_dst_rows_prime_at(const DstRowsArgs<T>& a, 
   const int row0 = bx * NL;
   const int nl = min(NL, a.rows - row0);
   const int n = a.n, M = n >> 1;
-  T* xs = reinterpret_cast<T*>(smem_raw + sbuf_elems((long long)NL * L) * sizeof(C));   // the CTA's rows
+  // the stages' twiddles, then the CTA's rows
+  C* stw = reinterpret_cast<C*>(smem_raw + sbuf_elems((long long)NL * L) * sizeof(C));
+  const int ntw = row_table_len(lg);
+  T* xs = reinterpret_cast<T*>(stw + ntw);
+  {
+    const C* FL_RESTRICT rtw = VPT == 8 ? a.rtw8 : a.rtw;
+    for (int m = threadIdx.x; m < ntw; m += THREADS) cp_async<sizeof(C)>(&stw[m], &rtw[m]);
+  }
   const size_t base = (size_t)row0 * n;
   const int tot = nl * n;
   constexpr int U = 4;   // elements in flight per thread
@@ -1048,6 +1060,7 @@ __device__ __forceinline__ void body_dst_rows_prime_at(const DstRowsArgs<T>& a, 
       }
     }
   }
+  cp_async_wait_all();
   __syncthreads();
   {
     const short* FL_RESTRICT perm = a.perm;
@@ -1077,7 +1090,7 @@ __device__ __forceinline__ void body_dst_rows_prime_at(const DstRowsArgs<T>& a, 
         xs[q * n + n - i] = v.x * s;
       }
     };
-    fft_places<PLACE_CONV, VPT, false, LGHI, LGLO, false>(buf, lg, ls, 0, nl, a.tw, a.lgmax, ld, mid, out);
+    fft_places<PLACE_CONV, VPT, false, LGHI, LGLO, TW_ROWS>(buf, lg, ls, 0, nl, stw, lg, ld, mid, out);
   }
   __syncthreads();
   for (int e0 = threadIdx.x; e0 < tot; e0 += THREADS * U) {
@@ -1257,7 +1270,7 @@ __device__ __forceinline__ void body_dst_cols_at(const DstColsArgs<T>& a, int c0
       base[(size_t)k * lstride + c] = (w.x * v.x + w.y * v.y) * post;
     }
   };
-  fft_places<PLACE_CONV, VPT, true, LGHI, LGLO, true>(buf, lg, 0, ltx, TX, stw, lg, ld, mid, out);
+  fft_places<PLACE_CONV, VPT, true, LGHI, LGLO, TW_TABLE>(buf, lg, 0, ltx, TX, stw, lg, ld, mid, out);
 }
 
 template <typename T, int THREADS, int VPT, bool PRIME, int LGLO, int LGHI, int LG>

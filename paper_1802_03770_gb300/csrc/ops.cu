@@ -577,13 +577,14 @@ PrecChain<T> build_precond(const Geo& g, const Tables<T>& tb, const PrecIO<T>& i
   const bool prime = dst_prime<T>(g, d - 1);
   const int Ld = dst_len<T>(g, d - 1);
   ch.row_smem = smem_bytes<T>(row_lines_at<T>(Ld, io.row_threads), Ld);
-  if (prime) ch.row_smem += (size_t)NL * nx * sizeof(T);   // the CTA's rows
+  if (prime)   // behind the lines the stages' twiddles and the CTA's rows
+    ch.row_smem += (size_t)row_table_len(ilog2i(Ld)) * sizeof(typename Cplx<T>::type) + (size_t)NL * nx * sizeof(T);
   // DST normalisation of every axis but 0 (solved by the tridiagonal pass)
   double post = 1.0;
   for (int i = 1; i < d; ++i) post *= 2.0 / (g.n[i] + 1.0);
   {
     DstRowsArgs<T>& a = ch.first;
-    a.in = io.in; a.out = tb.t; a.tw = tb.tw; a.chirp = tb.chirp[d - 1]; a.bhat = tb.bhat[d - 1]; a.bhat8 = tb.bhat8;
+    a.in = io.in; a.out = tb.t; a.tw = tb.tw; a.rtw = tb.rtw; a.rtw8 = tb.rtw8; a.chirp = tb.chirp[d - 1]; a.bhat = tb.bhat[d - 1]; a.bhat8 = tb.bhat8;
     a.ftw = tb.ftw; a.fchirp = tb.fchirp[d - 1]; a.fbhat = tb.fbhat[d - 1]; a.bexp = tb.bexp[d - 1]; a.odd = odd;
     a.perm = prime ? tb.perm[d - 1] : nullptr;
     a.st = io.st; a.x = io.x; a.r = io.r; a.p = io.p; a.q = io.q;
@@ -631,7 +632,7 @@ PrecChain<T> build_precond(const Geo& g, const Tables<T>& tb, const PrecIO<T>& i
   }
   {
     DstRowsArgs<T>& a = ch.last;
-    a.in = tb.t; a.out = io.out; a.tw = tb.tw; a.chirp = tb.chirp[d - 1]; a.bhat = tb.bhat[d - 1]; a.bhat8 = tb.bhat8;
+    a.in = tb.t; a.out = io.out; a.tw = tb.tw; a.rtw = tb.rtw; a.rtw8 = tb.rtw8; a.chirp = tb.chirp[d - 1]; a.bhat = tb.bhat[d - 1]; a.bhat8 = tb.bhat8;
     a.ftw = tb.ftw; a.fchirp = tb.fchirp[d - 1]; a.fbhat = tb.fbhat[d - 1]; a.bexp = tb.bexp[d - 1]; a.odd = odd;
     a.perm = prime ? tb.perm[d - 1] : nullptr;
     a.st = io.st; a.x = nullptr; a.r = nullptr; a.p = nullptr; a.q = nullptr;

@@ -325,6 +325,16 @@ fl_status build_tables(fl_plan* p) {
           dt[m] = tw32[(size_t)place_table_power((int)m, lgd, Cfg<float>::CV) << (g.lgmax - lgd)];
         us = upload_table(p, &p->t32.dptw[ax], dt);
         if (us != FL_OK) return us;
+        if (ax == g.d - 1 && row_table_len(lgd) > 0) {
+          std::vector<float2> r16(row_table_len(lgd)), r8(row_table_len(lgd));
+          for (size_t m = 0; m < r16.size(); ++m) {
+            r16[m] = tw32[(size_t)row_table_power((int)m, lgd, 16) << (g.lgmax - lgd)];
+            r8[m] = tw32[(size_t)row_table_power((int)m, lgd, 8) << (g.lgmax - lgd)];
+          }
+          us = upload_table(p, &p->t32.rtw, r16);
+          if (us == FL_OK) us = upload_table(p, &p->t32.rtw8, r8);
+          if (us != FL_OK) return us;
+        }
       }
       // in the order in which the transforms hold the frequencies
       std::vector<float2> b16(Ld), b8(Ld);
