@@ -149,8 +149,9 @@ fl_status fl_plan_describe(const fl_plan* plan, fl_plan_desc* desc);
  * preconditioner solves on the plan's stream (axis by axis, the others
  * kept), keeps the fastest, and writes the choice to tx_out (nullable).
  * For plans whose rows (the last axis) pad to 256 .. 2048 points it then
- * times the FP32 row passes in both row shapes (see fl_plan_set_row_shape)
- * and keeps the faster (fl_plan_row_shape reads the choice).
+ * times the FP32 row passes in row shapes 0 and 1 (see fl_plan_set_row_shape)
+ * and keeps the faster (fl_plan_row_shape reads the choice); where shape 0
+ * takes 256 x 8 in every row pass, it sets shape 1 without a trial.
  * It uses the plan's workspaces, waits for the stream, and invalidates the
  * plan's captured CG graphs; run it before solves, not during one. */
 fl_status fl_plan_set_tiles(fl_plan* plan, const int tx[6]);
@@ -159,11 +160,12 @@ fl_status fl_plan_autotune(fl_plan* plan, int tx_out[6]);
 /* CTA shape of the FP32 row passes (no counterpart in the paper): 0 = the
  * default (128 threads x 16 values per line; 256 x 8 in a pass over rows
  * padded to 256 .. 2048 points whose grid is at most about two CTAs per SM),
- * 1 = 256 threads x 8 throughout (rows padded to 256 .. 2048 points only,
- * else FL_INVALID_ARG).  Results agree to FP32 rounding (other radix plan),
- * not bit for bit.  Invalidates the plan's captured CG graphs.
- * fl_plan_row_shape returns the current shape (-1 for a NULL plan).
- * Lockstep batched solves use shape 1 when every plan of the batch has it,
+ * 1 = 256 threads x 8 throughout, 2 = 128 x 16 throughout (1 and 2: rows padded
+ * to 256 .. 2048 points only, else FL_INVALID_ARG).  Results agree to FP32
+ * rounding (other radix plan), not bit for bit.  Invalidates the plan's captured
+ * CG graphs.  fl_plan_row_shape returns the shape set last, by this call or the
+ * tuner, 0 before (-1 for a NULL plan).
+ * Lockstep batched solves use 256 x 8 when every plan of the batch has shape 1,
  * else 128 x 16; the persistent launch has its own CTA shape. */
 fl_status fl_plan_set_row_shape(fl_plan* plan, int shape);
 int fl_plan_row_shape(const fl_plan* plan);

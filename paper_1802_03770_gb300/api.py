@@ -256,7 +256,9 @@ class Plan:
         return list(arr)
 
     def set_row_shape(self, shape):
-        """CTA shape of the FP32 row passes: 0 = 128 x 16, 1 = 256 x 8."""
+        """CTA shape of the FP32 row passes: 0 = by the grid's size, 1 = 256
+        threads x 8 values per line, 2 = 128 x 16 (1 and 2: rows padded to 256
+        .. 2048 points)."""
         L.check(self._lib.fl_plan_set_row_shape(self._h, int(shape)), "fl_plan_set_row_shape")
 
     def row_shape(self):

@@ -263,18 +263,19 @@ void launch_rows_inv_w8(const RowsInvArgs<float>& a, int grid, size_t smem, cuda
 void launch_dst_rows_w8(const DstRowsArgs<float>& a, int grid, size_t smem, cudaStream_t s);   // either form
 cudaError_t configure_rows_w8();
 // Whether a plan's FP32 row pass of `ctas` CTAs on lines of L points takes
-// the 256 x 8 shape: where the plan asks for it, and by default where the
-// pass is a fraction of a wave, bound by one CTA's chain, which that shape
+// the 256 x 8 shape: as the plan asks (Tables::rshape), and by default where
+// the pass is a fraction of a wave, bound by one CTA's chain, which that shape
 // halves.  Larger grids are bound by instructions and keep 128 x 16.  Measured
 // in CUDA graphs, 128 x 16 -> 256 x 8: preconditioner 200^2 (50 CTAs) 23.8 ->
 // 14.6 us, 511^2 (256) 25.8 -> 21.9, 1000 x 500 (500) 27.7 -> 29.6, 600^2 (600)
 // 23.6 -> 26.8; apply 255^2 (32) 21.9 -> 19.5, 600^2 (300) 32.1 -> 29.7, 1024^2
 // (512) 35.8 -> 36.5; lines of 256 gain less (100^2 21.8 -> 21.1) and lose
 // from 250 CTAs on (40 x 100 x 100 59.0 -> 60.2).
+inline bool rows_w8_lines(int L) { return L >= 256 && L <= 2048; }   // the lines that have the choice
+inline bool rows_w8_rule(int L, int ctas) { return ctas <= (L >= 512 ? 304 : 152); }
 template <typename T> inline bool rows_w8(const Tables<T>& tb, int L, int ctas) {
-  if (sizeof(T) != 4 || L < 256 || L > 2048) return false;
-  if (tb.rshape == 1) return true;
-  return ctas <= (L >= 512 ? 304 : 152);
+  if (sizeof(T) != 4 || !rows_w8_lines(L)) return false;
+  return tb.rshape == 0 ? rows_w8_rule(L, ctas) : tb.rshape == 1;
 }
 
 // Whether a DST along an axis takes the odd extension (its points n = 2^k - 1).

@@ -1002,10 +1002,16 @@ fl_status autotune_precision(fl_plan* p) {
     }
     tb.tx[ax] = best_tx;
   }
-  // FP32 row passes: the 128 x 16 and the 256 x 8 CTA shape (rows_w8.cu)
+  // FP32 row passes: the default rule against the 256 x 8 CTA shape throughout
+  // (rows_w8); where the rule takes 256 x 8 in every pass, the two are the same
+  // kernels, and the shape is 256 x 8 without a trial
   if constexpr (sizeof(T) == 4) {
-    const int Lx = g.L[g.d - 1];
-    if (Lx >= 256 && Lx <= 2048) {
+    const int Lx = g.L[g.d - 1], Ld = dst_len<T>(g, g.d - 1);
+    const bool same = rows_w8_rule(Lx, apply_partials<T>(g)) &&
+                      (!with_prec || !rows_w8_lines(Ld) || rows_w8_rule(Ld, precond_partials<T>(g)));
+    if (rows_w8_lines(Lx) && same) {
+      tb.rshape = 1;
+    } else if (rows_w8_lines(Lx)) {
       int best_rs = 0;
       float best_ms = -1.0f;
       for (int rs = 0; rs < 2 && ce == cudaSuccess; ++rs) {
@@ -1257,9 +1263,9 @@ fl_status fl_plan_set_tiles(fl_plan* p, const int tx[6]) {
 fl_status fl_plan_set_row_shape(fl_plan* p, int shape) {
   if (!check_plan(p)) return fail(FL_INVALID_ARG, "NULL plan");
   const int Lx = p->g.L[p->g.d - 1];
-  if (shape != 0 && shape != 1) return fail(FL_INVALID_ARG, "row shape must be 0 or 1");
-  if (shape == 1 && !(Lx >= 256 && Lx <= 2048))
-    return fail(FL_INVALID_ARG, "row shape 1 needs padded rows of 256 .. 2048 points");
+  if (shape < 0 || shape > 2) return fail(FL_INVALID_ARG, "row shape must be 0, 1 or 2");
+  if (shape != 0 && !rows_w8_lines(Lx))
+    return fail(FL_INVALID_ARG, "row shapes 1 and 2 need padded rows of 256 .. 2048 points");
   p->t32.rshape = shape;
   p->gcache[0].release();
   p->gcache[1].release();

@@ -3,10 +3,9 @@
 // memory and partial-sum counts), radix-8 stages instead of radix-16.  Half
 // the values per thread shortens each CTA's dependent chain, which pays on
 // grids of up to two CTAs per SM and costs on larger ones; rows_w8 (chain.cuh)
-// holds the rule and its measurements, fl_plan_autotune times both shapes per
-// plan and may ask for this one throughout.  64 registers, four CTAs per SM
-// (at two it cost twice as much on full grids).  Compiled apart from ops.cu
-// so that the two build in parallel.
+// holds the rule and its measurements, fl_plan_autotune may ask for this one
+// throughout.  64 registers, four CTAs per SM (at two it cost twice as much on
+// full grids).  Compiled apart from ops.cu so that the two build in parallel.
 #include "chain.cuh"
 
 namespace fl {
