@@ -141,7 +141,8 @@ fl_status fl_plan_describe(const fl_plan* plan, fl_plan_desc* desc);
  * 64).  The tile width changes neither the arithmetic nor any result (each
  * line is transformed the same way), only the launch shape.
  *   tx[6]: FP32 axes 0..2, then FP64 axes 0..2; 0 = the default (the widest
- *   tile; half of it in FP32 3D passes whose spectrum fits the L2 cache).
+ *   tile; half of it in FP32 3D passes of a single problem whose spectrum fits
+ *   the L2 cache).
  * fl_plan_set_tiles sets them (FL_INVALID_ARG for a width out of range or
  * not a power of two; entries of axes without a strided pass are ignored).
  * fl_plan_autotune times, for each precision and each axis with a strided

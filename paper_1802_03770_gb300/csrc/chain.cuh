@@ -110,11 +110,15 @@ template <typename T> inline int default_tx(const Geo& g, int axis) {
 template <typename T> inline int plan_tx(const Geo& g, const Tables<T>& tb, int axis) {
   return tb.tx[axis] > 0 ? tb.tx[axis] : default_tx<T>(g, axis);
 }
-// a column-tile width tx narrowed to what a CTA of ct threads holds (ct = 0:
-// tx unchanged)
-template <typename T> inline int tile_at(int tx, int L, int ct) {
-  if (ct <= 0) return tx;
-  return std::max(1, std::min(tx, std::min(kMaxTx, (ct * Cfg<T>::CV) / L)));
+// the same for lines of L points and launches whose CTAs have ct threads
+// whatever the tile (batches; ct = 0: CTAs that fit the tile, plan_tx): at most
+// what such a CTA holds, and that by default.  Half tiles left half of the 512
+// threads of a lockstep launch without a butterfly: batches of sixteen 64^3
+// 27.3 -> 25.5 ms, six 96^3 48.3 -> 39.7, twelve 40^3 .. 90^3 47.3 -> 39.7.
+template <typename T> inline int tile_at(const Geo& g, const Tables<T>& tb, int axis, int L, int ct) {
+  if (ct <= 0) return plan_tx<T>(g, tb, axis);
+  const int full = std::max(1, std::min(kMaxTx, (ct * Cfg<T>::CV) / L));
+  return tb.tx[axis] > 0 ? std::min(tb.tx[axis], full) : full;
 }
 // shared-memory bytes of `lines` lines of L complex values (padded, SBuf)
 template <typename T> inline size_t smem_bytes(int lines, int L) {

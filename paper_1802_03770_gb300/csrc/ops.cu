@@ -508,7 +508,7 @@ ApplyChain<T> build_apply(const Geo& g, const Tables<T>& tb, const ApplyIO<T>& i
     a.rows_in = rows_in; a.rows_out = rows_out; a.lstride = lstride; a.ostride = ostride;
     a.nouter = nouter; a.mode = mode; a.sig_line = sig_line; a.sig_outer = sig_outer; a.Lo = Lo;
     const int L = g.L[axis];
-    const int tx = tile_at<T>(plan_tx<T>(g, tb, axis), L, io.col_threads);
+    const int tx = tile_at<T>(g, tb, axis, L, io.col_threads);
     a.ltx = ilog2i(tx);
     ch.cols_grid[ch.ncols] = dim3((g.H + tx - 1) / tx, nouter);
     ch.cols_smem[ch.ncols] = mode == COLS_CONV ? conv_tile_bytes<T>(tx, L) : cols_bytes<T>(tx, L);
@@ -605,7 +605,7 @@ PrecChain<T> build_precond(const Geo& g, const Tables<T>& tb, const PrecIO<T>& i
     const int L = dst_len<T>(g, axis);
     a.n = g.n[axis]; a.ncols = nx; a.lg = ilog2i(L); a.lgmax = g.lgmax;
     a.ostride = ostride; a.lstride = lstride;
-    const int tx = tile_at<T>(plan_tx<T>(g, tb, axis), L, io.col_threads);
+    const int tx = tile_at<T>(g, tb, axis, L, io.col_threads);
     a.ltx = ilog2i(tx);
     ch.cols_grid[ch.ncols] = dim3((nx + tx - 1) / tx, nouter);
     ch.cols_smem[ch.ncols] = cols_bytes<T>(tx, L);

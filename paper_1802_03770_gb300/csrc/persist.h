@@ -36,7 +36,7 @@ struct PBarrier {
 };
 // The persistent kernel's CTA shape: the row passes hold
 // row_lines_at(L, kPersistThreads) lines per CTA, the strided passes tiles
-// of at most tile_at(., L, kPersistThreads) columns and the tridiagonal
+// of at most kPersistThreads * Cfg::CV / L columns (tile_at) and the tridiagonal
 // pass kPersistTriCols columns.
 constexpr int kPersistThreads = 256;
 constexpr int kPersistTriCols = kPersistThreads / kTriSeg;

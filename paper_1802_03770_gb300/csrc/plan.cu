@@ -1742,6 +1742,7 @@ fl_status solve_batched_mixed(fl_plan* const* plans, int count, const double* co
       pi.in = p->v32.r; pi.out = p->v32.z; pi.dotw = p->v32.r; pi.dot_part = p->part[P_RZ];
       pi.mask = p->mask;
       pi.st = const_cast<PcgState*>(gate);
+      pi.col_threads = Cfg<float>::CT;
       pinit.add(build_precond<float>(g, p->t32, pi));
     }
     init[i] = BScalarArgs{st, gate, p->part[P_BB], vb, nullptr, 0,
@@ -1752,7 +1753,8 @@ fl_status solve_batched_mixed(fl_plan* const* plans, int count, const double* co
     ioa.pre = PRE_PUPDATE; ioa.u = prec[i] ? p->v32.z : p->v32.r; ioa.p = p->v32.p;
     ioa.mask = p->mask; ioa.st = st; ioa.out = p->v32.q; ioa.x = p->v32.p; ioa.cm = 1.0;
     ioa.dotw = p->v32.p; ioa.partials = p->part[P_PQ]; ioa.fin = FIN_PQ;
-    ioa.row_threads = ioa.col_threads = persist ? kPersistThreads : 0;
+    ioa.row_threads = persist ? kPersistThreads : 0;
+    ioa.col_threads = persist ? kPersistThreads : Cfg<float>::CT;
     apply32.add(build_apply<float>(g, p->t32, ioa));
     // the x/r update and the CG scalar step (in the last CTA of the last pass)
     if (prec[i]) {
@@ -1761,7 +1763,8 @@ fl_status solve_batched_mixed(fl_plan* const* plans, int count, const double* co
       pu.pre = DPRE_UPDATE; pu.out = p->v32.z; pu.x = p->v32.x; pu.r = p->v32.r; pu.p = p->v32.p;
       pu.q = p->v32.q; pu.rr_part = p->part[P_RR]; pu.dotw = p->v32.r; pu.dot_part = p->part[P_RZ];
       pu.st = st; pu.fin = FIN_STEP; pu.mask = p->mask;
-      pu.row_threads = pu.col_threads = persist ? kPersistThreads : 0;
+      pu.row_threads = persist ? kPersistThreads : 0;
+      pu.col_threads = persist ? kPersistThreads : Cfg<float>::CT;
       pu.tri_cols = persist ? kPersistTriCols : 0;
       pstep.add(build_precond<float>(g, p->t32, pu));
     } else {
