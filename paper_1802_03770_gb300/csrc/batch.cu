@@ -27,7 +27,7 @@ __device__ __forceinline__ int batch_problem(const int* __restrict__ off, int np
 
 #define FL_BATCHED_KERNEL(NAME, ARGS)                                                          \
   template <typename T, int THREADS, int VPT>                                                  \
-  __global__ void __launch_bounds__(THREADS, min_ctas<T>(THREADS))                               \
+  __global__ void __launch_bounds__(THREADS, min_ctas(THREADS))                                \
       kb_##NAME(const ARGS<T>* __restrict__ args, const int* __restrict__ off,                 \
                 const int* __restrict__ gx, int nprob) {                                       \
     pdl_wait();                                                                                \

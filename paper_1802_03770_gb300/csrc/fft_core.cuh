@@ -195,16 +195,16 @@ template <> struct LogR<8> { static constexpr int v = 3; };
 template <> struct LogR<16> { static constexpr int v = 4; };
 
 // w[r] = w1^r, r = 0..R-1, for w1 = exp(-2 pi i step / Lmax) (conjugated
-// for the inverse).  FP64, and FP32 with TWT (tw then points to a copy of the
-// table in shared memory): every power is loaded from the long-double table tw
-// (r * step < Lmax).  FP32 without: w1 = sincospif(-2 step / Lmax) (the argument
+// for the inverse).  FP64 and the strided FP32 passes (TABLE): every power is
+// loaded from the long-double table tw (r * step < Lmax), FP32 from a copy in
+// shared memory.  FP32 rows: w1 = sincospif(-2 step / Lmax) (the argument
 // is exact), w2 and w4 by squaring, w4 brought back to modulus 1 to first order,
 // the rest by products.  Without that w8..w15 have up to fifteen times the
 // modulus error of w1, which the two directions of a convolution add up:
 // preconditioner 640^2, error 5.9e-7, with it 3.3e-7 (18.8 -> 19.2 us, 256^3 380
 // -> 379).  w4 from the table 3.6e-7 (1024^2 32.9 -> 34.1), w1, w2, w4 and w8
 // from it 3.0e-7 (1024^2 35.8, 256^3 403).
-template <int R, bool TWT = false, typename C>
+template <int R, bool TABLE = false, typename C>
 __device__ __forceinline__ void twiddles(const C* FL_RESTRICT tw, int step, bool inv, C* w, int lgmax) {
   auto ld = [&](int i) {
     C t = tw[i];
@@ -212,7 +212,7 @@ __device__ __forceinline__ void twiddles(const C* FL_RESTRICT tw, int step, bool
     return t;
   };
   w[0] = cmake<C>(1, 0);
-  if constexpr (sizeof(w[0].x) == 8 || TWT) {
+  if constexpr (sizeof(w[0].x) == 8 || TABLE) {
 #pragma unroll
     for (int r = 1; r < R; ++r) w[r] = ld(r * step);
   } else {
@@ -260,7 +260,7 @@ enum { STAGE_FIRST = 0, STAGE_MID = 1, STAGE_LAST = 2 };
 __device__ __forceinline__ int sbuf_phys(int i) { return i + (i >> 4); }
 __host__ __device__ constexpr int clog2(int x) { return x <= 1 ? 0 : 1 + clog2(x / 2); }
 
-template <int R, int VPT, bool IL, int LG, int NS, int MODE, bool HALF, bool TWT, typename C,
+template <int R, int VPT, bool IL, int LG, int NS, int MODE, bool HALF, typename C,
           typename Load, typename Epi>
 __device__ __forceinline__ void stage_ct(SBuf<C> buf, int ls, int ltx, int nlines,
                                          const C* FL_RESTRICT tw, int lgmax, bool inv, Load& load,
@@ -301,7 +301,7 @@ __device__ __forceinline__ void stage_ct(SBuf<C> buf, int ls, int ltx, int nline
         if (NS > 1 && k != 0) {
           // twiddle w^(r k) = tw[r * k * Lmax / (NS R)]
           C w[R];
-          twiddles<R, TWT>(tw, k << (lgmax - clog2(NS * R)), inv, w, lgmax);
+          twiddles<R>(tw, k << (lgmax - clog2(NS * R)), inv, w, lgmax);
 #pragma unroll
           for (int r = 1; r < R; ++r) v[b][r] = cmul(v[b][r], w[r]);
         }
@@ -358,7 +358,7 @@ struct FftPlan {
   __host__ __device__ static constexpr int ns(int s) { return s == 0 ? 1 : ns(s - 1) * radix(s - 1); }
 };
 
-template <int LG, int VPT, bool IL, bool HALF, bool TWT, int ST, typename C, typename Load, typename Epi>
+template <int LG, int VPT, bool IL, bool HALF, int ST, typename C, typename Load, typename Epi>
 __device__ __forceinline__ void fft_io_stage(SBuf<C> buf, int ls, int ltx, int nlines,
                                              const C* FL_RESTRICT tw, int lgmax, bool inv, Load load,
                                              bool sync_load, Epi epi, bool sync_epi) {
@@ -366,11 +366,11 @@ __device__ __forceinline__ void fft_io_stage(SBuf<C> buf, int ls, int ltx, int n
   constexpr int R = P::radix(ST);
   constexpr int Ns = P::ns(ST);
   constexpr int MODE = ST == 0 ? STAGE_FIRST : (ST == P::S - 1 ? STAGE_LAST : STAGE_MID);
-  stage_ct<R, VPT, IL, LG, Ns, MODE, HALF, TWT>(buf, ls, ltx, nlines, tw, lgmax, inv, load, epi,
-                                          MODE == STAGE_FIRST ? sync_load : sync_epi);
+  stage_ct<R, VPT, IL, LG, Ns, MODE, HALF>(buf, ls, ltx, nlines, tw, lgmax, inv, load, epi,
+                                           MODE == STAGE_FIRST ? sync_load : sync_epi);
   if constexpr (ST + 1 < P::S)
-    fft_io_stage<LG, VPT, IL, HALF, TWT, ST + 1>(buf, ls, ltx, nlines, tw, lgmax, inv, load, sync_load,
-                                               epi, sync_epi);
+    fft_io_stage<LG, VPT, IL, HALF, ST + 1>(buf, ls, ltx, nlines, tw, lgmax, inv, load, sync_load,
+                                            epi, sync_epi);
 }
 
 // A full transform of `nlines` lines (IL: 2^ltx interleaved lines) of length
@@ -379,18 +379,18 @@ __device__ __forceinline__ void fft_io_stage(SBuf<C> buf, int ls, int ltx, int n
 // shared buffer (a barrier separates its reads from the first stage's
 // writes); sync_epi: the epilogue writes the shared buffer.  The buffer is
 // free again after a barrier that follows the call.
-template <int LG, int VPT, bool IL, bool HALF, bool TWT, typename C, typename Load, typename Epi>
+template <int LG, int VPT, bool IL, bool HALF, typename C, typename Load, typename Epi>
 __device__ __forceinline__ void fft_io_ct(SBuf<C> buf, int ls, int ltx, int nlines,
                                           const C* FL_RESTRICT tw, int lgmax, bool inv, Load load,
                                           bool sync_load, Epi epi, bool sync_epi) {
   if constexpr (FftPlan<LG, VPT>::S >= 2) {
-    fft_io_stage<LG, VPT, IL, HALF, TWT, 0>(buf, ls, ltx, nlines, tw, lgmax, inv, load, sync_load, epi,
-                                          sync_epi);
+    fft_io_stage<LG, VPT, IL, HALF, 0>(buf, ls, ltx, nlines, tw, lgmax, inv, load, sync_load, epi,
+                                       sync_epi);
   } else {
     // one stage: natural order in shared memory afterwards; each thread
     // hands on elements it reads (an epilogue writing the buffer rewrites
     // the element it was given)
-    stage_ct<FftPlan<LG, VPT>::radix(0), VPT, IL, LG, 1, STAGE_FIRST, HALF, TWT>(
+    stage_ct<FftPlan<LG, VPT>::radix(0), VPT, IL, LG, 1, STAGE_FIRST, HALF>(
         buf, ls, ltx, nlines, tw, lgmax, inv, load, epi, sync_load);
     constexpr int L = 1 << LG;
     const int total = IL ? (L << ltx) : nlines * L;
@@ -410,12 +410,12 @@ __device__ __forceinline__ void fft_io_ct(SBuf<C> buf, int ls, int ltx, int nlin
 #define FL_FFT_LEN(LGV)                                                                     \
   if constexpr (LGV >= LGLO && LGV <= LGHI) {                                               \
     if (lg == LGV) {                                                                        \
-      fft_io_ct<LGV, VPT, IL, HALF, TWT>(buf, ls, ltx, nlines, tw, lgmax, inv, load, sync_load, \
-                                         epi, sync_epi);                                    \
+      fft_io_ct<LGV, VPT, IL, HALF>(buf, ls, ltx, nlines, tw, lgmax, inv, load, sync_load,  \
+                                    epi, sync_epi);                                         \
       return;                                                                               \
     }                                                                                       \
   }
-template <int VPT, bool IL, bool HALF = false, int LGHI = 11, int LGLO = 4, bool TWT = false, typename C,
+template <int VPT, bool IL, bool HALF = false, int LGHI = 11, int LGLO = 4, typename C,
           typename Load, typename Epi>
 __device__ __forceinline__ void fft_io(SBuf<C> buf, int lg, int ls, int ltx, int nlines,
                                        const C* FL_RESTRICT tw, int lgmax, bool inv, Load load,
@@ -435,7 +435,7 @@ __device__ __forceinline__ void fft_io(SBuf<C> buf, int lg, int ls, int ltx, int
 
 // In-place transform of lines in shared memory (natural order in and out)
 // with the compile-time stage plan; ends with a barrier.
-template <int VPT, bool IL, int LGHI = 11, int LGLO = 4, bool TWT = false, typename C>
+template <int VPT, bool IL, int LGHI = 11, int LGLO = 4, typename C>
 __device__ __forceinline__ void fft_smem(SBuf<C> buf, int lg, int ls, int ltx, int nlines,
                                          const C* FL_RESTRICT tw, int lgmax, bool inv) {
   auto ld = [=](int q, int k) -> C { return IL ? buf[(k << ltx) + q] : buf[q * ls + k]; };
@@ -443,7 +443,7 @@ __device__ __forceinline__ void fft_smem(SBuf<C> buf, int lg, int ls, int ltx, i
     if (IL) buf[(k << ltx) + q] = v;
     else buf[q * ls + k] = v;
   };
-  fft_io<VPT, IL, false, LGHI, LGLO, TWT>(buf, lg, ls, ltx, nlines, tw, lgmax, inv, ld, true, st, true);
+  fft_io<VPT, IL, false, LGHI, LGLO>(buf, lg, ls, ltx, nlines, tw, lgmax, inv, ld, true, st, true);
   __syncthreads();
 }
 

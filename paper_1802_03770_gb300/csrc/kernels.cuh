@@ -112,7 +112,6 @@ __device__ __forceinline__ double cta_sum_partials(const double* FL_RESTRICT par
 // The wide instantiations for the longest lines (LGLO > 4: one line of 4096
 // or 8192 points per CTA) ask for one CTA only, so that the compiler keeps
 // the row bodies' registers.
-template <typename T = float>
 constexpr int min_ctas(int threads, int lglo = 4) {
   return lglo > 4 ? 1 : (threads <= 128 ? FL_ROW_MIN_CTAS : (threads == 256 ? 4 : 2));
 }
@@ -399,7 +398,7 @@ __device__ __forceinline__ void body_rows_fwd(const RowsFwdArgs<T>& a, int bx, i
 }
 
 template <typename T, int THREADS, int VPT, int LGLO = 4>
-__global__ void __launch_bounds__(THREADS, min_ctas<T>(THREADS, LGLO)) k_rows_fwd(RowsFwdArgs<T> a) {
+__global__ void __launch_bounds__(THREADS, min_ctas(THREADS, LGLO)) k_rows_fwd(RowsFwdArgs<T> a) {
   pdl_wait();
   body_rows_fwd<T, THREADS, VPT, LGLO>(a, blockIdx.x, blockIdx.y);
   pdl_release();
@@ -544,7 +543,7 @@ __device__ __forceinline__ void body_cols(const ColsArgs<T>& a, int bx, int by) 
 }
 
 template <typename T, int THREADS, int VPT, int LGLO = 4>
-__global__ void __launch_bounds__(THREADS, min_ctas<T>(THREADS, LGLO)) k_cols(ColsArgs<T> a) {
+__global__ void __launch_bounds__(THREADS, min_ctas(THREADS, LGLO)) k_cols(ColsArgs<T> a) {
   pdl_wait();
   body_cols<T, THREADS, VPT, LGLO>(a, blockIdx.x, blockIdx.y);
   pdl_release();
@@ -697,7 +696,7 @@ __device__ __forceinline__ void body_rows_inv(const RowsInvArgs<T>& a, int bx, i
 }
 
 template <typename T, int THREADS, int VPT, int LGLO = 4>
-__global__ void __launch_bounds__(THREADS, min_ctas<T>(THREADS, LGLO)) k_rows_inv(RowsInvArgs<T> a) {
+__global__ void __launch_bounds__(THREADS, min_ctas(THREADS, LGLO)) k_rows_inv(RowsInvArgs<T> a) {
   pdl_wait();
   body_rows_inv<T, THREADS, VPT, LGLO>(a, blockIdx.x, blockIdx.y);
   pdl_release();
@@ -1164,19 +1163,19 @@ __device__ __forceinline__ void body_dst_rows(const DstRowsArgs<T>& a, int bx, i
 }
 
 template <typename T, int THREADS, int VPT, int LGLO = 4>
-__global__ void __launch_bounds__(THREADS, min_ctas<T>(THREADS, LGLO)) k_dst_rows(DstRowsArgs<T> a) {
+__global__ void __launch_bounds__(THREADS, min_ctas(THREADS, LGLO)) k_dst_rows(DstRowsArgs<T> a) {
   pdl_wait();
   body_dst_rows_as<T, THREADS, VPT, DST_CHIRP, LGLO>(a, blockIdx.x, blockIdx.y);
   pdl_release();
 }
 template <typename T, int THREADS, int VPT, int LGLO = 4>
-__global__ void __launch_bounds__(THREADS, min_ctas<T>(THREADS, LGLO)) k_dst_rows_odd(DstRowsArgs<T> a) {
+__global__ void __launch_bounds__(THREADS, min_ctas(THREADS, LGLO)) k_dst_rows_odd(DstRowsArgs<T> a) {
   pdl_wait();
   body_dst_rows_as<T, THREADS, VPT, DST_ODD, LGLO>(a, blockIdx.x, blockIdx.y);
   pdl_release();
 }
 template <typename T, int THREADS, int VPT, int LGLO = 4>
-__global__ void __launch_bounds__(THREADS, min_ctas<T>(THREADS, LGLO)) k_dst_rows_prime(DstRowsArgs<T> a) {
+__global__ void __launch_bounds__(THREADS, min_ctas(THREADS, LGLO)) k_dst_rows_prime(DstRowsArgs<T> a) {
   pdl_wait();
   body_dst_rows_as<T, THREADS, VPT, DST_PRIME, LGLO>(a, blockIdx.x, blockIdx.y);
   pdl_release();
@@ -1310,13 +1309,13 @@ __device__ __forceinline__ void body_dst_cols(const DstColsArgs<T>& a, int bx, i
 }
 
 template <typename T, int THREADS, int VPT, int LGLO = 4>
-__global__ void __launch_bounds__(THREADS, min_ctas<T>(THREADS, LGLO)) k_dst_cols(DstColsArgs<T> a) {
+__global__ void __launch_bounds__(THREADS, min_ctas(THREADS, LGLO)) k_dst_cols(DstColsArgs<T> a) {
   pdl_wait();
   body_dst_cols_as<T, THREADS, VPT, false, LGLO>(a, blockIdx.x, blockIdx.y);
   pdl_release();
 }
 template <typename T, int THREADS, int VPT, int LGLO = 4>
-__global__ void __launch_bounds__(THREADS, min_ctas<T>(THREADS, LGLO)) k_dst_cols_prime(DstColsArgs<T> a) {
+__global__ void __launch_bounds__(THREADS, min_ctas(THREADS, LGLO)) k_dst_cols_prime(DstColsArgs<T> a) {
   pdl_wait();
   body_dst_cols_as<T, THREADS, VPT, true, LGLO>(a, blockIdx.x, blockIdx.y);
   pdl_release();
