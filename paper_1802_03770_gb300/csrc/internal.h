@@ -39,7 +39,7 @@ struct FxR;
 template <typename T>
 struct Tables {
   typedef typename std::conditional<sizeof(T) == 4, float2, double2>::type C;
-  C* tw = nullptr;            // exp(-2 pi i k / Lmax)
+  C* tw = nullptr;            // FP64: exp(-2 pi i k / Lmax), for the symbol's set-up
   T* sig = nullptr;           // FP32: kernel symbol / prod L
   // FP64 passes: the constants of the fixed-point transforms (fix_core.cuh)
   FxW* ftw = nullptr;         // exp(-2 pi i k / Lmax)
@@ -49,13 +49,15 @@ struct Tables {
   FxW* fbhat[3] = {nullptr, nullptr, nullptr};   // / 2^bexp
   int bexp[3] = {0, 0, 0};
   C* ptw[3] = {nullptr, nullptr, nullptr};     // FP32: twiddle tables of the strided passes' stages
-  // FP32 axes with n + 1 prime: orders and stage twiddles of Rader's convolution (dst_prime)
+  // FP32 axes with n + 1 prime: orders of Rader's convolution (dst_prime), its
+  // stages' twiddles along the strided axis
   short* perm[3] = {nullptr, nullptr, nullptr};
   C* dptw[3] = {nullptr, nullptr, nullptr};
-  // twiddle tables of its rows, for the 16- and the 8-value stage plan (row_table_power)
+  // and those of its rows, for the 16- and the 8-value stage plan (row_table_power)
   C* rtw = nullptr;
   C* rtw8 = nullptr;
-  // FP32 DST tables
+  // FP32 DST tables: chirps where the form is the chirp convolution, the kernel's
+  // spectrum of either convolution
   C* chirp[3] = {nullptr, nullptr, nullptr};
   C* bhat[3] = {nullptr, nullptr, nullptr};   // by place of the 16-value stage plan
   C* bhat8 = nullptr;         // last axis, by place of the 8-value plan

@@ -270,7 +270,6 @@ struct RowsFwdArgs {
   const float* x32;        // PRE_ACCUM
   const uint8_t* mask;     // nullable: Omega inside the box
   typename Cplx<T>::type* S;
-  const typename Cplx<T>::type* tw;
   const PcgState* st;
   int rows, n, H, lg, lgmax;
   int rows_per_plane, plane_stride;  // spectrum row = (r / rpp) * ps + r % rpp
@@ -349,9 +348,10 @@ __device__ __forceinline__ void body_rows_fwd_at(const RowsFwdArgs<T>& a, int bx
   }
   __syncthreads();
   {
+    const C* const calc = nullptr;   // twiddles are computed
     auto ld = [=](int q, int k) -> C { return k < hL ? buf[q * ls + k] : cmake<C>((T)0, (T)0); };
     auto st = [=](int q, int k, C v) { buf[q * ls + k] = v; };
-    fft_io<VPT, false, true, LGHI, LGLO>(buf, lg, ls, 0, nl, a.tw, a.lgmax, false, ld,
+    fft_io<VPT, false, true, LGHI, LGLO>(buf, lg, ls, 0, nl, calc, a.lgmax, false, ld,
                                                        true, st, true);
   }
   __syncthreads();
@@ -558,7 +558,6 @@ __global__ void __launch_bounds__(THREADS, min_ctas(THREADS, LGLO)) k_cols(ColsA
 template <typename T>
 struct RowsInvArgs {
   const typename Cplx<T>::type* S;
-  const typename Cplx<T>::type* tw;
   const uint8_t* mask;
   const PcgState* st;
   T* out;                  // nullable
@@ -627,7 +626,8 @@ __device__ __forceinline__ void body_rows_inv_at(const RowsInvArgs<T>& a, int bx
     put(q, hL, a.S[spec(2 * q) + hL], hb ? a.S[spec(2 * q + 1) + hL] : cmake<C>((T)0, (T)0));
   }
   __syncthreads();
-  fft_smem<VPT, false, LGHI, LGLO>(buf, lg, ls, 0, nl, a.tw, a.lgmax, true);
+  const C* const calc = nullptr;   // twiddles are computed
+  fft_smem<VPT, false, LGHI, LGLO>(buf, lg, ls, 0, nl, calc, a.lgmax, true);
   DotAcc<T> part;
   const T* FL_RESTRICT xin = (a.cx != 0.0) ? a.x : nullptr;
   const T* FL_RESTRICT bin = (a.cb != 0.0) ? a.b : nullptr;
@@ -713,7 +713,6 @@ template <typename T>
 struct DstRowsArgs {
   const T* in;             // DPRE_NONE: input rows
   T* out;
-  const typename Cplx<T>::type* tw;
   // FP32, n + 1 prime, lines of up to 2^kRowTableLg points: the stages' twiddle
   // tables (row_table_power) of the plans with 16 and with 8 values per thread
   const typename Cplx<T>::type* rtw;
@@ -859,7 +858,8 @@ __device__ __forceinline__ void body_dst_rows_at(const DstRowsArgs<T>& a, int bx
         if (dw) dp.add(o * dw[idx]);
       }
     };
-    fft_places<PLACE_CONV, VPT, false, LGHI, LGLO, TW_CALC>(buf, lg, ls, 0, nl, a.tw, a.lgmax, ld, mid, out);
+    const C* const calc = nullptr;   // twiddles are computed
+    fft_places<PLACE_CONV, VPT, false, LGHI, LGLO, TW_CALC>(buf, lg, ls, 0, nl, calc, a.lgmax, ld, mid, out);
   }
   dst_rows_finish(a, bx, rr, dp, red);
 }
@@ -967,7 +967,8 @@ __device__ __forceinline__ void body_dst_rows_odd_at(const DstRowsArgs<T>& a, in
         if (dw) dp.add(o * dw[idx]);
       }
     };
-    fft_io<VPT, false, false, LGHI, LGLO>(buf, lg, ls, 0, nl, a.tw, a.lgmax, false, ld, true, epi, false);
+    const C* const calc = nullptr;   // twiddles are computed
+    fft_io<VPT, false, false, LGHI, LGLO>(buf, lg, ls, 0, nl, calc, a.lgmax, false, ld, true, epi, false);
   }
   dst_rows_finish(a, bx, rr, dp, red);
 }

@@ -494,7 +494,7 @@ ApplyChain<T> build_apply(const Geo& g, const Tables<T>& tb, const ApplyIO<T>& i
   {
     RowsFwdArgs<T>& a = ch.fwd;
     a.u = io.u; a.p = io.p; a.acc = io.acc; a.x32 = io.x32; a.mask = io.mask;
-    a.S = tb.S; a.tw = tb.tw; a.st = io.st;
+    a.S = tb.S; a.st = io.st;
     a.rows = (int)rows; a.n = g.n[d - 1]; a.H = g.H; a.lg = g.lg[d - 1]; a.lgmax = g.lgmax;
     a.rows_per_plane = rpp; a.plane_stride = pstride; a.pre = io.pre; a.ftw = tb.ftw;
   }
@@ -524,7 +524,7 @@ ApplyChain<T> build_apply(const Geo& g, const Tables<T>& tb, const ApplyIO<T>& i
   }
   {
     RowsInvArgs<T>& a = ch.inv;
-    a.S = tb.S; a.tw = tb.tw; a.mask = io.mask; a.st = io.st;
+    a.S = tb.S; a.mask = io.mask; a.st = io.st;
     a.out = io.out; a.out32 = io.out32;
     // the epilogue's x is the apply input (after any pre-op)
     a.x = io.x; a.b = io.b; a.dotw = io.dotw; a.partials = io.partials;
@@ -584,7 +584,7 @@ PrecChain<T> build_precond(const Geo& g, const Tables<T>& tb, const PrecIO<T>& i
   for (int i = 1; i < d; ++i) post *= 2.0 / (g.n[i] + 1.0);
   {
     DstRowsArgs<T>& a = ch.first;
-    a.in = io.in; a.out = tb.t; a.tw = tb.tw; a.rtw = tb.rtw; a.rtw8 = tb.rtw8; a.chirp = tb.chirp[d - 1]; a.bhat = tb.bhat[d - 1]; a.bhat8 = tb.bhat8;
+    a.in = io.in; a.out = tb.t; a.rtw = tb.rtw; a.rtw8 = tb.rtw8; a.chirp = tb.chirp[d - 1]; a.bhat = tb.bhat[d - 1]; a.bhat8 = tb.bhat8;
     a.ftw = tb.ftw; a.fchirp = tb.fchirp[d - 1]; a.fbhat = tb.fbhat[d - 1]; a.bexp = tb.bexp[d - 1]; a.odd = odd;
     a.perm = prime ? tb.perm[d - 1] : nullptr;
     a.st = io.st; a.x = io.x; a.r = io.r; a.p = io.p; a.q = io.q;
@@ -632,7 +632,7 @@ PrecChain<T> build_precond(const Geo& g, const Tables<T>& tb, const PrecIO<T>& i
   }
   {
     DstRowsArgs<T>& a = ch.last;
-    a.in = tb.t; a.out = io.out; a.tw = tb.tw; a.rtw = tb.rtw; a.rtw8 = tb.rtw8; a.chirp = tb.chirp[d - 1]; a.bhat = tb.bhat[d - 1]; a.bhat8 = tb.bhat8;
+    a.in = tb.t; a.out = io.out; a.rtw = tb.rtw; a.rtw8 = tb.rtw8; a.chirp = tb.chirp[d - 1]; a.bhat = tb.bhat[d - 1]; a.bhat8 = tb.bhat8;
     a.ftw = tb.ftw; a.fchirp = tb.fchirp[d - 1]; a.fbhat = tb.fbhat[d - 1]; a.bexp = tb.bexp[d - 1]; a.odd = odd;
     a.perm = prime ? tb.perm[d - 1] : nullptr;
     a.st = io.st; a.x = nullptr; a.r = nullptr; a.p = nullptr; a.q = nullptr;

@@ -251,19 +251,20 @@ fl_status build_tables(fl_plan* p) {
   fl_status us = upload_table(p, &p->t64.ftw, twx);
   if (us != FL_OK) return us;
   FL_CUDA(dalloc(p, &p->t64.tw, Lmax * sizeof(double2)));
-  FL_CUDA(dalloc(p, &p->t32.tw, Lmax * sizeof(float2)));
   FL_CUDA(cudaMemcpy(p->t64.tw, tw64.data(), Lmax * sizeof(double2), cudaMemcpyHostToDevice));
-  FL_CUDA(cudaMemcpy(p->t32.tw, tw32.data(), Lmax * sizeof(float2), cudaMemcpyHostToDevice));
   for (int ax = 0; ax < g.d; ++ax) {
     const int n = g.n[ax], L = g.L[ax];
     const long long N1 = n + 1;
-    // stage twiddles of the strided passes
-    std::vector<float2> pt(place_table_len(g.lg[ax]));
-    for (size_t m = 0; m < pt.size(); ++m)
-      pt[m] = tw32[(size_t)place_table_power((int)m, g.lg[ax], Cfg<float>::CV) << (g.lgmax - g.lg[ax])];
-    us = upload_table(p, &p->t32.ptw[ax], pt);
-    if (us != FL_OK) return us;
-    if (ax > 0) {   // axis 0 has no DST (tridiagonal pass)
+    const bool last = ax == g.d - 1;   // the rows; the other axes have strided passes
+    if (!last) {   // stage twiddles of the strided passes
+      std::vector<float2> pt(place_table_len(g.lg[ax]));
+      for (size_t m = 0; m < pt.size(); ++m)
+        pt[m] = tw32[(size_t)place_table_power((int)m, g.lg[ax], Cfg<float>::CV) << (g.lgmax - g.lg[ax])];
+      us = upload_table(p, &p->t32.ptw[ax], pt);
+      if (us != FL_OK) return us;
+    }
+    // axis 0 has no DST (tridiagonal pass), rows of 2^k - 1 points no convolution
+    if (ax > 0 && !(last && dst_odd(g, ax))) {
       // c_m = exp(i pi m^2 / (2 N1)), with m^2 reduced mod 4 N1
       auto chirp = [&](long long m) {
         const long long m2 = (m * m) % (4 * N1);
@@ -320,12 +321,13 @@ fl_status build_tables(fl_plan* p) {
         }
         us = upload_table(p, &p->t32.perm[ax], perm);
         if (us != FL_OK) return us;
-        std::vector<float2> dt(place_table_len(lgd));
-        for (size_t m = 0; m < dt.size(); ++m)
-          dt[m] = tw32[(size_t)place_table_power((int)m, lgd, Cfg<float>::CV) << (g.lgmax - lgd)];
-        us = upload_table(p, &p->t32.dptw[ax], dt);
-        if (us != FL_OK) return us;
-        if (ax == g.d - 1 && row_table_len(lgd) > 0) {
+        if (!last) {
+          std::vector<float2> dt(place_table_len(lgd));
+          for (size_t m = 0; m < dt.size(); ++m)
+            dt[m] = tw32[(size_t)place_table_power((int)m, lgd, Cfg<float>::CV) << (g.lgmax - lgd)];
+          us = upload_table(p, &p->t32.dptw[ax], dt);
+          if (us != FL_OK) return us;
+        } else if (row_table_len(lgd) > 0) {
           std::vector<float2> r16(row_table_len(lgd)), r8(row_table_len(lgd));
           for (size_t m = 0; m < r16.size(); ++m) {
             r16[m] = tw32[(size_t)row_table_power((int)m, lgd, 16) << (g.lgmax - lgd)];
@@ -345,9 +347,9 @@ fl_status build_tables(fl_plan* p) {
       p->t64.bexp[ax] = bexp;
       us = upload_table(p, &p->t64.fchirp[ax], cx);
       if (us == FL_OK) us = upload_table(p, &p->t64.fbhat[ax], bx);
-      if (us == FL_OK) us = upload_table(p, &p->t32.chirp[ax], c32);
+      if (us == FL_OK && !dst_prime<float>(g, ax)) us = upload_table(p, &p->t32.chirp[ax], c32);
       if (us == FL_OK) us = upload_table(p, &p->t32.bhat[ax], b16);
-      if (us == FL_OK && ax == g.d - 1) us = upload_table(p, &p->t32.bhat8, b8);
+      if (us == FL_OK && last) us = upload_table(p, &p->t32.bhat8, b8);
       if (us != FL_OK) return us;
     }
     // eigenvalues of C h^d L along this axis: c (-a) 4 sin^2(pi k / (2 (n+1)))
