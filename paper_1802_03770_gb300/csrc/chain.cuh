@@ -270,11 +270,13 @@ cudaError_t configure_rows_w8();
 // the 256 x 8 shape: as the plan asks (Tables::rshape), and by default where
 // the pass is a fraction of a wave, bound by one CTA's chain, which that shape
 // halves.  Larger grids are bound by instructions and keep 128 x 16.  Measured
-// in CUDA graphs, 128 x 16 -> 256 x 8: preconditioner 200^2 (50 CTAs) 23.8 ->
-// 14.6 us, 511^2 (256) 25.8 -> 21.9, 1000 x 500 (500) 27.7 -> 29.6, 600^2 (600)
-// 23.6 -> 26.8; apply 255^2 (32) 21.9 -> 19.5, 600^2 (300) 32.1 -> 29.7, 1024^2
-// (512) 35.8 -> 36.5; lines of 256 gain less (100^2 21.8 -> 21.1) and lose
-// from 250 CTAs on (40 x 100 x 100 59.0 -> 60.2).
+// in CUDA graphs, 128 x 16 -> 256 x 8: preconditioner 200^2 (50 CTAs) 14.1 ->
+// 9.9 us, 511^2 (64) 20.4 -> 14.0, 640^2 (320) 17.8 -> 19.3, 1000 x 500 (500) 21.6
+// -> 23.3, 1024^2 (1024) 29.4 -> 34.7; apply 255^2 (32) 22.0 -> 17.7, 600^2 (300)
+// 29.6 -> 26.4, 1024^2 (512) 33.5 -> 34.0.  Applies would gain a little further
+// up (768^2, 384 CTAs, 31.4 -> 29.4), the sine transforms lose there (18.5 ->
+// 19.8).  Lines of 256 gain less: 100^2 preconditioner 10.6 -> 9.9, 20 x 100 x
+// 100 apply (125 CTAs) 32.8 -> 30.8, 40 x 100 x 100 (250) 40.9 -> 39.9.
 inline bool rows_w8_lines(int L) { return L >= 256 && L <= 2048; }   // the lines that have the choice
 inline bool rows_w8_rule(int L, int ctas) { return ctas <= (L >= 512 ? 304 : 152); }
 template <typename T> inline bool rows_w8(const Tables<T>& tb, int L, int ctas) {
@@ -287,8 +289,9 @@ inline bool dst_odd(const Geo& g, int axis) { return g.L[axis] == 2 * (g.n[axis]
 // Whether an FP32 DST along an axis is Rader's convolution of half the length
 // (n + 1 an odd prime; lines of 16 points are the shortest), and the length of
 // the DST's transforms.  Not where rows of 256 points take the 256 x 8 shape by
-// rows_w8, which lines of 128 do not have (preconditioner 96^2 9.4 us so, 12.8
-// by Rader; 96^3, more CTAs, 54.7 and 38.5).
+// rows_w8, which lines of 128 do not have (preconditioner 96^2 9.1 us so, 11.4
+// by Rader, 300 x 96 10.9 and 13.5; 66^3, more CTAs, 27.5 and 28.2, 130^3 155
+// and 69).
 template <typename T> inline bool dst_prime(const Geo& g, int axis) {
   const int q = g.n[axis] + 1;
   if (sizeof(T) != 4 || g.L[axis] < 32 || q % 2 == 0) return false;

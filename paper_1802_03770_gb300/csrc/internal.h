@@ -59,8 +59,8 @@ struct Tables {
   // FP32 DST tables: chirps where the form is the chirp convolution, the kernel's
   // spectrum of either convolution
   C* chirp[3] = {nullptr, nullptr, nullptr};
-  C* bhat[3] = {nullptr, nullptr, nullptr};   // by place of the 16-value stage plan
-  C* bhat8 = nullptr;         // last axis, by place of the 8-value plan
+  C* bhat[3] = {nullptr, nullptr, nullptr};   // by place of the 16-value stage plan (last axis: row_place)
+  C* bhat8 = nullptr;         // last axis, by row_place of the 8-value plan
   C* S = nullptr;             // operator spectrum workspace
   T* t = nullptr;             // preconditioner workspace (N)
   T* mu[3] = {nullptr, nullptr, nullptr};  // eigenvalues of C h^d L per axis

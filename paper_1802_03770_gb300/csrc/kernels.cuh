@@ -718,8 +718,8 @@ struct DstRowsArgs {
   const typename Cplx<T>::type* rtw;
   const typename Cplx<T>::type* rtw8;
   const typename Cplx<T>::type* chirp;   // c_{j+1}, j = 0..n-1
-  // FFT_L of conj(c_m) embedded circularly, / L, by place (place_frequency) of
-  // the stage plans with 16 and with 8 values per thread
+  // FFT_L of conj(c_m) embedded circularly, / L, in the order (row_place) of the
+  // stage plans with 16 and with 8 values per thread
   const typename Cplx<T>::type* bhat;
   const typename Cplx<T>::type* bhat8;
   PcgState* st;            // DPRE_UPDATE: alpha from here; FIN_STEP: updated
@@ -797,9 +797,9 @@ __device__ __forceinline__ void body_dst_rows_at(const DstRowsArgs<T>& a, int bx
   const int nl = min(NL, a.rows - row0);
   // Both transforms in place (fft_places), the first stage's legs from global
   // memory with all loads before the first use, the sine coefficients from
-  // the last stage's registers: 256^3 213 -> 157 us (DST along the middle axis
-  // 204 -> 130), 255^2 preconditioner 14.1 -> 10.8 us, 1024^2 rows unchanged
-  // (18.6: one wave, bound by its loads and one CTA's chain).
+  // the last stage's registers.  Against autosort stages with the rows staged
+  // first: preconditioner 1024^2 32.0 -> 29.5 us, 700 x 1001 27.7 -> 24.9, 200^2
+  // 14.6 -> 9.9 (one wave or less, bound by its loads and one CTA's chain).
   DotAcc<T> rr, dp;
   const bool update = a.pre == DPRE_UPDATE;
   const T al = update ? (T)a.st->alpha : (T)0;
@@ -996,10 +996,10 @@ __device__ __forceinline__ void body_dst_rows_odd_fixed(const DstRowsArgs<T>& a,
 // g^a mod p for a < M, then for b < M the index 2m (m = +-g^-b in 1..M),
 // negative where the sign is.  The rows go through shared memory in their own
 // order, so global reads and writes are one contiguous run per CTA.
-// Chirp convolutions before, this after (CUDA graphs): preconditioner 256^3 594
-// -> 391 us, 192^3 330 -> 207, 96^3 54.7 -> 39.1, 768^2 27.7 -> 19.5, 256^2
-// 10.75 -> 11.3 (few CTAs, one chain).  The twiddle tables (TW_ROWS) are 10 us
-// of 256^3 and 5 of 192^3; smaller grids do not feel them.
+// By chirp convolutions and so (CUDA graphs): preconditioner 256^3 588 and 292
+// us, 192^3 324 and 152, 130^3 155 and 69, 768^2 24.4 and 18.3; few CTAs, one
+// chain: 256^2 9.9 and 10.9, 192^2 9.4 and 10.7.  The twiddle tables (TW_ROWS) are
+// 7 us of 256^3, 2 of 192^3 and 0.3 of 256^2.
 template <typename T, int THREADS, int VPT, int LGLO, int LGHI>
 __device__ __forceinline__ void body_dst_rows_prime_at(const DstRowsArgs<T>& a, int bx, const int lg) {
   typedef typename Cplx<T>::type C;

@@ -338,11 +338,11 @@ fl_status build_tables(fl_plan* p) {
           if (us != FL_OK) return us;
         }
       }
-      // in the order in which the transforms hold the frequencies
+      // in the order in which the transforms hold and read the frequencies
       std::vector<float2> b16(Ld), b8(Ld);
       for (int k = 0; k < Ld; ++k) {
-        b16[k] = b32[place_frequency(k, lgd, 16)];
-        b8[k] = b32[place_frequency(k, lgd, 8)];
+        b16[last ? row_place(k, lgd, 16) : k] = b32[place_frequency(k, lgd, 16)];
+        b8[row_place(k, lgd, 8)] = b32[place_frequency(k, lgd, 8)];
       }
       p->t64.bexp[ax] = bexp;
       us = upload_table(p, &p->t64.fchirp[ax], cx);
