@@ -198,12 +198,17 @@ template <> struct LogR<16> { static constexpr int v = 4; };
 // for the inverse).  FP64 and the strided FP32 passes (TABLE): every power is
 // loaded from the long-double table tw (r * step < Lmax), FP32 from a copy in
 // shared memory.  FP32 rows: w1 = sincospif(-2 step / Lmax) (the argument
-// is exact), w2 and w4 by squaring, w4 brought back to modulus 1 to first order,
-// the rest by products.  Without that w8..w15 have up to fifteen times the
-// modulus error of w1, which the two directions of a convolution add up:
-// preconditioner 640^2, error 5.9e-7, with it 3.3e-7 (18.8 -> 19.2 us, 256^3 380
-// -> 379).  w4 from the table 3.6e-7 (1024^2 32.9 -> 34.1), w1, w2, w4 and w8
-// from it 3.0e-7 (1024^2 35.8, 256^3 403).
+// is exact), w2 and w4 by squaring, w4 and in radix-8 stages w2 brought back to
+// modulus 1 to first order, the rest by products.  Without that w8..w15 have up
+// to fifteen times the modulus error of w1, which the two directions of a
+// convolution add up: preconditioner 640^2, error 5.9e-7, with w4 so 3.3e-7
+// (before it 18.5 us, with it 18.4).  w2 in radix-8 stages: apply 200^2 1.74 ->
+// 1.55e-7, preconditioner 200^2 2.87 -> 2.52e-7 at the same time; in radix-16
+// stages too it would cost 1024^2 33.5 -> 34.5 us for 1 % of the error.
+__device__ __forceinline__ float2 to_unit(float2 w) {
+  const float e = -0.5f * fmaf(w.x, w.x, fmaf(w.y, w.y, -1.0f));
+  return make_float2(fmaf(w.x, e, w.x), fmaf(w.y, e, w.y));
+}
 template <int R, bool TABLE = false, typename C>
 __device__ __forceinline__ void twiddles(const C* FL_RESTRICT tw, int step, bool inv, C* w, int lgmax) {
   auto ld = [&](int i) {
@@ -223,12 +228,11 @@ __device__ __forceinline__ void twiddles(const C* FL_RESTRICT tw, int step, bool
     }
     if (R >= 4) {
       w[2] = cmul(w[1], w[1]);
+      if (R == 8) w[2] = to_unit(w[2]);
       w[3] = cmul(w[1], w[2]);
     }
     if (R >= 8) {
-      w[4] = cmul(w[2], w[2]);
-      const float e = -0.5f * fmaf(w[4].x, w[4].x, fmaf(w[4].y, w[4].y, -1.0f));
-      w[4] = cmake<C>(fmaf(w[4].x, e, w[4].x), fmaf(w[4].y, e, w[4].y));
+      w[4] = to_unit(cmul(w[2], w[2]));
       w[5] = cmul(w[4], w[1]);
       w[6] = cmul(w[4], w[2]);
       w[7] = cmul(w[4], w[3]);

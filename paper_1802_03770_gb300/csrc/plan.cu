@@ -225,6 +225,30 @@ FxW fix_const(long double re, long double im) {
   return FxW{x.h, x.l, y.h, y.l};
 }
 
+// A root of unity in FP32 for the operator's strided passes: of the neighbours
+// of the rounded parts the pair with the least modulus and phase error, the first
+// at twice the weight.  The in-place stages use one table in both directions, so
+// that its phase errors largely cancel and its modulus errors add: with each part
+// rounded by itself the error of the 256^3 apply was 2.16e-7, so 2.08 (2.11 with
+// autosort stages), at 160^3 1.84, 1.76 (1.81).  Rader's convolutions gain nothing
+// (256^3 preconditioner 3.73 and 3.83e-7) and keep the rounded parts.
+float2 root32(long double cs, long double sn) {
+  float2 best = make_float2((float)cs, (float)sn);
+  const float x0 = best.x, y0 = best.y;
+  if (x0 == 0.0f || y0 == 0.0f) return best;   // a quarter turn is exact
+  long double least = 1e30L;
+  for (int i = -1; i <= 1; ++i)
+    for (int j = -1; j <= 1; ++j) {
+      const float x = i ? nextafterf(x0, 2.0f * i) : x0, y = j ? nextafterf(y0, 2.0f * j) : y0;
+      const long double m = (long double)x * x + (long double)y * y - 1.0L, ph = x * sn - y * cs;
+      if (m * m + ph * ph < least) {
+        least = m * m + ph * ph;
+        best = make_float2(x, y);
+      }
+    }
+  return best;
+}
+
 template <typename X>
 fl_status upload_table(fl_plan* p, X** dst, const std::vector<X>& v) {
   FL_CUDA(dalloc(p, dst, v.size() * sizeof(X)));
@@ -239,13 +263,14 @@ fl_status build_tables(fl_plan* p) {
   const int Lmax = 1 << g.lgmax;
   const long double pi = 3.141592653589793238462643383279502884L;
   std::vector<double2> tw64(Lmax);
-  std::vector<float2> tw32(Lmax);
+  std::vector<float2> tw32(Lmax), root(Lmax);
   std::vector<FxW> twx(Lmax);
   for (int k = 0; k < Lmax; ++k) {
     const long double ang = -2.0L * pi * (long double)k / (long double)Lmax;
     const long double cs = cosl(ang), sn = sinl(ang);
     tw64[k] = make_double2((double)cs, (double)sn);
     tw32[k] = make_float2((float)cs, (float)sn);
+    root[k] = root32(cs, sn);
     twx[k] = fix_const(cs, sn);
   }
   fl_status us = upload_table(p, &p->t64.ftw, twx);
@@ -259,7 +284,7 @@ fl_status build_tables(fl_plan* p) {
     if (!last) {   // stage twiddles of the strided passes
       std::vector<float2> pt(place_table_len(g.lg[ax]));
       for (size_t m = 0; m < pt.size(); ++m)
-        pt[m] = tw32[(size_t)place_table_power((int)m, g.lg[ax], Cfg<float>::CV) << (g.lgmax - g.lg[ax])];
+        pt[m] = root[(size_t)place_table_power((int)m, g.lg[ax], Cfg<float>::CV) << (g.lgmax - g.lg[ax])];
       us = upload_table(p, &p->t32.ptw[ax], pt);
       if (us != FL_OK) return us;
     }
