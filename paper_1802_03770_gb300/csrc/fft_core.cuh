@@ -198,18 +198,22 @@ template <> struct LogR<16> { static constexpr int v = 4; };
 // for the inverse).  FP64 and the strided FP32 passes (TABLE): every power is
 // loaded from the long-double table tw (r * step < Lmax), FP32 from a copy in
 // shared memory.  FP32 rows: w1 = sincospif(-2 step / Lmax) (the argument
-// is exact), w2 and w4 by squaring, w4 and in radix-8 stages w2 brought back to
-// modulus 1 to first order, the rest by products.  Without that w8..w15 have up
+// is exact), w2 and w4 by squaring, w4 and in some radix-8 stages w2 brought back
+// to modulus 1 to first order, the rest by products.  Without that w8..w15 have up
 // to fifteen times the modulus error of w1, which the two directions of a
 // convolution add up: preconditioner 640^2, error 5.9e-7, with w4 so 3.3e-7
-// (before it 18.5 us, with it 18.4).  w2 in radix-8 stages: apply 200^2 1.74 ->
-// 1.55e-7, preconditioner 200^2 2.87 -> 2.52e-7 at the same time; in radix-16
-// stages too it would cost 1024^2 33.5 -> 34.5 us for 1 % of the error.
+// (before it 18.5 us, with it 18.4).  w2 (apply 200^2, white noise 1.74 -> 1.51e-7,
+// preconditioner 200^2 2.87 -> 2.52e-7, the same times) costs it some phase, which
+// the operator amplifies where the input is smooth: so in inverse passes, and with
+// UNIT2 in the forward ones of 8 values per thread or of 1024 points and more,
+// not in the others (160^3, Gaussians 1.760e-6 without, 1.800 with it in both
+// directions, 1.773 so; white noise 1.91e-7, 1.76, 1.75).  In radix-16 stages too
+// it would cost 1024^2 33.5 -> 34.5 us for 1 % of the error.
 __device__ __forceinline__ float2 to_unit(float2 w) {
   const float e = -0.5f * fmaf(w.x, w.x, fmaf(w.y, w.y, -1.0f));
   return make_float2(fmaf(w.x, e, w.x), fmaf(w.y, e, w.y));
 }
-template <int R, bool TABLE = false, typename C>
+template <int R, bool TABLE = false, bool UNIT2 = false, typename C>
 __device__ __forceinline__ void twiddles(const C* FL_RESTRICT tw, int step, bool inv, C* w, int lgmax) {
   auto ld = [&](int i) {
     C t = tw[i];
@@ -228,7 +232,7 @@ __device__ __forceinline__ void twiddles(const C* FL_RESTRICT tw, int step, bool
     }
     if (R >= 4) {
       w[2] = cmul(w[1], w[1]);
-      if (R == 8) w[2] = to_unit(w[2]);
+      if ((UNIT2 || inv) && R == 8) w[2] = to_unit(w[2]);
       w[3] = cmul(w[1], w[2]);
     }
     if (R >= 8) {
@@ -305,7 +309,7 @@ __device__ __forceinline__ void stage_ct(SBuf<C> buf, int ls, int ltx, int nline
         if (NS > 1 && k != 0) {
           // twiddle w^(r k) = tw[r * k * Lmax / (NS R)]
           C w[R];
-          twiddles<R>(tw, k << (lgmax - clog2(NS * R)), inv, w, lgmax);
+          twiddles<R, false, (VPT == 8 || LG >= 10)>(tw, k << (lgmax - clog2(NS * R)), inv, w, lgmax);
 #pragma unroll
           for (int r = 1; r < R; ++r) v[b][r] = cmul(v[b][r], w[r]);
         }
@@ -559,7 +563,7 @@ __device__ __forceinline__ void place_twiddles(const C* FL_RESTRICT tw, int j, i
 #pragma unroll
     for (int r = 1; r < R; ++r) w[r] = t[r << (LGB - LogR<R>::v)];
   } else {
-    twiddles<R, false>(tw, j << (lgmax - LGB), false, w, lgmax);
+    twiddles<R, false, true>(tw, j << (lgmax - LGB), false, w, lgmax);
   }
 }
 
