@@ -3,8 +3,11 @@
 // its local index l = b - off[i] is split as (l mod gx[i], l div gx[i]) into
 // the (x, y) block index the single-problem kernel would have had.  The
 // per-problem argument structs live in device memory and are the same the
-// single-problem launchers build, so a batched pass computes exactly what
-// the single launches compute.
+// single-problem launchers build, so a batched pass computes what the single
+// launches compute: the same bits in FP64 and in the strided and tridiagonal
+// passes, and in the FP32 row passes where both take the same row shape (single
+// launches of small grids run 256 x 8 by default, lockstep ones where every plan
+// asks for it), else to FP32 rounding.
 #include "chain.cuh"
 
 namespace fl {

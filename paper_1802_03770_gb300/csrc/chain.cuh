@@ -70,8 +70,8 @@ constexpr int kMaxLen = 8192;     // longest padded FFT line
 
 // Threads of a row (column) pass on lines of length L: the Cfg shape while a
 // CTA of that shape holds at least one line (tile), else one line of L
-// values per CTA (FP32 rows: 4096 on 256 and 8192 on 512 threads; FP64 rows
-// and columns: 8192 on 512 threads).
+// values per CTA (FP32 rows: 4096 on 256 and 8192 on 512 threads; FP64 rows:
+// 4096 on 512 and 8192 on 1024, columns: 8192 on 1024).
 template <typename T> inline int row_threads(int L) {
   return L <= Cfg<T>::RT * Cfg<T>::RV ? Cfg<T>::RT : L / Cfg<T>::RV;
 }
