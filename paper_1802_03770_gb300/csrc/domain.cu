@@ -22,10 +22,11 @@
 // vectors and factorised as L D L^T (right-looking, one launch per pivot);
 // the same eliminations applied to the identity give W = L^{-1}.  Each
 // application is then s = -W^T D^{-1} W E^T w: two triangular matrix-vector
-// products over the whole GPU (FP64, for either precision of the box
-// solves), bound by the FP64 rate and the launches.  The blocked
-// substitutions they replace ran in one CTA, one dependent block of 32
-// unknowns after another: 86 us for |Gamma| = 255 between events, now 12 + 7.
+// products (FP64, for either precision of the box solves), bound by the launches
+// and the latency of the gathers (the FP64 pipe would take a quarter of the time
+// at |Gamma| = 1023).  The blocked substitutions they replace ran in one CTA, one
+// dependent block of 32 unknowns after another: 86 us for |Gamma| = 255 between
+// events, now 13 + 7 (FP32 box solves 14 + 7); |Gamma| = 1023: 18 + 10 (30 + 10).
 #include "chain.cuh"
 #include "domain.h"
 

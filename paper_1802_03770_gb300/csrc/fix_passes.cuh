@@ -14,10 +14,10 @@
 // 1.7 operations per clock and SM).  These are bound by the integer pipes
 // (math-pipe throttle is the largest stall, issue 0.5 to 0.64 per cycle);
 // FP64 instructions are left in the epilogues only (two to six per output).
-// Measured on one GB300, applies in a CUDA graph, FP64 form -> this one:
-// 64^2 155 -> 40 us, 512^2 203 -> 58 us, 1024^2 508 -> 140 us, 256^3 13.0 ->
-// 3.1 ms; preconditioner solves 148 -> 62, 200 -> 81, 711 -> 171 us and 16.9
-// -> 4.8 ms.
+// Measured on one GB300 in CUDA graphs, FP64 form -> this one: applies 64^2 154
+// -> 39 us, 512^2 208 -> 57 us, 1024^2 507 -> 139 us, 256^3 13.0 -> 3.1 ms;
+// preconditioner solves (with the tridiagonal pass's change) 147 -> 34, 200 ->
+// 60, 710 -> 166 us and 16.9 -> 3.5 ms.
 #pragma once
 
 namespace fl {

@@ -882,6 +882,7 @@ __device__ __forceinline__ void body_dst_rows_fixed(const DstRowsArgs<T>& a, int
 // The same where n + 1 is half the line length (n = 2^k - 1, the paper's grids;
 // then L = 2 (n + 1)): the odd extension z_{L-j} = -z_j of z = a + i b, two rows
 // of sines in one transform of length L, Z_k = -2 i sum_j z_j sin(pi jk/(n+1)).
+// The rounding of the pair is that of its larger row.
 // One transform per two rows instead of four (a chirp convolution per row):
 // preconditioner 1023^2 33.4 -> 22.2 us, 255^3 966 -> 484 us (with the other
 // changes since), FP64 511^2 59 -> 38 us.
@@ -1644,9 +1645,10 @@ __device__ __forceinline__ void body_tri_cols_f64(const TriArgs<T>& a, int bx) {
 
 // The body for m <= M rows per segment: with M = 32 throughout, a 3D plan of
 // 256^3 (m = 8) spent most of its instructions on rows that are not there
-// and held one CTA per SM (149 us, now 47 us); 24 where 32 would leave a
-// quarter of them empty (preconditioner 700 x 1001 28.3 -> 28.1 us, 640^2 19.2 ->
-// 18.6).
+// and held one CTA per SM (149 us, now 42 us); 24 where 32 would leave a
+// quarter of them empty (preconditioner 640^2 17.76 -> 17.45 us, 768^2 18.56 ->
+// 18.16, 700 x 1001 25.07 -> 24.86), in single launches only: the batched and the
+// persistent kernels hold every variant in one body, and take 32 there.
 template <typename T, int TC, int M>
 __device__ __forceinline__ void body_tri_cols_m(const TriArgs<T>& a, int bx) {
   if constexpr (sizeof(T) == 8) body_tri_cols_f64<T, TC, M>(a, bx);
