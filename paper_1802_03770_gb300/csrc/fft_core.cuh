@@ -21,9 +21,10 @@
 // run in the symbol's set-up only.
 //
 // Twiddles: FP64 stages load every power w^r from a table
-// tw[k] = exp(-2 pi i k / Lmax) computed on the host in long double, FP32
-// column passes from a copy in shared memory; the other FP32 stages compute
-// them (see twiddles()).
+// tw[k] = exp(-2 pi i k / Lmax) computed on the host in long double; the FP32
+// strided passes and the short prime-length sine rows load them from tables per
+// stage in shared memory (see place_twiddles), the other FP32 rows compute them
+// (see twiddles()).
 //
 // Two storage layouts: lines of stride ls (element j of line q at
 // q * ls + j, ls a multiple of 16), and 2^ltx interleaved lines (element j
@@ -495,8 +496,8 @@ __host__ __device__ __forceinline__ int place_frequency(int p, int lg, int vpt) 
 // Where rows keep what belongs to place p (mid's third argument): the legs r of
 // the last stage in runs over its butterflies q, since neighbouring threads have
 // neighbouring q.  Read by place, at a stride of R, the kernel spectrum of a row
-// took eight to sixteen times the L1 wavefronts, twice those of all the shared
-// memory traffic: preconditioner 1024^2 32.9 -> 29.5 us, 700 x 1001 28.0 -> 24.9,
+// took eight (R = 8) or sixteen times the L1 wavefronts, by count as many as all the
+// shared-memory traffic and more: preconditioner 1024^2 32.9 -> 29.5 us, 700 x 1001 28.0 -> 24.9,
 // 256^3 390 -> 292, the same bits.
 inline int row_place(int p, int lg, int vpt) {
   int lr = 0, lgb = lg;
