@@ -205,16 +205,19 @@ template <> struct LogR<16> { static constexpr int v = 4; };
 // convolution add up: preconditioner 640^2, error 5.9e-7, with w4 so 3.3e-7
 // (before it 18.5 us, with it 18.4).  w2 (apply 200^2, white noise 1.74 -> 1.51e-7,
 // preconditioner 200^2 2.87 -> 2.52e-7, the same times) costs it some phase, which
-// the operator amplifies where the input is smooth: so in inverse passes, and with
-// UNIT2 in the forward ones of 8 values per thread or of 1024 points and more,
-// not in the others (160^3, Gaussians 1.760e-6 without, 1.800 with it in both
-// directions, 1.773 so; white noise 1.91e-7, 1.76, 1.75).  In radix-16 stages too
-// it would cost 1024^2 33.5 -> 34.5 us for 1 % of the error.
+// the operator amplifies where the input is smooth: so with UNIT2_BOTH (8 values
+// per thread, or 1024 points and more) in both directions, with UNIT2_INV (512
+// points) in inverse passes only (160^3, Gaussians 1.760e-6 without, 1.800 with it
+// in both directions, 1.773 so; white noise 1.91e-7, 1.76, 1.75).  Shorter lines
+// of 16 values are below the autosort passes' error without, and one CTA's chain
+// (64^2 apply 22.2 us, 22.4 with it).  In radix-16 stages too it would cost 1024^2
+// 33.5 -> 34.5 us for 1 % of the error.
+enum { UNIT2_NONE = 0, UNIT2_INV = 1, UNIT2_BOTH = 2 };
 __device__ __forceinline__ float2 to_unit(float2 w) {
   const float e = -0.5f * fmaf(w.x, w.x, fmaf(w.y, w.y, -1.0f));
   return make_float2(fmaf(w.x, e, w.x), fmaf(w.y, e, w.y));
 }
-template <int R, bool TABLE = false, bool UNIT2 = false, typename C>
+template <int R, bool TABLE = false, int UNIT2 = UNIT2_NONE, typename C>
 __device__ __forceinline__ void twiddles(const C* FL_RESTRICT tw, int step, bool inv, C* w, int lgmax) {
   auto ld = [&](int i) {
     C t = tw[i];
@@ -233,7 +236,7 @@ __device__ __forceinline__ void twiddles(const C* FL_RESTRICT tw, int step, bool
     }
     if (R >= 4) {
       w[2] = cmul(w[1], w[1]);
-      if ((UNIT2 || inv) && R == 8) w[2] = to_unit(w[2]);
+      if (R == 8 && (UNIT2 == UNIT2_BOTH || (UNIT2 == UNIT2_INV && inv))) w[2] = to_unit(w[2]);
       w[3] = cmul(w[1], w[2]);
     }
     if (R >= 8) {
@@ -310,7 +313,8 @@ __device__ __forceinline__ void stage_ct(SBuf<C> buf, int ls, int ltx, int nline
         if (NS > 1 && k != 0) {
           // twiddle w^(r k) = tw[r * k * Lmax / (NS R)]
           C w[R];
-          twiddles<R, false, (VPT == 8 || LG >= 10)>(tw, k << (lgmax - clog2(NS * R)), inv, w, lgmax);
+          constexpr int U2 = VPT == 8 || LG >= 10 ? UNIT2_BOTH : (LG == 9 ? UNIT2_INV : UNIT2_NONE);
+          twiddles<R, false, U2>(tw, k << (lgmax - clog2(NS * R)), inv, w, lgmax);
 #pragma unroll
           for (int r = 1; r < R; ++r) v[b][r] = cmul(v[b][r], w[r]);
         }
@@ -564,7 +568,7 @@ __device__ __forceinline__ void place_twiddles(const C* FL_RESTRICT tw, int j, i
 #pragma unroll
     for (int r = 1; r < R; ++r) w[r] = t[r << (LGB - LogR<R>::v)];
   } else {
-    twiddles<R, false, true>(tw, j << (lgmax - LGB), false, w, lgmax);
+    twiddles<R, false, UNIT2_BOTH>(tw, j << (lgmax - LGB), false, w, lgmax);
   }
 }
 

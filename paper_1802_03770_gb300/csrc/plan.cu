@@ -225,13 +225,15 @@ FxW fix_const(long double re, long double im) {
   return FxW{x.h, x.l, y.h, y.l};
 }
 
-// A root of unity in FP32 for the strided passes: of the neighbours of the rounded
-// parts the pair with the least modulus and phase error, m^2 + ph^2 / 3 of twice the
-// first and the second.  The in-place stages use one table in both directions, so
-// that its phase errors largely cancel and its modulus errors add: the error of
-// the 200^3 apply, white noise, 1.99 -> 1.93e-7, at more weight on the modulus 1.74,
-// but 2.45 instead of 2.41e-6 on Gaussians.  Rader's convolutions gain nothing (256^3
-// preconditioner 3.73 and 3.83e-7) and keep the rounded parts.
+// A root of unity in FP32 for the strided passes of 512 points and more: of the
+// neighbours of the rounded parts the pair with the least modulus and phase error,
+// m^2 + ph^2 / 3 of twice the first and the second.  The in-place stages use one
+// table in both directions, so that its phase errors largely cancel and its
+// modulus errors add: the error of the 200^3 apply, white noise, 1.99 -> 1.93e-7,
+// at more weight on the modulus 1.74, but 2.45 instead of 2.41e-6 on Gaussians.
+// Shorter lines are below the autosort passes' error with the rounded parts, and up
+// to 2 % lower on Gaussians; Rader's convolutions gain nothing (256^3
+// preconditioner 3.73 and 3.83e-7).
 float2 root32(double cs, double sn) {
   float x[3], y[3];
   x[0] = (float)cs;
@@ -288,8 +290,9 @@ fl_status build_tables(fl_plan* p) {
     const bool last = ax == g.d - 1;   // the rows; the other axes have strided passes
     if (!last) {   // stage twiddles of the strided passes
       std::vector<float2> pt(place_table_len(g.lg[ax]));
+      const std::vector<float2>& from = g.lg[ax] >= 9 ? root : tw32;
       for (size_t m = 0; m < pt.size(); ++m)
-        pt[m] = root[(size_t)place_table_power((int)m, g.lg[ax], Cfg<float>::CV) << (g.lgmax - g.lg[ax])];
+        pt[m] = from[(size_t)place_table_power((int)m, g.lg[ax], Cfg<float>::CV) << (g.lgmax - g.lg[ax])];
       us = upload_table(p, &p->t32.ptw[ax], pt);
       if (us != FL_OK) return us;
     }
